@@ -55,7 +55,15 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   s.L = L;
   s.n_reads = n_reads;
   s.n_words = (L + 31) / 32;
-  s.n_tiles = (s.n_words + kTileWords - 1) / kTileWords;
+  // phase-1 tiles (one thread block each): 16 waves of pass B's resident blocks where the input
+  // is long enough for that, never less than one sub-step of 256 words (a tile's fixed work,
+  // its partition cursors and its share of the sketch, is then still small beside it).  With
+  // 8192 words for every size, 0.2 M bases ran on one SM (pass A 56 + pass B 223 us; now 8 +
+  // 16), 10 M bases on 39 (76 + 287; 25 + 68) and 100 M bases of k = 63 in two waves of which
+  // the second was a quarter full (215 + 916; 165 + 678).
+  const uint64_t tw = (s.n_words / kTilesWanted + kTileWordsStep) / kTileWordsStep * kTileWordsStep;
+  s.tile_words = (uint32_t)(tw < (uint64_t)kTileWordsMax ? tw : (uint64_t)kTileWordsMax);
+  s.n_tiles = (s.n_words + s.tile_words - 1) / s.tile_words;
   s.k = k;
   s.canonical = canonical ? 1 : 0;
   s.kw = k <= 32 ? 1 : 2;
@@ -111,8 +119,6 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.codes = take(s.n_words * 8);
   lay.inv = take(s.n_words * 4);
   lay.tf = take(s.n_tiles * 8);
-  lay.hist = take(s.n_tiles * P1 * 4);
-  lay.toff = take(s.n_tiles * P1 * 8);
   lay.cst = take((P1 + 1) * 8);
   lay.fb = take((P1 + 1) * 4);
   lay.fm = take(P1 * 4);
@@ -123,7 +129,8 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.fc = take(nf * 8);
   lay.look = take(nf * 8);
   lay.kbuf = take(s.cap_kb * s.kw * 8);
-  lay.sbuf = take(s.cap_kb * s.kw * 8);
+  const uint64_t hist_bytes = s.n_tiles * P1 * 4;  // pass A's histogram lies in sbuf's memory
+  lay.sbuf = take(std::max<uint64_t>(s.cap_kb * s.kw * 8, hist_bytes));
   lay.meta = take(sizeof(Meta));
   lay.total = at;
   return (uint32_t)nf;
@@ -136,8 +143,7 @@ Buffers layout_buffers(const Layout& lay, uint8_t* ws) {
   b.codes64 = (uint64_t*)(ws + lay.codes);
   b.inv32 = (uint32_t*)(ws + lay.inv);
   b.tile_first = (uint64_t*)(ws + lay.tf);
-  b.hist = (uint32_t*)(ws + lay.hist);
-  b.toff = (uint64_t*)(ws + lay.toff);
+  b.hist = (uint32_t*)(ws + lay.sbuf);
   b.cstart = (uint64_t*)(ws + lay.cst);
   b.fine_base = (uint32_t*)(ws + lay.fb);
   b.fine_m = (uint32_t*)(ws + lay.fm);

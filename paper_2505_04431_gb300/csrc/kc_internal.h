@@ -6,7 +6,7 @@
 //   inv32[w]     bit i set iff byte 32w+i is not one of ACGTacgt, or lies past
 //                the end of the input.
 //   hist[t][c]   phase-1 histogram: valid windows of tile t in coarse partition c.
-//   toff[t][c]   write offset of tile t inside partition c (bucket-major scan).
+//                (in sbuf's memory: read by pass B, before sbuf is written).
 //   kbuf         keys grouped by coarse partition (the owner partition of
 //                Algorithm 3's AsyncAdd, here a key range so that outputs concatenate
 //                in sorted order).
@@ -18,9 +18,10 @@
 namespace kc {
 
 constexpr int kWordBases = 32;                 // bases per packed code word
-constexpr int kTileWords = 8192;               // one phase-1 tile = 262144 bases
-constexpr uint64_t kTileBases = (uint64_t)kTileWords * kWordBases;
-constexpr int kPackThreads = 512;              // pass A: one code word per thread per sub-step
+constexpr int kTileWordsMax = 8192;            // a phase-1 tile has 256 .. 8192 code words (Shape::tile_words)
+constexpr int kTileWordsStep = 256;
+constexpr uint64_t kTilesWanted = 4864;        // 16 waves of pass B's 2 blocks on each of 152 SMs
+constexpr int kPackThreads = 256;              // pass A: one code word per thread per sub-step
 constexpr int kMaxCoarseLog2 = 12;             // at most 4096 coarse partitions
 constexpr int kMaxFine = 4096;                 // at most this many fine partitions per coarse one
 // bases per coarse partition aimed at when the plan sets no partition count
@@ -78,7 +79,8 @@ struct Shape {
   uint64_t L;           // bases
   uint64_t n_reads;
   uint64_t n_words;     // ceil(L / 32)
-  uint64_t n_tiles;     // ceil(n_words / kTileWords)
+  uint64_t n_tiles;     // ceil(n_words / tile_words)
+  uint32_t tile_words;  // code words of a phase-1 tile (a multiple of kTileWordsStep)
   int k;
   int canonical;
   int kw;               // key words: 1 or 2
@@ -108,8 +110,7 @@ struct Buffers {
   uint64_t* codes64;
   uint32_t* inv32;
   uint64_t* tile_first;   // first read index whose start is >= the tile's halo start
-  uint32_t* hist;         // [n_tiles][P1]
-  uint64_t* toff;         // [n_tiles][P1]
+  uint32_t* hist;         // [n_tiles][P1], in sbuf's memory
   uint64_t* cstart;       // [P1 + 1] coarse partition starts
   uint32_t* fine_base;    // [P1 + 1] first fine index of each coarse partition
   uint32_t* fine_m;       // [P1] fine partitions of each coarse partition
@@ -117,7 +118,7 @@ struct Buffers {
   uint32_t* fhist;        // [nf_max] keys per fine partition (fine split); then distinct keys | deferred bit 31
   uint64_t* foff;         // [nf_max + 1] fine partition starts
   uint32_t* flo;          // [nf_max + 1] first range-map value u of each fine partition (0 after the last)
-  unsigned long long* fcur;  // [nf_max] fine scatter cursors
+  unsigned long long* fcur;  // [nf_max] pass B's partition cursors; then fine scatter cursors
   unsigned long long* look;  // [nf_max] look-back status words
   uint64_t* kbuf;
   uint64_t* sbuf;
@@ -155,7 +156,7 @@ struct BatchPlan {
   uint32_t grid[16] = {};
 };
 enum BatchKernel {
-  BK_CLEAR, BK_CHECK, BK_TILE_FIRST, BK_PACK, BK_COL_SCAN, BK_BUCKET_SCAN, BK_SCATTER, BK_FINE_PLAN, BK_FINE_HIST,
+  BK_CLEAR, BK_CHECK, BK_TILE_FIRST, BK_PACK, BK_BUCKET_SCAN, BK_SCATTER, BK_FINE_PLAN, BK_FINE_HIST,
   BK_FINE_SCAN, BK_FINE_SCATTER, BK_COUNT, BK_SCAN_DISTINCT, BK_COMPACT, BK_N
 };
 
@@ -197,7 +198,7 @@ struct ShapeOpts {
   int tight_slack = 0;     // testing: sampled regions get no slack
 };
 struct Layout {  // byte offsets into the count's scratch block
-  size_t reads, offs, codes, inv, tf, hist, toff, cst, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
+  size_t reads, offs, codes, inv, tf, cst, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
   size_t total;
 };
 // Fills s and lay for L bases and n_reads reads; copy_reads / copy_offs: the scratch holds a

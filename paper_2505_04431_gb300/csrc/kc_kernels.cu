@@ -5,7 +5,8 @@
 //                           rolling forward / reverse-complement keys (Algorithm 1's
 //                           kmer = (kmer << 2) OR Encode), owner partition of every
 //                           valid window, per-tile partition histogram.
-//   scans   k_col_scan, k_bucket_scan   exact write offsets per (tile, partition).
+//   scan    k_bucket_scan   partition starts; a tile then reserves its run in each partition
+//                           with one atomic add on that partition's cursor.
 //   pass B  k_scatter       recomputes the keys from the packed codes and writes each
 //                           key to its owner partition.  A tile's keys are first
 //                           grouped per partition in shared memory (a counting sort)
@@ -263,11 +264,12 @@ __global__ void k_check_offsets_batch(BatchTab t) {
 }
 
 // first read whose start is >= the halo start of each tile (lower bound in offsets)
-__device__ __forceinline__ void tile_first_body(const uint64_t* offsets, uint64_t n_reads, uint64_t n_tiles,
-                                                uint64_t* tile_first, uint32_t bid) {
+__device__ __forceinline__ void tile_first_body(const uint64_t* offsets, const Shape& s, uint64_t* tile_first,
+                                                uint32_t bid) {
   const uint64_t t = bid * (uint64_t)blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  const uint64_t pos = t * kTileBases;
+  const uint64_t n_reads = s.n_reads;
+  if (t >= s.n_tiles) return;
+  const uint64_t pos = t * s.tile_words * kWordBases;
   const uint64_t halo = pos >= 64 ? pos - 64 : 0;
   uint64_t lo = 0, hi = n_reads;
   while (lo < hi) {
@@ -276,12 +278,12 @@ __device__ __forceinline__ void tile_first_body(const uint64_t* offsets, uint64_
   }
   tile_first[t] = lo;
 }
-__global__ void k_tile_first(const uint64_t* offsets, uint64_t n_reads, uint64_t n_tiles, uint64_t* tile_first) {
-  tile_first_body(offsets, n_reads, n_tiles, tile_first, blockIdx.x);
+__global__ void k_tile_first(const uint64_t* offsets, Shape s, uint64_t* tile_first) {
+  tile_first_body(offsets, s, tile_first, blockIdx.x);
 }
 __global__ void k_tile_first_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  tile_first_body(d.b.offsets, d.s.n_reads, d.s.n_tiles, d.b.tile_first, bid);
+  tile_first_body(d.b.offsets, d.s, d.b.tile_first, bid);
 }
 
 // ------------------------------------------------------------------ phase 1 helpers
@@ -570,8 +572,8 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
   }
   __syncthreads();
   const uint64_t len = len_s;
-  for (int sub = 0; sub < kTileWords / kPackThreads; ++sub) {
-    const uint64_t j0 = tile * kTileWords + (uint64_t)sub * kPackThreads;
+  for (int sub = 0; sub < (int)s.tile_words / kPackThreads; ++sub) {
+    const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * kPackThreads;
     if (j0 >= s.n_words) break;
     __syncthreads();
     if (t < 2) {
@@ -613,60 +615,28 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
     }
   }
   __syncthreads();
-  for (int c = t; c < P1; c += kPackThreads) b.hist[tile * P1 + c] = hist_s[c];
+  // the tile's counts, and the partitions' totals (cstart holds them until k_bucket_scan)
+  for (int c = t; c < P1; c += kPackThreads) {
+    const uint32_t n = hist_s[c];
+    b.hist[tile * P1 + c] = n;
+    if (n) atomicAdd(reinterpret_cast<unsigned long long*>(&b.cstart[c]), (unsigned long long)n);
+  }
 }
 template <int KW>
-__global__ void __launch_bounds__(kPackThreads, KW == 1 ? 2 : 1) k_pack_count(Shape s, Buffers b) {
+__global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count(Shape s, Buffers b) {
   pack_count_body<KW>(s, b, blockIdx.x);
 }
 template <int KW>
-__global__ void __launch_bounds__(kPackThreads, KW == 1 ? 2 : 1) k_pack_count_batch(BatchTab t) {
+__global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
   pack_count_body<KW>(d.s, d.b, bid);
 }
 
 // ------------------------------------------------------------------ scans
-// Column scan of hist[tile][c]: toff[tile][c] = keys of partition c in tiles before `tile`.
-__device__ __forceinline__ void col_scan_body(const uint32_t* hist, uint64_t* toff, uint64_t* ccount, uint64_t n_tiles, int P1,
-                                              uint32_t bid) {
-  __shared__ uint64_t part[32][33];
-  const int lane = threadIdx.x, w = threadIdx.y;
-  const int c = bid * 32 + lane;
-  const uint64_t per = (n_tiles + 31) / 32;
-  const uint64_t lo = min(n_tiles, (uint64_t)w * per), hi = min(n_tiles, lo + per);
-  uint64_t s = 0;
-  if (c < P1)
-    for (uint64_t t = lo; t < hi; ++t) s += hist[t * P1 + c];
-  part[w][lane] = s;
-  __syncthreads();
-  if (w == 0) {
-    uint64_t run = 0;
-    for (int ww = 0; ww < 32; ++ww) {
-      const uint64_t x = part[ww][lane];
-      part[ww][lane] = run;
-      run += x;
-    }
-    if (c < P1) ccount[c] = run;
-  }
-  __syncthreads();
-  if (c < P1) {
-    uint64_t run = part[w][lane];
-    for (uint64_t t = lo; t < hi; ++t) {
-      toff[t * P1 + c] = run;
-      run += hist[t * P1 + c];
-    }
-  }
-}
-__global__ void k_col_scan(const uint32_t* hist, uint64_t* toff, uint64_t* ccount, uint64_t n_tiles, int P1) {
-  col_scan_body(hist, toff, ccount, n_tiles, P1, blockIdx.x);
-}
-__global__ void k_col_scan_batch(BatchTab t) {
-  KC_BATCH_PROLOGUE(t);
-  col_scan_body(d.b.hist, d.b.toff, d.b.cstart, d.s.n_tiles, 1 << d.s.b1, bid);
-}
-
-// Partition starts and the total number of windows.  One block.
-__device__ __forceinline__ void bucket_scan_body(const uint64_t* ccount, uint64_t* cstart, int P1, Meta* meta) {
+// Partition starts (also pass B's cursors) from the partitions' totals, and the total number
+// of windows.  One block.
+__device__ __forceinline__ void bucket_scan_body(const uint64_t* ccount, uint64_t* cstart, unsigned long long* cursor,
+                                                 int P1, Meta* meta) {
   extern __shared__ uint64_t sc[];  // [P1]
   __shared__ uint64_t wt[32];
   for (int c = threadIdx.x; c < P1; c += blockDim.x) {
@@ -676,18 +646,18 @@ __device__ __forceinline__ void bucket_scan_body(const uint64_t* ccount, uint64_
   }
   __syncthreads();
   const uint64_t K = block_exclusive_scan<uint64_t>(sc, P1, wt);
-  for (int c = threadIdx.x; c < P1; c += blockDim.x) cstart[c] = sc[c];
+  for (int c = threadIdx.x; c < P1; c += blockDim.x) cstart[c] = cursor[c] = sc[c];
   if (threadIdx.x == 0) {
     cstart[P1] = K;
     meta->n_windows = K;
   }
 }
-__global__ void k_bucket_scan(const uint64_t* ccount, uint64_t* cstart, int P1, Meta* meta) {
-  bucket_scan_body(ccount, cstart, P1, meta);
+__global__ void k_bucket_scan(const uint64_t* ccount, uint64_t* cstart, unsigned long long* cursor, int P1, Meta* meta) {
+  bucket_scan_body(ccount, cstart, cursor, P1, meta);
 }
 __global__ void k_bucket_scan_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  bucket_scan_body(d.b.cstart, d.b.cstart, 1 << d.s.b1, d.b.meta);
+  bucket_scan_body(d.b.cstart, d.b.cstart, d.b.fcur, 1 << d.s.b1, d.b.meta);
 }
 
 // Fine split of every coarse partition, after pass B: the distinct-key estimate (a sampled
@@ -817,13 +787,16 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   const int wl = t / TPW, h = t % TPW;  // code word of the thread within the sub-step, half
   const uint64_t tile = bid;
   for (int c = t; c < P1; c += NT) {
-    cursor[c] = b.cstart[c] + b.toff[tile * P1 + c];
+    // the tile's run in partition c, reserved at once (the order of the tiles' runs inside a
+    // partition does not matter to any later step)
+    const uint32_t n = DIRECT ? 0u : b.hist[tile * P1 + c];
+    cursor[c] = n ? atomicAdd(&b.fcur[c], (unsigned long long)n) : 0ull;
     hist[PAD(c)] = 0;
   }
   for (int i = t; i < kHllRegs; i += NT) hll_s[i] = 0;
   if (t == 0) rcur_s = b.tile_first[tile];
-  for (int sub = 0; sub < kTileWords / NW; ++sub) {
-    const uint64_t j0 = tile * kTileWords + (uint64_t)sub * NW;
+  for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
+    const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
     if (j0 >= s.n_words) break;
     __syncthreads();
     if (t < 2) {
@@ -936,11 +909,7 @@ template <int KW, int NT, bool KEEP_C>
 __global__ void __launch_bounds__(NT, 2) k_scatter(Shape s, Buffers b) {
   scatter_body<KW, NT, KEEP_C>(s, b, blockIdx.x);
 }
-// Aggregation ablation: the partition cursors start at the partition starts, and pass B
-// writes every key on its own through them.
-__global__ void k_direct_cursors(const uint64_t* cstart, unsigned long long* cur, int P1) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < P1; c += gridDim.x * blockDim.x) cur[c] = cstart[c];
-}
+// Aggregation ablation: pass B writes every key on its own through the partition cursors.
 template <int KW>
 __global__ void __launch_bounds__(256, 2) k_scatter_direct(Shape s, Buffers b) {
   scatter_body<KW, 256, false, true>(s, b, blockIdx.x);
@@ -2344,7 +2313,7 @@ int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, con
     KC_STEP("k_check_offsets");
   }
   if (s.n_tiles == 0) return launches;
-  k_tile_first<<<(unsigned)((s.n_tiles + 127) / 128), 128, 0, st>>>(b.offsets, s.n_reads, s.n_tiles, b.tile_first);
+  k_tile_first<<<(unsigned)((s.n_tiles + 127) / 128), 128, 0, st>>>(b.offsets, s, b.tile_first);
   ++launches;
   KC_STEP("k_tile_first");
   const size_t smA = (size_t)(P1 + 32) * 4;
@@ -2352,9 +2321,6 @@ int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, con
   else k_pack_count<2><<<(unsigned)s.n_tiles, kPackThreads, smA, st>>>(s, b);
   ++launches;
   KC_STEP("k_pack_count");
-  k_col_scan<<<(unsigned)((P1 + 31) / 32), dim3(32, 32), 0, st>>>(b.hist, b.toff, b.cstart /* as ccount */, s.n_tiles, P1);
-  ++launches;
-  KC_STEP("k_col_scan");
   return launches;
 }
 
@@ -2362,9 +2328,9 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
   cudaStream_t st = (cudaStream_t)stream;
   const int P1 = 1 << s.b1;
   int launches = 0;
-  // partition starts (cstart holds the per-partition counts written by k_col_scan; the
-  // scan reads them into shared memory before overwriting)
-  k_bucket_scan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.cstart, P1, b.meta);
+  // partition starts (cstart holds the per-partition totals added up by pass A; the scan
+  // reads them into shared memory before overwriting)
+  k_bucket_scan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.cstart, b.fcur, P1, b.meta);
   ++launches;
   KC_STEP("k_bucket_scan");
   if (s.n_tiles > 0) {
@@ -2377,9 +2343,6 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     const bool keep_c = per_sm >= 2;
     const unsigned gt = (unsigned)s.n_tiles;
     if (s.aggr & kAggrNoSmemBuckets) {
-      k_direct_cursors<<<(P1 + 255) / 256, 256, 0, st>>>(b.cstart, b.fcur, P1);
-      ++launches;
-      KC_STEP("k_direct_cursors");
       if (s.kw == 1) k_scatter_direct<1><<<gt, 256, smB, st>>>(s, b);
       else k_scatter_direct<2><<<gt, 256, smB, st>>>(s, b);
     } else if (s.kw == 1) {
@@ -2440,13 +2403,12 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
 
 uint32_t batch_blocks(BatchKernel k, const Shape& s, int n_sms, uint64_t bases_total) {
   auto clampu = [](uint64_t v, uint64_t lo, uint64_t hi) { return (uint32_t)(v < lo ? lo : (v > hi ? hi : v)); };
-  const uint64_t P1 = 1ull << s.b1, nsm = (uint64_t)n_sms;
+  const uint64_t nsm = (uint64_t)n_sms;
   switch (k) {
     case BK_CLEAR: return clampu((s.nf_max + 2047) / 2048, 1, 32);
     case BK_CHECK: return clampu((s.n_reads + 255) / 256, 1, 64);
     case BK_TILE_FIRST: return (uint32_t)((s.n_tiles + 127) / 128);
     case BK_PACK: return (uint32_t)s.n_tiles;
-    case BK_COL_SCAN: return s.n_tiles ? (uint32_t)((P1 + 31) / 32) : 0u;
     case BK_SCATTER: return (uint32_t)s.n_tiles;
     case BK_FINE_HIST:
     case BK_FINE_SCATTER: return clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
@@ -2484,8 +2446,6 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
     KC_BLAUNCH(BK_PACK, (k_pack_count_batch<2><<<bp.grid[BK_PACK], kPackThreads, (size_t)(P1 + 32) * 4, st>>>(tab(BK_PACK))),
                "k_pack_count");
   }
-  KC_BLAUNCH(BK_COL_SCAN, (k_col_scan_batch<<<bp.grid[BK_COL_SCAN], dim3(32, 32), 0, st>>>(tab(BK_COL_SCAN))),
-             "k_col_scan");
   KC_BLAUNCH(BK_BUCKET_SCAN,
              (k_bucket_scan_batch<<<bp.grid[BK_BUCKET_SCAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_BUCKET_SCAN))),
              "k_bucket_scan");
