@@ -1387,16 +1387,13 @@ struct Table {
 };
 
 // Count kernel shared memory: a hash table of 2^bT_max slots (key + count), a bucket
-// histogram of hist_max(kw) entries and the 16-bit slot numbers of up to 3/4 of the slots
-// in output order.
+// histogram of 16-bit entries (at most one bucket per slot, and the end of the last), and for
+// up to 3/4 of the slots, grouped by bucket, the slot numbers and (64-bit keys) the keys.
 constexpr int kTableLog2Cap = kCountThreads == 1024 ? 13 : 12;  // 8 slots per thread
-__host__ __device__ constexpr int hist_max(int kw) {
-  return kCountThreads == 1024 ? (kw == 1 ? 16384 : 8192) : 4096;
-}
 
 size_t count_kernel_smem(int kw, int bT_max, int /*unused*/) {
   const size_t slots = (size_t)1 << bT_max;
-  return slots * (size_t)(kw * 8 + 4) + padded_len(hist_max(kw)) * 4 + ((3 * slots) >> 2) * 2 + 256;
+  return slots * (size_t)(kw * 8 + 4) + slots * 2 + 16 + ((3 * slots) >> 2) * (kw == 1 ? 10 : 2) + 256;
 }
 
 // The largest table whose block (8 KB of static shared memory included) fits the opt-in
@@ -1478,63 +1475,79 @@ __device__ __forceinline__ int count_insert(Table<KW> tb, typename KeyT<KW>::T k
   return 0;
 }
 
+// An empty table and an empty bucket histogram (at most one bucket per slot).
 template <int KW>
-__device__ __forceinline__ void table_clear(Table<KW> tb, uint32_t nslots) {
+__device__ __forceinline__ void table_clear(Table<KW> tb, uint32_t nslots, uint32_t* hist, uint32_t* big_n) {
   typedef typename KeyT<KW>::T K;
   for (uint32_t i = threadIdx.x; i < nslots; i += blockDim.x) {
     tb.keys[i] = all_ones<K>();
     tb.counts[i] = 0;
   }
+  for (uint32_t i = threadIdx.x; i < nslots / 2; i += blockDim.x) hist[i] = 0;
+  if (threadIdx.x == 0) *big_n = 0;
 }
 
-// Count the keys in[0, n) (only those in [lo, hi] when `ranged`).  The all-ones key is
-// counted apart in *special (it marks empty slots); it exists only when the k-mer fills
-// the key word (full_width).  Sets *ovf if a key found no slot.
+// Clear the table and count the keys in[0, n) (only those in [lo, hi] when `ranged`).  The
+// all-ones key is counted apart in *special (it marks empty slots); it exists only when the
+// k-mer fills the key word (full_width).  Sets *ovf if a key found no slot.  Each thread's
+// first keys are loaded before the table is cleared, and its next keys before the current ones
+// are inserted, so that a load's latency is covered by the clearing or by the inserts.
 // With MERGE, a warp whose active keys are all equal adds them with one atomic (the
 // heavy-hitter merge of the paper's L3 layer); without it (the default) every key is added
 // on its own: on GB300 the shared-memory atomics absorb equal keys faster than the merge's
 // warp vote costs, even for a single key.
 template <int KW, bool MERGE = false>
 __device__ void count_all(Table<KW> tb, const uint64_t* in, uint64_t n, bool ranged, typename KeyT<KW>::T lo,
-                          typename KeyT<KW>::T hi, int bT, bool full_width, uint32_t limit, uint32_t* n_new,
-                          uint32_t* ovf, uint32_t* special, uint32_t* status) {
+                          typename KeyT<KW>::T hi, int bT, bool full_width, uint32_t limit, uint32_t* hist,
+                          uint32_t* big_n, uint32_t* n_new, uint32_t* ovf, uint32_t* special, uint32_t* status) {
   typedef typename KeyT<KW>::T K;
-  constexpr int kIn = KW == 1 ? 8 : 2;  // loads in flight per thread (u128 keys: register-bound at 64)
+  constexpr int kIn = KW == 1 ? 4 : 2;  // keys per thread and batch (two batches held: register-bound at 64)
   const K EMPTY = all_ones<K>();
   const int lane = threadIdx.x & 31;
   const bool check = n > limit;  // a count can pass the limit only in a partition that large
   uint32_t claimed = 0;
-  for (uint64_t base = 0; base < n; base += kIn * (uint64_t)blockDim.x) {
-    K kk[kIn];
-    bool aa[kIn];
+  K nxt[kIn];
+  auto load = [&](uint64_t base) {
 #pragma unroll
     for (int m = 0; m < kIn; ++m) {
       const uint64_t i = base + (uint64_t)m * blockDim.x + threadIdx.x;
-      kk[m] = 0;
-      aa[m] = i < n;
-      if (aa[m]) load_key(in, i, kk[m]);
+      nxt[m] = 0;
+      if (i < n) load_key(in, i, nxt[m]);
     }
+  };
+  load(0);
+  table_clear<KW>(tb, 1u << bT, hist, big_n);
+  block_sync();
+  for (uint64_t base = 0; base < n; base += kIn * (uint64_t)blockDim.x) {
+    K kk[kIn];
+#pragma unroll
+    for (int m = 0; m < kIn; ++m) kk[m] = nxt[m];
+    load(base + kIn * (uint64_t)blockDim.x);
 #pragma unroll
     for (int m = 0; m < kIn; ++m) {
       const K key = kk[m];
-      bool act = aa[m];
+      bool act = base + (uint64_t)m * blockDim.x + threadIdx.x < n;
       if (ranged) act = act && key >= lo && key <= hi && key != EMPTY;
-      // a warp whose active keys all equal lane 0's key (a heavy hitter) adds them at once;
-      // lane 0's own key counts only if it is active, so any inactive lane 0 is harmless
-      const K k0 = shfl_key(key, 0);
-      if (MERGE && __all_sync(0xffffffffu, !act || key == k0)) {
-        const unsigned am = __ballot_sync(0xffffffffu, act);
-        if (am && lane == __ffs(am) - 1) {
-          const uint32_t inc = __popc(am);
-          if (full_width && k0 == EMPTY) {
-            if (atomicAdd(special, inc) > limit - inc) atomicOr(status, ST_COUNT_OVERFLOW);
-          } else {
-            const int r = count_insert<KW>(tb, k0, inc, bT, check, limit, status);
-            if (!r) atomicOr(ovf, 1u);
-            claimed += r == 2;
+      if constexpr (MERGE) {
+        // a warp whose active keys all equal lane 0's key (a heavy hitter) adds them at once;
+        // lane 0's own key counts only if it is active, so any inactive lane 0 is harmless
+        const K k0 = shfl_key(key, 0);
+        if (__all_sync(0xffffffffu, !act || key == k0)) {
+          const unsigned am = __ballot_sync(0xffffffffu, act);
+          if (am && lane == __ffs(am) - 1) {
+            const uint32_t inc = __popc(am);
+            if (full_width && k0 == EMPTY) {
+              if (atomicAdd(special, inc) > limit - inc) atomicOr(status, ST_COUNT_OVERFLOW);
+            } else {
+              const int r = count_insert<KW>(tb, k0, inc, bT, check, limit, status);
+              if (!r) atomicOr(ovf, 1u);
+              claimed += r == 2;
+            }
           }
+          continue;
         }
-      } else if (act) {
+      }
+      if (act) {
         if (full_width && key == EMPTY) {
           if (atomicAdd(special, 1u) >= limit) atomicOr(status, ST_COUNT_OVERFLOW);
         } else {
@@ -1627,19 +1640,22 @@ constexpr int kRankRegs = (kRankPer + 1) / 2;  // ranks (< 2^13) are kept two pe
 __device__ __forceinline__ uint32_t rank_get(const uint32_t (&rk)[kRankRegs], int m) {
   return (rk[m >> 1] >> (16 * (m & 1))) & 0xffffu;
 }
-constexpr uint32_t kBigBucket = 256;  // buckets above this are sorted by a warp, not ranked by counting
+// buckets above this are sorted by a warp, not ranked by counting
+__host__ __device__ constexpr uint32_t big_bucket(int kw) { return kw == 1 ? 512 : 256; }
+constexpr int kBigMax = 32;  // more than d / big_bucket <= 6144 / 257
 
-constexpr int kBigMax = 32;  // more than d / kBigBucket <= 6144 / 257
-
-// Exclusive scan of the padded array data (logical element i at data[PAD(i)]) by the
-// worker warps (warp 0 is busy with the look-back meanwhile); returns the total.
-__device__ uint32_t workers_exclusive_scan_pad(uint32_t* data, int n, uint32_t* warp_tmp) {
+// Exclusive scan of `words` words of two 16-bit counts each (worker warps; warp 0 is busy with
+// the look-back meanwhile).  The total fits in 16 bits.
+__device__ void workers_exclusive_scan16(uint32_t* data, int words, uint32_t* warp_tmp) {
   constexpr int nt = kWorkers, nw = kWorkers / 32;
   const int t = threadIdx.x - 32, lane = t & 31, wid = t >> 5;
-  const int per = (n + nt - 1) / nt;
-  const int lo = min(n, t * per), hi = min(n, lo + per);
+  const int per = ((words + nt - 1) / nt) | 1;  // odd: the threads' words fall in distinct banks
+  const int lo = min(words, t * per), hi = min(words, lo + per);
   uint32_t s = 0;
-  for (int i = lo; i < hi; ++i) s += data[PAD(i)];
+  for (int i = lo; i < hi; ++i) {
+    const uint32_t v = data[i];
+    s += (v & 0xffffu) + (v >> 16);
+  }
   uint32_t x = s;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -1648,38 +1664,59 @@ __device__ uint32_t workers_exclusive_scan_pad(uint32_t* data, int n, uint32_t* 
   }
   if (lane == 31) warp_tmp[wid] = x;
   bar_workers();
-  if (wid == 0) {
-    uint32_t w = lane < nw ? warp_tmp[lane] : 0;
+  // every warp adds up the warps before it (no second barrier for a scan by one warp)
+  uint32_t before = lane < wid && lane < nw ? warp_tmp[lane] : 0;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, w, d);
-      if (lane >= d) w += y;
-    }
-    if (lane < nw) warp_tmp[lane] = w;
-  }
-  bar_workers();
-  uint32_t run = x - s + (wid ? warp_tmp[wid - 1] : 0);
-  const uint32_t total = warp_tmp[nw - 1];
+  for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+  uint32_t run = before + x - s;
   for (int i = lo; i < hi; ++i) {
-    const uint32_t v = data[PAD(i)];
-    data[PAD(i)] = run;
-    run += v;
+    const uint32_t v = data[i], a = v & 0xffffu;
+    data[i] = run | ((run + a) << 16);
+    run += a + (v >> 16);
   }
   bar_workers();
-  return total;
 }
 
-// Order the table's d occupied slots for output (worker warps only).  The key range
-// [lo, hi] of the table is read from range_s[0..1] (written by worker 0 before the call).  NB
-// buckets (key - lo) >> sh, one to two per key; an ordered counting sort of the slot
-// numbers into idx[0, d), bucket by bucket (buckets ascending, slots unordered inside a
-// bucket); hist[PAD(b)] is left holding bucket b's first position, and big_s[0, *big_n)
-// lists the buckets above kBigBucket entries.
+// The buckets of a table's keys inside their range [lo, lo + width]: the top bB bits of
+// (key - lo), aligned to the width of the range.
+template <class K>
+struct OrderMap {
+  K lo, width;
+  int rs, ls;  // w = low word of ((key - lo) >> rs), << ls
+  int bs;      // bucket = w >> bs
+};
+template <class K>
+__device__ __forceinline__ OrderMap<K> order_map(K lo, K hi, uint32_t NB) {
+  OrderMap<K> o;
+  o.lo = lo;
+  o.width = hi - lo;
+  const int nb = bitlen(o.width);
+  o.rs = nb > 32 ? nb - 32 : 0;
+  o.ls = nb >= 32 ? 0 : min(32 - nb, 31);  // nb = 0: the only offset is 0
+  o.bs = 32 - (31 - __clz(NB));
+  return o;
+}
+__device__ __forceinline__ uint32_t bucket_of(uint64_t off, const OrderMap<uint64_t>& o) {
+  return (__funnelshift_rc((uint32_t)off, (uint32_t)(off >> 32), o.rs) << o.ls) >> o.bs;
+}
+__device__ __forceinline__ uint32_t bucket_of(u128 off, const OrderMap<u128>& o) {
+  const uint32_t o0 = (uint32_t)off, o1 = (uint32_t)(off >> 32), o2 = (uint32_t)(off >> 64), o3 = (uint32_t)(off >> 96);
+  const int q = o.rs >> 5;
+  const uint32_t a = q == 0 ? o0 : (q == 1 ? o1 : (q == 2 ? o2 : o3));
+  const uint32_t b = q == 0 ? o1 : (q == 1 ? o2 : (q == 2 ? o3 : 0u));
+  return (__funnelshift_r(a, b, o.rs & 31) << o.ls) >> o.bs;
+}
+
+// Group the table's d occupied slots by bucket (worker warps only): an ordered counting sort
+// of the slot numbers into idx[0, d) and, for 64-bit keys, of the keys into gkey[0, d), buckets
+// ascending, slots unordered inside a bucket.  hist (cleared before) is left holding bucket
+// b's first position in its b-th 16 bits, d after the last; big_s[0, *big_n) lists the
+// buckets above kBigBucket entries.
 template <int KW>
-__device__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, const typename KeyT<KW>::T* range_s,
-                             uint32_t* hist, uint16_t* idx, uint32_t* wtmp, uint32_t* big_s, uint32_t* big_n,
-                             typename KeyT<KW>::T& lo, int& sh, uint32_t& NB, uint32_t* status,
-                             unsigned long long* prof = nullptr) {
+__device__ __forceinline__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, uint32_t NB,
+                                             const OrderMap<typename KeyT<KW>::T>& o, uint32_t* hist, uint16_t* idx,
+                                             uint64_t* gkey, uint32_t* wtmp, uint32_t* big_s, uint32_t* big_n,
+                                             uint32_t* status, unsigned long long* prof = nullptr) {
   typedef typename KeyT<KW>::T K;
   const K EMPTY = all_ones<K>();
   long long tm = clock64();
@@ -1691,16 +1728,6 @@ __device__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, const ty
       tm = now;
     }
   };
-  NB = 1;
-  while (NB < (uint32_t)hist_max(KW) && NB < d) NB <<= 1;
-  for (uint32_t i = t; i < NB; i += kWorkers) hist[PAD(i)] = 0;
-  if (t == 0) *big_n = 0;
-  bar_workers();
-  mark(2);
-  lo = range_s[0];
-  const K hi = range_s[1];
-  const int bB = 31 - __clz(NB);
-  sh = d == 0 ? 0 : max(0, bitlen(K(hi - lo)) - bB);
   uint32_t br[kSlotsPerWorker];
 #pragma unroll
   for (int m = 0; m < kSlotsPerWorker; ++m) {
@@ -1709,13 +1736,15 @@ __device__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, const ty
     if (s < nslots) {
       const K key = tb.keys[s];
       if (key != EMPTY) {
-        if (key < lo || key > hi) {  // cannot happen: the range holds every key of the table
+        const K off = key - o.lo;
+        if (off > o.width) {  // cannot happen: the range holds every key of the table
           atomicOr(status, ST_INTERNAL);
         } else {
-          const uint32_t bk = (uint32_t)((key - lo) >> sh);
-          const uint32_t r = atomicAdd(&hist[PAD(bk)], 1u);
-          br[m] = (bk << 16) | r;  // NB <= 2^14, rank < 2^16
-          if (r == kBigBucket) {   // the entry that takes bucket bk past kBigBucket
+          const uint32_t bk = bucket_of(off, o);
+          const uint32_t half = 16 * (bk & 1);
+          const uint32_t r = (atomicAdd(&hist[bk >> 1], 1u << half) >> half) & 0xffffu;
+          br[m] = (bk << 16) | r;  // bucket below 2^13, rank below 2^13
+          if (r == big_bucket(KW)) {   // the entry that takes bucket bk past big_bucket
             const uint32_t q = atomicAdd(big_n, 1u);
             if (q < kBigMax) big_s[q] = bk;
             else atomicOr(status, ST_INTERNAL);
@@ -1726,62 +1755,75 @@ __device__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, const ty
   }
   bar_workers();
   mark(5);
-  workers_exclusive_scan_pad(hist, (int)NB, wtmp);
+  if (t == 0) reinterpret_cast<uint16_t*>(hist)[NB] = (uint16_t)d;  // past the scanned words (NB > 1), or scanned as 0
+  workers_exclusive_scan16(hist, (int)(NB / 2), wtmp);
   mark(6);
+  const uint16_t* start = reinterpret_cast<const uint16_t*>(hist);
 #pragma unroll
   for (int m = 0; m < kSlotsPerWorker; ++m)
-    if (br[m] != 0xffffffffu) idx[hist[PAD(br[m] >> 16)] + (br[m] & 0xffffu)] = (uint16_t)(t + m * kWorkers);
+    if (br[m] != 0xffffffffu) {
+      const uint32_t pos = start[br[m] >> 16] + (br[m] & 0xffffu);
+      idx[pos] = (uint16_t)(t + m * kWorkers);
+      if constexpr (KW == 1) gkey[pos] = tb.keys[t + m * kWorkers];
+    }
   bar_workers();
   mark(7);
 }
 
-// Worker warps: the rank of the entry at each bucket-grouped position j (its bucket's
-// first position plus the number of smaller keys in the bucket).  The rare bucket above
-// kBigBucket entries is first sorted in place by one warp and ranked by position.
+// Worker warps: the rank of the entry at each bucket-grouped position j (its bucket's first
+// position plus the number of smaller keys in the bucket).  64-bit keys are read in grouped
+// order (consecutive words, no slot number first); 128-bit keys, for whose copies there is no
+// room, through their slot numbers.  The rare bucket above big_bucket entries is first sorted
+// in place by one warp and ranked by position (it pays above 512 keys: on the repeat genome,
+// whose copies' variants share long prefixes, sorting from 256 up and reading every key through
+// its slot number took 1147 M SM cycles of ranking and sorting, this takes 498 M).
 template <int KW>
-__device__ __forceinline__ void rank_slots(Table<KW> tb, const uint16_t* idx_c, uint16_t* idx, uint32_t d,
-                                           const uint32_t* hist, uint32_t NB, typename KeyT<KW>::T lo, int sh,
+__device__ __forceinline__ void rank_slots(Table<KW> tb, uint16_t* idx, const uint64_t* gkey, uint32_t d,
+                                           const uint32_t* hist, const OrderMap<typename KeyT<KW>::T>& o,
                                            const uint32_t* big_s, uint32_t n_big, uint32_t (&rank)[kRankRegs],
                                            unsigned long long* prof) {
   typedef typename KeyT<KW>::T K;
   const int t = threadIdx.x - 32, wid = t >> 5;
+  const uint16_t* start = reinterpret_cast<const uint16_t*>(hist);
   long long tm = clock64();
   constexpr int kWarps = kWorkers / 32;
-  if (n_big) {  // rare: one warp per big bucket
-    for (uint32_t q = wid; q < min(n_big, (uint32_t)kBigMax); q += kWarps) {
-      const uint32_t bk = big_s[q];
-      const uint32_t a = hist[PAD(bk)];
-      const uint32_t e = bk + 1 < NB ? hist[PAD(bk + 1)] : d;
-      warp_sort_idx<K>(tb.keys, idx, a, e - a);
-    }
-    bar_workers();
-  }
-  if (prof && t == 0) {
-    const long long now = clock64();
-    atomicAdd(&prof[3], (unsigned long long)(now - tm));
-    tm = now;
-  }
 #pragma unroll
   for (int m = 0; m < kRankRegs; ++m) rank[m] = 0xffffffffu;
 #pragma unroll
   for (int m = 0; m < kRankPer; ++m) {
     const uint32_t j = t + m * kWorkers;
     if (j < d) {
-      const K key = tb.keys[idx_c[j]];
-      const uint32_t bk = (uint32_t)((key - lo) >> sh);
-      const uint32_t a = hist[PAD(bk)];
-      const uint32_t e = bk + 1 < NB ? hist[PAD(bk + 1)] : d;
+      K key;
+      if constexpr (KW == 1) key = gkey[j];
+      else key = tb.keys[idx[j]];
+      const uint32_t bk = bucket_of((K)(key - o.lo), o);
+      const uint32_t a = start[bk], e = start[bk + 1];
       uint32_t r = a;
-      if (e - a > kBigBucket) {
+      if (e - a > big_bucket(KW)) {
         r = j;
       } else {
-        for (uint32_t q = a; q < e; ++q) r += tb.keys[idx_c[q]] < key;
+        for (uint32_t q = a; q < e; ++q) {
+          if constexpr (KW == 1) r += gkey[q] < key;
+          else r += tb.keys[idx[q]] < key;
+        }
       }
       const int sh = 16 * (m & 1);
       rank[m >> 1] = (rank[m >> 1] & ~(0xffffu << sh)) | (r << sh);
     }
   }
-  if (prof && t == 0) atomicAdd(&prof[4], (unsigned long long)(clock64() - tm));
+  if (prof && t == 0) {
+    const long long now = clock64();
+    atomicAdd(&prof[4], (unsigned long long)(now - tm));
+    tm = now;
+  }
+  if (n_big) {  // rare: one warp per big bucket (none of whose entries was looked up above)
+    bar_workers();
+    for (uint32_t q = wid; q < min(n_big, (uint32_t)kBigMax); q += kWarps) {
+      const uint32_t a = start[big_s[q]], e = start[big_s[q] + 1];
+      warp_sort_idx<K>(tb.keys, idx, a, e - a);
+    }
+  }
+  if (prof && t == 0) atomicAdd(&prof[3], (unsigned long long)(clock64() - tm));
 }
 
 // Worker threads: write the entry at each grouped position j to out[base + rank].  Ranks
@@ -1815,8 +1857,9 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
   extern __shared__ __align__(16) uint8_t sm[];
   const uint32_t cap_slots = 1u << s.bT_max;
   const uint32_t dcap = (3u * cap_slots) >> 2;  // most distinct keys a table is ordered with
-  uint32_t* hist = reinterpret_cast<uint32_t*>(sm + (size_t)cap_slots * (KW * 8 + 4));
-  uint16_t* idx = reinterpret_cast<uint16_t*>(hist + padded_len(hist_max(KW)));  // [dcap]
+  uint32_t* hist = reinterpret_cast<uint32_t*>(sm + (size_t)cap_slots * (KW * 8 + 4));  // [cap_slots / 2 + 4]
+  uint64_t* gkey = reinterpret_cast<uint64_t*>(hist + cap_slots / 2 + 4);               // [dcap] (KW == 1)
+  uint16_t* idx = reinterpret_cast<uint16_t*>(gkey + (KW == 1 ? dcap : 0));             // [dcap]
   __shared__ uint64_t excl_s, next_s[3];  // next ticket, its input range
   __shared__ volatile uint32_t ordered_s;  // the workers have ranked the current table
   __shared__ uint32_t next_u[2];          // its range-map interval: [next_u[0], next_u[1] - 1]
@@ -1877,6 +1920,13 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       if (threadIdx.x == 0) atomicOr(&b.meta->status, ST_INTERNAL);
       n = 0;
     }
+    if (threadIdx.x == blockDim.x - 1) {
+      // the partition's key range, from its range-map interval (flo[NF] = 0, so the last
+      // interval ends at 2^32 - 1); by a thread of the warp with the fewest keys to count
+      uint32_t xlo, xhi;
+      x_range(next_u[0], next_u[1] - 1u, s.canonical, xlo, xhi);
+      key_range(xlo, xhi, s.k, range_s[0], range_s[1]);
+    }
     const uint64_t* in = b.sbuf + f0 * KW;
     // table: at least twice the keys (at most that many distinct), within the cap
     int bT = 6;
@@ -1885,11 +1935,8 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
     tb.keys = reinterpret_cast<K*>(sm);
     tb.counts = reinterpret_cast<uint32_t*>(tb.keys + (1u << bT));
     phase(7);
-    table_clear<KW>(tb, 1u << bT);
-    block_sync();
-    phase(0);
-    count_all<KW, MERGE>(tb, in, n, false, K(0), K(0), bT, s.k == 32 * KW, s.count_limit, &nnew_s, &ovf_s,
-                         &special_s, &b.meta->status);
+    count_all<KW, MERGE>(tb, in, n, false, K(0), K(0), bT, s.k == 32 * KW, s.count_limit, hist, &big_n, &nnew_s,
+                         &ovf_s, &special_s, &b.meta->status);
     block_sync();
     phase(1);
     const uint32_t dn = nnew_s;
@@ -1921,22 +1968,12 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
         }
       } else {
         const long long tm = clock64();
-        if (threadIdx.x == 32) {
-          // every key of the partition lies in the key range of its range-map interval.
-          // next_u still holds this partition's interval (the next one is fetched during
-          // the write-out); flo[NF] = 0, so the last interval ends at 2^32 - 1
-          const uint32_t ulo = next_u[0], uhi = next_u[1] - 1u;
-          uint32_t xlo, xhi;
-          x_range(ulo, uhi, s.canonical, xlo, xhi);
-          key_range(xlo, xhi, s.k, range_s[0], range_s[1]);
-        }
-        K lo;
-        int sh;
-        uint32_t NB;
-        bucket_slots<KW>(tb, 1u << bT, dn, range_s, hist, idx, wtmp, big_s, &big_n, lo, sh, NB, &b.meta->status,
-                         prof);
+        uint32_t NB = 2;
+        while (NB < dn) NB <<= 1;
+        const OrderMap<K> om = order_map<K>(range_s[0], range_s[1], NB);
+        bucket_slots<KW>(tb, 1u << bT, dn, NB, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status, prof);
         if (prof && threadIdx.x == 32) atomicAdd(&prof[1], (unsigned long long)(clock64() - tm));
-        rank_slots<KW>(tb, idx, idx, dn, hist, NB, lo, sh, big_s, big_n, rank, prof);
+        rank_slots<KW>(tb, idx, gkey, dn, hist, om, big_s, big_n, rank, prof);
         bar_workers();
         if (threadIdx.x == 32) ordered_s = 1;
       }
@@ -2011,10 +2048,8 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
           special_s = 0;
           nnew_s = 0;
         }
-        table_clear<KW>(tb, cap_slots);
-        block_sync();
-        count_all<KW, MERGE>(tb, in, n, true, lo, hi, bTf, s.k == 32 * KW, s.count_limit, &nnew_s, &ovf_s,
-                             &special_s, &b.meta->status);
+        count_all<KW, MERGE>(tb, in, n, true, lo, hi, bTf, s.k == 32 * KW, s.count_limit, hist, &big_n, &nnew_s,
+                             &ovf_s, &special_s, &b.meta->status);
         block_sync();
         const uint32_t dn2 = nnew_s;
         const K width = hi - lo;
@@ -2038,16 +2073,11 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
         {
           uint32_t rank2[kRankRegs];
           if (wid > 0) {
-            if (threadIdx.x == 32) {
-              range_s[0] = lo;
-              range_s[1] = hi;
-            }
-            K lo2;
-            int sh2;
-            uint32_t NB2;
-            bucket_slots<KW>(tb, cap_slots, dn2, range_s, hist, idx, wtmp, big_s, &big_n, lo2, sh2, NB2,
-                             &b.meta->status);
-            rank_slots<KW>(tb, idx, idx, dn2, hist, NB2, lo2, sh2, big_s, big_n, rank2, nullptr);
+            uint32_t NB2 = 2;
+            while (NB2 < dn2) NB2 <<= 1;
+            const OrderMap<K> om = order_map<K>(lo, hi, NB2);
+            bucket_slots<KW>(tb, cap_slots, dn2, NB2, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status);
+            rank_slots<KW>(tb, idx, gkey, dn2, hist, om, big_s, big_n, rank2, nullptr);
           }
           block_sync();
           if (wid > 0) emit_slots<KW>(tb, idx, dn2, rank2, base, b.out_keys, b.out_counts, s.cap, &b.meta->status);
