@@ -1079,7 +1079,12 @@ __device__ __forceinline__ uint64_t fine_region(const Shape& sh, const Buffers& 
   const uint64_t n_c = e - a, s_c = sampled_below(e) - sampled_below(a);
   if (s_c < 1024) return n_c;
   const float f = (float)n_c / (float)s_c, cnt = (float)b.fhist[g];
-  const float slack = sh.tight_slack ? 0.f : 5.5f * f * sqrtf(cnt + 1.f) + 16.f;
+  float slack = sh.tight_slack ? 0.f : 5.5f * f * sqrtf(cnt + 1.f) + 16.f;
+  // a partition far above its coarse partition's average holds k-mers of tandem repeats, which
+  // come many at a time (a read inside an array holds each of them 20 times and more), so its
+  // sampled count varies more than a random sample's: an eighth on top.  (Without it, 72 M
+  // windows with 3% satellite arrays took the exact split again in most counts, 225 to 350 us.)
+  if (!sh.tight_slack && cnt * (float)b.fine_m[c] > 4.f * (float)s_c) slack += 0.125f * f * cnt;
   const uint64_t r = (uint64_t)(cnt * f + slack) + (sh.tight_slack ? 0 : 1);
   return r < n_c ? r : n_c;
 }
@@ -1396,7 +1401,7 @@ size_t count_kernel_smem(int kw, int bT_max, int /*unused*/) {
   return slots * (size_t)(kw * 8 + 4) + slots * 2 + 16 + ((3 * slots) >> 2) * (kw == 1 ? 10 : 2) + 256;
 }
 
-// The largest table whose block (8 KB of static shared memory included) fits the opt-in
+// The largest table whose block (12 KB of static shared memory included) fits the opt-in
 // limit, with kCountBlocksPerSM blocks on one SM (each also keeps 1 KB for the system).
 int table_log2_max(int kw, size_t smem_optin, size_t smem_per_sm) {
   size_t budget = smem_optin;
@@ -1406,7 +1411,7 @@ int table_log2_max(int kw, size_t smem_optin, size_t smem_per_sm) {
   }
   int best = 6;
   for (int bt = 6; bt <= kTableLog2Cap; ++bt)
-    if (count_kernel_smem(kw, bt, 0) + 8192 <= budget) best = bt;
+    if (count_kernel_smem(kw, bt, 0) + 12288 <= budget) best = bt;
   return best;
 }
 
@@ -1572,41 +1577,29 @@ template <> __device__ __forceinline__ int bitlen(u128 v) {
   return hi ? 128 - __clzll(hi) : 64 - __clzll((uint64_t)v);
 }
 
-// Block-wide min of mn and max of mx (all threads; the result is returned to all).
+// The median of up to kSplitSample keys taken from a table's slots (all threads; at least two
+// sampled keys lie in [lo, hi], else false): *out is in (lo, hi].  samp: kSplitSample entries.
+constexpr int kSplitSample = 256;
 template <class K>
-__device__ void block_range(K mn, K mx, K* red_lo, K* red_hi, K& lo, K& hi) {
-  const K EMPTY = ~(K)0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int dd = 16; dd > 0; dd >>= 1) {
-    const K a = shfl_key(mn, (lane + dd) & 31), c = shfl_key(mx, (lane + dd) & 31);
-    mn = a < mn ? a : mn;
-    mx = c > mx ? c : mx;
+__device__ bool median_key(const K* keys, uint32_t nslots, K lo, K hi, K* samp, K* out) {
+  const K EMPTY = all_ones<K>();
+  const uint32_t step = nslots > kSplitSample ? nslots / kSplitSample : 1;
+  const uint32_t n = min(nslots, (uint32_t)kSplitSample);
+  block_sync();
+  K mine = EMPTY;
+  if (threadIdx.x < n) {
+    mine = keys[threadIdx.x * step];
+    if (mine < lo || mine > hi) mine = EMPTY;
+    samp[threadIdx.x] = mine;
   }
-  if (lane == 0) {
-    red_lo[wid] = mn;
-    red_hi[wid] = mx;
+  const uint32_t have = __syncthreads_count(mine != EMPTY);
+  if (mine != EMPTY) {
+    uint32_t below = 0;
+    for (uint32_t i = 0; i < n; ++i) below += samp[i] < mine;
+    if (below == have / 2) *out = mine;
   }
-  __syncthreads();
-  if (wid == 0) {  // one warp combines the per-warp results
-    const int nw = (int)(blockDim.x >> 5);
-    mn = lane < nw ? red_lo[lane] : EMPTY;
-    mx = lane < nw ? red_hi[lane] : K(0);
-#pragma unroll
-    for (int dd = 16; dd > 0; dd >>= 1) {
-      const K a = shfl_key(mn, (lane + dd) & 31), c = shfl_key(mx, (lane + dd) & 31);
-      mn = a < mn ? a : mn;
-      mx = c > mx ? c : mx;
-    }
-    __syncwarp();
-    if (lane == 0) {
-      red_lo[0] = mn;
-      red_hi[0] = mx;
-    }
-  }
-  __syncthreads();
-  lo = red_lo[0];
-  hi = red_hi[0];
+  block_sync();
+  return have >= 2;
 }
 
 // Sort idx[a, a+c) by the keys the slots hold, by one warp: a bitonic network whose
@@ -1865,7 +1858,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
   __shared__ uint32_t next_u[2];          // its range-map interval: [next_u[0], next_u[1] - 1]
   __shared__ uint32_t ovf_s, special_s, nnew_s;
   __shared__ uint32_t wtmp[32];
-  __shared__ K red_lo[32], red_hi[32];
+  __shared__ K split_s, samp_s[kSplitSample];
   __shared__ K stk_lo[160], stk_hi[160];
   __shared__ K range_s[2];
   __shared__ uint32_t big_s[kBigMax], big_n;
@@ -2007,31 +2000,27 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       // partition's key range into sub-ranges, each counted in its own table and ordered;
       // the exclusive prefix is resolved first because the partial outputs are written
       // before the total is known.  A sub-range narrower than the table holds fewer
-      // distinct keys than slots, so the splitting ends.
+      // distinct keys than slots, so the splitting ends.  The range is split at the median of a
+      // sample of the keys in the table that overflowed, not in its middle: the keys that make
+      // a partition overflow are mostly variants of a repeat and share long prefixes, so that
+      // halving the range leaves them together for many passes over the partition's keys.
+      // (72 M windows, 3% of them satellite arrays: count kernel 1271 -> 721 us.)
       if (wid == 0) {
         const uint64_t ex = g == 0 ? 0 : lookback(b.look, g, &b.meta->status, s.spin_limit);
         if (lane == 0) excl_s = ex;
       }
       if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&b.meta->n_overflow), 1ull);
-      K mn = EMPTY, mx = 0;
-      for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        K key;
-        load_key(in, i, key);
-        if (key != EMPTY) {
-          mn = key < mn ? key : mn;
-          mx = key > mx ? key : mx;
-        }
-      }
       {
-        K a, c;
-        block_range<K>(mn, mx, red_lo, red_hi, a, c);
+        // the table just filled holds a sample of the partition's distinct keys (unless it was
+        // a smaller table than the largest): the first split is at their median
+        const K lo = range_s[0], hi = range_s[1];
+        const bool split = bT == s.bT_max && median_key<K>(tb.keys, cap_slots, lo, hi, samp_s, &split_s);
         if (threadIdx.x == 0) {
-          stk_n = 0;
-          if (a <= c) {
-            stk_lo[0] = a;
-            stk_hi[0] = c;
-            stk_n = 1;
-          }
+          stk_lo[0] = split ? split_s : lo;
+          stk_hi[0] = hi;
+          stk_lo[1] = lo;
+          stk_hi[1] = split ? split_s - 1 : hi;
+          stk_n = split ? 2 : 1;
         }
       }
       block_sync();
@@ -2052,17 +2041,16 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
                              &ovf_s, &special_s, &b.meta->status);
         block_sync();
         const uint32_t dn2 = nnew_s;
-        const K width = hi - lo;
         if (ovf_s || dn2 > dcap) {
+          const bool split = median_key<K>(tb.keys, cap_slots, lo, hi, samp_s, &split_s);
           if (threadIdx.x == 0) {
-            if (width == 0 || stk_n + 2 > 160) {
-              atomicOr(&b.meta->status, ST_INTERNAL);  // a single key cannot overflow
+            if (!split || stk_n + 2 > 160) {
+              atomicOr(&b.meta->status, ST_INTERNAL);  // a table that overflowed holds many keys
             } else {
-              const K mid = lo + (width >> 1);
-              stk_lo[stk_n] = mid + 1;
+              stk_lo[stk_n] = split_s;
               stk_hi[stk_n] = hi;
               stk_lo[stk_n + 1] = lo;
-              stk_hi[stk_n + 1] = mid;
+              stk_hi[stk_n + 1] = split_s - 1;
               stk_n += 2;
             }
           }
@@ -2087,10 +2075,12 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       }
       // the all-ones key, if present, is the largest key of all
       uint32_t sp = 0;
-      for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        K key;
-        load_key(in, i, key);
-        sp += key == EMPTY;
+      if (s.k == 32 * KW) {
+        for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
+          K key;
+          load_key(in, i, key);
+          sp += key == EMPTY;
+        }
       }
   #pragma unroll
       for (int dd = 16; dd > 0; dd >>= 1) sp += __shfl_xor_sync(0xffffffffu, sp, dd);
