@@ -1415,7 +1415,7 @@ int table_log2_max(int kw, size_t smem_optin, size_t smem_per_sm) {
   return best;
 }
 
-constexpr int kProbeLimit = 128;
+constexpr int kProbeLimit = 64;  // at the 3/4 load that a table is ordered with, 1 key in 10^8 probes longer
 constexpr int kWorkers = kCountThreads - 32;  // warps 1.. load and sort while warp 0 looks back
 constexpr int kSlotsPerWorker = ((1 << kTableLog2Cap) + kWorkers - 1) / kWorkers;
 
@@ -1528,6 +1528,11 @@ __device__ void count_all(Table<KW> tb, const uint64_t* in, uint64_t n, bool ran
 #pragma unroll
     for (int m = 0; m < kIn; ++m) kk[m] = nxt[m];
     load(base + kIn * (uint64_t)blockDim.x);
+    if (ranged) {  // a key without a slot: this part is counted again in smaller ones, so stop here
+      bool stop = *reinterpret_cast<volatile uint32_t*>(ovf) != 0;
+      if constexpr (MERGE) stop = __any_sync(0xffffffffu, stop);  // the merge below takes whole warps
+      if (stop) break;
+    }
 #pragma unroll
     for (int m = 0; m < kIn; ++m) {
       const K key = kk[m];
@@ -2005,11 +2010,8 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       // a partition overflow are mostly variants of a repeat and share long prefixes, so that
       // halving the range leaves them together for many passes over the partition's keys.
       // (72 M windows, 3% of them satellite arrays: count kernel 1271 -> 721 us.)
-      if (wid == 0) {
-        const uint64_t ex = g == 0 ? 0 : lookback(b.look, g, &b.meta->status, s.spin_limit);
-        if (lane == 0) excl_s = ex;
-      }
       if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&b.meta->n_overflow), 1ull);
+      bool have_prefix = false;
       {
         // the table just filled holds a sample of the partition's distinct keys (unless it was
         // a smaller table than the largest): the first split is at their median
@@ -2057,17 +2059,23 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
           block_sync();
           continue;
         }
-        const uint64_t base = excl_s + written;
         {
           uint32_t rank2[kRankRegs];
-          if (wid > 0) {
+          if (wid == 0) {  // the prefix is waited for while the first part is ordered
+            if (!have_prefix) {
+              const uint64_t ex = g == 0 ? 0 : lookback(b.look, g, &b.meta->status, s.spin_limit);
+              if (lane == 0) excl_s = ex;
+            }
+          } else {
             uint32_t NB2 = 2;
             while (NB2 < dn2) NB2 <<= 1;
             const OrderMap<K> om = order_map<K>(lo, hi, NB2);
             bucket_slots<KW>(tb, cap_slots, dn2, NB2, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status);
             rank_slots<KW>(tb, idx, gkey, dn2, hist, om, big_s, big_n, rank2, nullptr);
           }
+          have_prefix = true;
           block_sync();
+          const uint64_t base = excl_s + written;
           if (wid > 0) emit_slots<KW>(tb, idx, dn2, rank2, base, b.out_keys, b.out_counts, s.cap, &b.meta->status);
         }
         written += dn2;
