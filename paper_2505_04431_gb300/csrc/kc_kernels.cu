@@ -799,17 +799,10 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
     if (j0 >= s.n_words) break;
     __syncthreads();
-    if (t < 2) {
-      if (sub > 0) {
-        code_s[t] = code_s[NW + t];
-        inv_s[t] = inv_s[NW + t];
-      } else if (j0 + t >= 2) {
-        code_s[t] = b.codes64[j0 + t - 2];
-        inv_s[t] = b.inv32[j0 + t - 2];
-      } else {
-        code_s[t] = 0;
-        inv_s[t] = ~0u;
-      }
+    if (t < 2) {  // the two words before: from memory again (the shared copies are being overwritten)
+      const bool in = j0 + t >= 2;
+      code_s[t] = in ? b.codes64[j0 + t - 2] : 0;
+      inv_s[t] = in ? b.inv32[j0 + t - 2] : ~0u;
     }
     for (int w = t; w < NW; w += NT) {
       const uint64_t jw = j0 + w;
