@@ -534,10 +534,10 @@ __device__ __forceinline__ uint32_t top32_shl(uint64_t a, uint64_t b, int sh) {
 // value's top word: where the top words differ they decide which value is smaller, and
 // where they tie both values share them.
 template <int KW, int WPT>
-__device__ __forceinline__ uint32_t win_top32(const Win& W, int i, int canonical) {
+__device__ __forceinline__ uint32_t win_top32(const Win& W, int i, int canonical, uint32_t& f, uint32_t& r) {
   const uint32_t m = (uint32_t)(W.m0 >> 32);
-  const uint32_t f = top32_shl(W.s0, W.s1, 2 * i) & m;
-  const uint32_t r = top32_shl(W.r0, W.r1, 2 * (WPT - 1 - i)) & m;
+  f = top32_shl(W.s0, W.s1, 2 * i) & m;
+  r = top32_shl(W.r0, W.r1, 2 * (WPT - 1 - i)) & m;
   return canonical ? min(f, r) : f;
 }
 __device__ __forceinline__ void top_to_key(uint64_t c0, uint64_t, int k, uint64_t& key) {
@@ -609,7 +609,8 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
       win_setup<KW, 32>(code_s[t], code_s[t + 1], code, vm, 0, s.k, W);
 #pragma unroll
       for (int i = 0; i < 32; ++i) {  // an invalid window goes to bin P1 + lane, never read: no branch
-        const uint32_t c = coarse_field(umap(win_top32<KW, 32>(W, i, s.canonical), s.canonical), s.b1);
+        uint32_t f, r;
+        const uint32_t c = coarse_field(umap(win_top32<KW, 32>(W, i, s.canonical, f, r), s.canonical), s.b1);
         atomicAdd(&hist_s[((W.valid >> i) & 1u) ? c : (uint32_t)P1 + (t & 31)], 1u);
       }
     }
@@ -670,7 +671,7 @@ __device__ __forceinline__ void fine_plan_body(const uint64_t* cstart, const uin
   __shared__ float zsum_s[32], zeros_s[32];
   __shared__ double target_s;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // HyperLogLog estimate over the 1/64 hash-sample of the keys
+  // HyperLogLog estimate over the 1/64 sample of the keys
   float z = 0.f, zeros = 0.f;
   for (int i = threadIdx.x; i < kHllRegs; i += blockDim.x) {
     const uint32_t r = hll[i];
@@ -747,22 +748,40 @@ __global__ void k_fine_plan_batch(BatchTab t) {
 }
 
 // ------------------------------------------------------------------ pass B
-// Per sub-step, NT threads x WPT windows: every key is computed once and kept in registers,
-// its rank inside its partition taken with a shared-memory atomic (counting sort, step 1);
-// after the block scan of the partition histogram the keys go to their partition's run in
-// the staging buffer, and the runs leave in order.  A 1/64 hash sample of the keys feeds a
-// HyperLogLog sketch (distinct-key estimate for sizing the fine partitions).
 __device__ __forceinline__ uint64_t key_hash(uint64_t key) { return key * 0x9E3779B97F4A7C15ull; }
 __device__ __forceinline__ uint64_t key_hash(u128 key) {
   return ((uint64_t)key ^ ((uint64_t)(key >> 64) * 0xC2B2AE3D27D4EB4Full)) * 0x9E3779B97F4A7C15ull;
 }
 
-// KEEP_C: each window's coarse partition is kept in shared memory (taken in phase 1,
-// carried to the staging and the write-out) instead of being recomputed from the key
-// twice; used when two blocks per SM still fit.
+// The distinct-key sketch: a HyperLogLog over a 1/64 sample of the keys, chosen by the sum of
+// the window's top forward and reverse-complement words (its first and its last 16 bases: the
+// words that its partition is found from, the same on either strand).  The first bases alone
+// would take or leave the variants of a repeat together: on the repeat genome that estimate
+// was 11% low.  A register is read before it is raised: after the first few thousand keys
+// hardly one still rises.
+__device__ __forceinline__ bool sketch_sampled(uint32_t f, uint32_t r) {
+  return ((f + r) * 0x9E3779B1u) >> (32 - kHllSampleLog2) == 0;
+}
+template <class K>
+__device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
+  const uint64_t h = key_hash(key);
+  const uint32_t reg = (uint32_t)(h >> (64 - kHllLog2));
+  const uint32_t v = (uint32_t)min(__clzll(h << kHllLog2) + 1, 64 - kHllLog2 + 1);
+  if (v > hll[reg]) atomicMax(&hll[reg], v);
+}
+
+// Per sub-step, NT threads x WPT windows.  A window's partition comes from the top 32 bits of
+// its canonical value alone, and its rank inside the partition from a shared-memory atomic (a
+// counting sort's first step); after the block scan of the partition histogram the whole keys
+// are computed, go to their partition's run in the staging buffer, and the runs leave in
+// order.  Bound by instruction issue and latency, not by HBM (19.2 GB written in 12.3 ms at 2.4 G
+// windows): no key is kept in registers across the scan (each is computed once, after it) and
+// a staged key's partition is found from the key again, so that three blocks fit an SM (80
+// registers, 73 KB).  With the keys held and the partitions kept in shared memory there were
+// two (128 registers) and it took 15.1 ms.
 // DIRECT (the aggregation ablation without per-block buckets): every valid window takes its
 // slot with a global atomic on its partition's cursor and is written on its own.
-template <int KW, int NT, bool KEEP_C, bool DIRECT = false>
+template <int KW, int NT, bool DIRECT = false>
 __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, uint32_t bid) {
   typedef typename KeyT<KW>::T K;
   constexpr int WPT = KW == 1 ? 32 : 16;    // windows per thread
@@ -773,14 +792,11 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   const int P1 = 1 << s.b1;
   K* stage = reinterpret_cast<K*>(sm);                                                // [SUB]
   unsigned long long* cursor = reinterpret_cast<unsigned long long*>(stage + SUB);   // [P1] absolute write positions
-  uint32_t* hist = reinterpret_cast<uint32_t*>(cursor + P1);                            // [padded P1]
-  uint32_t* soff = hist + padded_len(P1 + 32);                                          // [padded P1]
-  uint16_t* rawc = reinterpret_cast<uint16_t*>(soff + padded_len(P1 + 32));  // KEEP_C: [SUB], window i of thread t at i * NT + t
-  uint16_t* stage_c = rawc + SUB;                                        // KEEP_C: [SUB], partition of each staged key
+  uint32_t* hist = reinterpret_cast<uint32_t*>(cursor + P1);                            // [padded P1 + 32]
+  uint32_t* soff = hist + padded_len(P1 + 32);                                          // [padded P1 + 32]
   __shared__ uint64_t code_s[NW + 2];
   __shared__ uint32_t inv_s[NW + 2];
   __shared__ uint32_t st_s[NW + 2];
-  __shared__ uint32_t hll_s[kHllRegs];
   __shared__ uint64_t rcur_s;
   __shared__ uint32_t wt[32];
   const int t = threadIdx.x;
@@ -793,7 +809,6 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     cursor[c] = n ? atomicAdd(&b.fcur[c], (unsigned long long)n) : 0ull;
     hist[PAD(c)] = 0;
   }
-  for (int i = t; i < kHllRegs; i += NT) hll_s[i] = 0;
   if (t == 0) rcur_s = b.tile_first[tile];
   for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
@@ -814,79 +829,79 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     __syncthreads();
     build_starts(b.offsets, s.n_reads, j0, NW, st_s, &rcur_s);
     __syncthreads();
-    const uint64_t j = j0 + wl;
-    K keys[WPT];
-    uint32_t rr[WPT / 2];
-    uint32_t valid = 0;
+    const int sw = wl + 2;
+    const uint32_t vm = j0 + wl < s.n_words ? valid_mask(inv_s[sw - 2], inv_s[sw - 1], inv_s[sw], st_s[sw - 2],
+                                                         st_s[sw - 1], st_s[sw], s.k)
+                                            : 0u;
+    Win W;
+    win_setup<KW, WPT>(code_s[sw - 2], code_s[sw - 1], code_s[sw], vm, h, s.k, W);
+    const uint32_t valid = W.valid & (WPT == 32 ? 0xffffffffu : 0xffffu);
+    uint32_t cr[WPT];  // each window's partition and its rank there
+    // every window is ranked without a branch (so that the windows' dependency chains
+    // interleave): an invalid window is ranked in bin P1 + lane, which no scan reads (one such
+    // bin per lane, so that a warp's invalid windows do not share an address), and only the
+    // rare sketch update depends on the window being valid
 #pragma unroll
-    for (int i = 0; i < WPT / 2; ++i) rr[i] = 0;
-    if (j < s.n_words) {
-      Win W;
-      const int sw = wl + 2;
-      const uint32_t vm = valid_mask(inv_s[sw - 2], inv_s[sw - 1], inv_s[sw], st_s[sw - 2], st_s[sw - 1], st_s[sw], s.k);
-      win_setup<KW, WPT>(code_s[sw - 2], code_s[sw - 1], code_s[sw], vm, h, s.k, W);
-      valid = W.valid & (WPT == 32 ? 0xffffffffu : 0xffffu);
-      // every window is computed and ranked without a branch (so that the windows' dependency
-      // chains interleave): an invalid window is ranked in bin P1 + lane, which no scan reads
-      // (one such bin per lane, so that a warp's invalid windows do not share an address), and
-      // only the rare sketch update depends on the window being valid
-#pragma unroll
-      for (int i = 0; i < WPT; ++i) {
+    for (int i = 0; i < WPT; ++i) {
+      uint32_t f, r;
+      const uint32_t x = win_top32<KW, WPT>(W, i, s.canonical, f, r);
+      const uint32_t c = coarse_field(umap(x, s.canonical), s.b1);
+      const bool v = (valid >> i) & 1u;
+      if constexpr (DIRECT) {
+        if (v) {
+          uint64_t c0, c1;
+          K key;
+          win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+          top_to_key(c0, c1, s.k, key);
+          const unsigned long long pos = atomicAdd(&b.fcur[c], 1ull);
+          if (pos < s.cap) store_key(b.kbuf, pos, key);
+          else atomicOr(&b.meta->status, ST_INTERNAL);
+        }
+      } else {
+        const uint32_t cc = v ? c : (uint32_t)P1 + (t & 31);
+        cr[i] = (cc << 16) | atomicAdd(&hist[PAD(cc)], 1u);  // bin below 2^13, rank below 2^13
+      }
+      if (v && sketch_sampled(f, r)) {
         uint64_t c0, c1;
+        K key;
         win_top<KW, WPT>(W, i, s.canonical, c0, c1);
-        top_to_key(c0, c1, s.k, keys[i]);
-        const uint32_t c = coarse_field(umap((uint32_t)(c0 >> 32), s.canonical), s.b1);
-        const uint64_t hh = key_hash(keys[i]);
-        const bool v = (valid >> i) & 1u;
-        if constexpr (DIRECT) {
-          if (v) {
-            const unsigned long long pos = atomicAdd(&b.fcur[c], 1ull);
-            if (pos < s.cap) store_key(b.kbuf, pos, keys[i]);
-            else atomicOr(&b.meta->status, ST_INTERNAL);
-          }
-        } else {
-          if constexpr (KEEP_C) rawc[i * NT + t] = (uint16_t)c;
-          const uint32_t cc = v ? c : (uint32_t)P1 + (t & 31);
-          rr[i >> 1] |= (atomicAdd(&hist[PAD(cc)], 1u) & 0xffffu) << (16 * (i & 1));
-        }
-        if (v && (hh >> (64 - kHllSampleLog2)) == 0) {
-          const uint32_t reg = (uint32_t)(hh >> (64 - kHllSampleLog2 - kHllLog2)) & (kHllRegs - 1);
-          const uint64_t rest = hh << (kHllSampleLog2 + kHllLog2);
-          atomicMax(&hll_s[reg], (uint32_t)min(__clzll(rest) + 1, 64 - kHllSampleLog2 - kHllLog2 + 1));
-        }
+        top_to_key(c0, c1, s.k, key);
+        sketch_add(b.hll, key);
       }
     }
     if constexpr (DIRECT) continue;
     __syncthreads();
     for (int c = t; c < P1; c += NT) soff[PAD(c)] = hist[PAD(c)];
     __syncthreads();
-    block_exclusive_scan_pad<uint32_t>(soff, P1, wt);
+    const uint32_t n_sub = block_exclusive_scan_pad<uint32_t>(soff, P1, wt);
+    // during the write-out cursor[c] holds cursor[c] - soff[c]: staged position i of partition c
+    // goes to cursor[c] + i.  A run that would pass the end of the keys array (it cannot, if
+    // pass A saw the same reads) is recorded and the sub-step not written.
+    bool fits = true;
+    for (int c = t; c < P1; c += NT) {
+      fits = fits && cursor[c] + hist[PAD(c)] <= s.cap;
+      cursor[c] -= soff[PAD(c)];
+    }
 #pragma unroll
     for (int i = 0; i < WPT; ++i) {
       // an invalid window is staged at slot SUB - 1, which no valid window takes then (with
       // one window invalid, at most SUB - 1 are valid) and the write-out never reads
-      uint32_t c;
-      if constexpr (KEEP_C) c = rawc[i * NT + t];
-      else c = coarse_of(keys[i], s.k, s.canonical, s.b1);  // same field as above, from the key
-      const uint32_t pos = (valid & (1u << i)) ? soff[PAD(c)] + ((rr[i >> 1] >> (16 * (i & 1))) & 0xffffu)
-                                               : (uint32_t)(SUB - 1);
-      stage[pos] = keys[i];
-      if constexpr (KEEP_C) stage_c[pos] = (uint16_t)c;
+      uint64_t c0, c1;
+      K key;
+      win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+      top_to_key(c0, c1, s.k, key);
+      const uint32_t pos = (valid & (1u << i)) ? soff[PAD(cr[i] >> 16)] + (cr[i] & 0xffffu) : (uint32_t)(SUB - 1);
+      stage[pos] = key;
     }
-    __syncthreads();
-    const uint32_t n_sub = soff[PAD(P1 - 1)] + hist[PAD(P1 - 1)];
-    // during the write-out cursor[c] holds cursor[c] - soff[c]: staged position i of
-    // partition c goes to cursor[c] + i
-    for (int c = t; c < P1; c += NT) cursor[c] -= soff[PAD(c)];
-    __syncthreads();
-    for (uint32_t i = t; i < n_sub; i += NT) {
-      const K key = stage[i];
-      uint32_t c;
-      if constexpr (KEEP_C) c = stage_c[i];
-      else c = coarse_of(key, s.k, s.canonical, s.b1);  // runs are grouped by partition
-      const uint64_t pos = cursor[c] + i;
-      if (pos < s.cap) store_key(b.kbuf, pos, key);
-      else atomicOr(&b.meta->status, ST_INTERNAL);
+    fits = __syncthreads_and(fits);
+    if (fits) {
+      for (uint32_t i = t; i < n_sub; i += NT) {
+        const K key = stage[i];
+        const uint32_t c = coarse_of(key, s.k, s.canonical, s.b1);  // same field as above, from the key
+        store_key(b.kbuf, cursor[c] + i, key);
+      }
+    } else if (t == 0) {
+      atomicOr(&b.meta->status, ST_INTERNAL);
     }
     __syncthreads();
     for (int c = t; c < P1; c += NT) {
@@ -894,24 +909,21 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
       hist[PAD(c)] = 0;
     }
   }
-  __syncthreads();
-  for (int i = t; i < kHllRegs; i += NT)
-    if (hll_s[i]) atomicMax(&b.hll[i], hll_s[i]);
 }
-template <int KW, int NT, bool KEEP_C>
-__global__ void __launch_bounds__(NT, 2) k_scatter(Shape s, Buffers b) {
-  scatter_body<KW, NT, KEEP_C>(s, b, blockIdx.x);
+template <int KW, int NT>
+__global__ void __launch_bounds__(NT, 3) k_scatter(Shape s, Buffers b) {
+  scatter_body<KW, NT>(s, b, blockIdx.x);
 }
 // Aggregation ablation: pass B writes every key on its own through the partition cursors.
 template <int KW>
 __global__ void __launch_bounds__(256, 2) k_scatter_direct(Shape s, Buffers b) {
-  scatter_body<KW, 256, false, true>(s, b, blockIdx.x);
+  scatter_body<KW, 256, true>(s, b, blockIdx.x);
 }
 
-template <int KW, int NT, bool KEEP_C>
-__global__ void __launch_bounds__(NT, 2) k_scatter_batch(BatchTab t) {
+template <int KW, int NT>
+__global__ void __launch_bounds__(NT, 3) k_scatter_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  scatter_body<KW, NT, KEEP_C>(d.s, d.b, bid);
+  scatter_body<KW, NT>(d.s, d.b, bid);
 }
 
 // ------------------------------------------------------------------ phase 2: fine split
@@ -2255,10 +2267,10 @@ __global__ void __launch_bounds__(256) k_compact_batch(BatchTab t) {
 }
 
 // ------------------------------------------------------------------ launches
-constexpr size_t kScatterStaticSmem = 9216;  // pass B's static shared memory (batched form included), rounded up
-static size_t scatter_smem(int kw, int nt, int P1, bool keep_c) {
+constexpr size_t kScatterStaticSmem = 6144;  // pass B's static shared memory (batched form included), rounded up
+static size_t scatter_smem(int kw, int nt, int P1) {
   const size_t sub = (size_t)nt * (kw == 1 ? 32 : 16);
-  return sub * (size_t)(kw * 8) + (size_t)P1 * 8 + 2 * padded_len(P1 + 32) * 4 + (keep_c ? sub * 4 : 0);
+  return sub * (size_t)(kw * 8) + (size_t)P1 * 8 + 2 * padded_len(P1 + 32) * 4;
 }
 static size_t fine_hist_smem(int P1) { return (size_t)(P1 + 1) * 8 + kFineLocalCap * 4 + 16; }
 static size_t fine_scatter_smem(int kw, int P1) {
@@ -2280,10 +2292,8 @@ int configure_kernels(int device) {
   }
   KC_SET(k_pack_count<1>);
   KC_SET(k_pack_count<2>);
-  KC_SET((k_scatter<1, 256, false>));
-  KC_SET((k_scatter<2, 256, false>));
-  KC_SET((k_scatter<1, 256, true>));
-  KC_SET((k_scatter<2, 256, true>));
+  KC_SET((k_scatter<1, 256>));
+  KC_SET((k_scatter<2, 256>));
   KC_SET(k_scatter_direct<1>);
   KC_SET(k_scatter_direct<2>);
   KC_SET(k_fine_plan);
@@ -2298,10 +2308,8 @@ int configure_kernels(int device) {
   KC_SET(k_bucket_scan);
   KC_SET(k_pack_count_batch<1>);
   KC_SET(k_pack_count_batch<2>);
-  KC_SET((k_scatter_batch<1, 256, false>));
-  KC_SET((k_scatter_batch<2, 256, false>));
-  KC_SET((k_scatter_batch<1, 256, true>));
-  KC_SET((k_scatter_batch<2, 256, true>));
+  KC_SET((k_scatter_batch<1, 256>));
+  KC_SET((k_scatter_batch<2, 256>));
   KC_SET(k_fine_plan_batch);
   KC_SET(k_fine_hist_batch<1>);
   KC_SET(k_fine_hist_batch<2>);
@@ -2356,23 +2364,16 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
   ++launches;
   KC_STEP("k_bucket_scan");
   if (s.n_tiles > 0) {
-    const size_t smB = scatter_smem(s.kw, 256, P1, false), smK = scatter_smem(s.kw, 256, P1, true);
+    const size_t smB = scatter_smem(s.kw, 256, P1);
     if (smB + kScatterStaticSmem > s.smem_budget) return -(int)cudaErrorInvalidConfiguration;
-    // keep each window's coarse partition in shared memory if two blocks per SM still fit
-    int per_sm = 0;
-    if (s.kw == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter<1, 256, true>, 256, smK);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter<2, 256, true>, 256, smK);
-    const bool keep_c = per_sm >= 2;
     const unsigned gt = (unsigned)s.n_tiles;
     if (s.aggr & kAggrNoSmemBuckets) {
       if (s.kw == 1) k_scatter_direct<1><<<gt, 256, smB, st>>>(s, b);
       else k_scatter_direct<2><<<gt, 256, smB, st>>>(s, b);
     } else if (s.kw == 1) {
-      if (keep_c) k_scatter<1, 256, true><<<gt, 256, smK, st>>>(s, b);
-      else k_scatter<1, 256, false><<<gt, 256, smB, st>>>(s, b);
+      k_scatter<1, 256><<<gt, 256, smB, st>>>(s, b);
     } else {
-      if (keep_c) k_scatter<2, 256, true><<<gt, 256, smK, st>>>(s, b);
-      else k_scatter<2, 256, false><<<gt, 256, smB, st>>>(s, b);
+      k_scatter<2, 256><<<gt, 256, smB, st>>>(s, b);
     }
     ++launches;
     KC_STEP("k_scatter");
@@ -2472,19 +2473,11 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
              (k_bucket_scan_batch<<<bp.grid[BK_BUCKET_SCAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_BUCKET_SCAN))),
              "k_bucket_scan");
   if (bp.grid[BK_SCATTER]) {
-    const size_t smB = scatter_smem(bp.kw, 256, P1, false), smK = scatter_smem(bp.kw, 256, P1, true);
+    const size_t smB = scatter_smem(bp.kw, 256, P1);
     if (smB + kScatterStaticSmem > s0.smem_budget) return -(int)cudaErrorInvalidConfiguration;
-    int per_sm = 0;
-    if (bp.kw == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter_batch<1, 256, true>, 256, smK);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter_batch<2, 256, true>, 256, smK);
     const unsigned g = bp.grid[BK_SCATTER];
-    if (bp.kw == 1) {
-      if (per_sm >= 2) k_scatter_batch<1, 256, true><<<g, 256, smK, st>>>(tab(BK_SCATTER));
-      else k_scatter_batch<1, 256, false><<<g, 256, smB, st>>>(tab(BK_SCATTER));
-    } else {
-      if (per_sm >= 2) k_scatter_batch<2, 256, true><<<g, 256, smK, st>>>(tab(BK_SCATTER));
-      else k_scatter_batch<2, 256, false><<<g, 256, smB, st>>>(tab(BK_SCATTER));
-    }
+    if (bp.kw == 1) k_scatter_batch<1, 256><<<g, 256, smB, st>>>(tab(BK_SCATTER));
+    else k_scatter_batch<2, 256><<<g, 256, smB, st>>>(tab(BK_SCATTER));
     ++launches;
     KC_STEP("k_scatter");
   }
