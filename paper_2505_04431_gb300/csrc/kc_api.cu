@@ -95,6 +95,17 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   const uint64_t nf_bound = s.cap / s.fine_target + P1 + 1;
   const uint64_t nf_lim = P1 * kMaxFine;
   s.nf_max = nf_bound < nf_lim ? nf_bound : nf_lim;
+  // Inputs that would be a single coarse partition (12 Mi bases of 64-bit keys, 6 Mi of 128-bit
+  // keys) are partitioned once: pass A already knows the windows per bin and the sketch, so
+  // pass B can write the fine partitions, and the fine split's kernels and its pass over the
+  // keys fall away (10 M bases, k=31: 310 -> 219 us of kernels).  A plan that asks for a
+  // partition count or for one of the variants of the two-level path gets that; so do tables so
+  // small that there would be more fine partitions than pass B stages in shared memory.
+  s.one_level = L > 0 && b1 == 0 && !o.p_hint && !o.force_sampled && !(o.aggr & kAggrNoSmemBuckets) &&
+                s.nf_max <= kOneLevelFine;
+  // bins of at most 5/8 of a fine partition, even if every base starts a distinct key: a
+  // partition takes its target and up to a bin more, within the 3/4 load a table is ordered with
+  s.bb = std::min(kMaxBinsLog2, std::max(kMinBinsLog2, ceil_log2_u64(8 * s.cap / (5 * s.fine_target) + 1)));
   // a sampled fine layout: regions hold their estimate plus slack (about a fifth of the keys
   // in all, and at least 16 keys each); a layout that does not fit falls back to the exact one
   s.fine_sampled = o.allow_sampled && (o.force_sampled || L >= kFineSampledMinBases) ? 1 : 0;
@@ -119,7 +130,9 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.codes = take(s.n_words * 8);
   lay.inv = take(s.n_words * 4);
   lay.tf = take(s.n_tiles * 8);
-  lay.cst = take((P1 + 1) * 8);
+  const uint64_t bins = s.one_level ? 1ull << s.bb : 0;
+  lay.cst = take(std::max<uint64_t>((P1 + 1) * 8, bins * 4));
+  lay.bmap = take(bins * 2);
   lay.fb = take((P1 + 1) * 4);
   lay.fm = take(P1 * 4);
   lay.hll = take((size_t)kHllRegs * 4);
@@ -128,8 +141,9 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.flo = take((nf + 1) * 4);
   lay.fc = take(nf * 8);
   lay.look = take(nf * 8);
-  lay.kbuf = take(s.cap_kb * s.kw * 8);
-  const uint64_t hist_bytes = s.n_tiles * P1 * 4;  // pass A's histogram lies in sbuf's memory
+  // one-level: no coarse-grouped keys, only the counts of deferred runs
+  lay.kbuf = take(s.one_level ? s.cap * 4 : s.cap_kb * s.kw * 8);
+  const uint64_t hist_bytes = s.one_level ? 0 : s.n_tiles * P1 * 4;  // pass A's histogram lies in sbuf's memory
   lay.sbuf = take(std::max<uint64_t>(s.cap_kb * s.kw * 8, hist_bytes));
   lay.meta = take(sizeof(Meta));
   lay.total = at;
@@ -145,6 +159,8 @@ Buffers layout_buffers(const Layout& lay, uint8_t* ws) {
   b.tile_first = (uint64_t*)(ws + lay.tf);
   b.hist = (uint32_t*)(ws + lay.sbuf);
   b.cstart = (uint64_t*)(ws + lay.cst);
+  b.bins = (uint32_t*)(ws + lay.cst);
+  b.bmap = (uint16_t*)(ws + lay.bmap);
   b.fine_base = (uint32_t*)(ws + lay.fb);
   b.fine_m = (uint32_t*)(ws + lay.fm);
   b.hll = (uint32_t*)(ws + lay.hll);
@@ -159,16 +175,6 @@ Buffers layout_buffers(const Layout& lay, uint8_t* ws) {
   return b;
 }
 
-int clear_scratch(const Shape& s, const Buffers& b, void* stream) {
-  const cudaStream_t st = (cudaStream_t)stream;
-  const size_t P1 = (size_t)1 << s.b1;
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(b.meta, 0, sizeof(Meta), st)) != cudaSuccess) return (int)e;
-  if ((e = cudaMemsetAsync(b.fhist, 0, (size_t)s.nf_max * 4, st)) != cudaSuccess) return (int)e;
-  if ((e = cudaMemsetAsync(b.hll, 0, (size_t)kHllRegs * 4, st)) != cudaSuccess) return (int)e;
-  if ((e = cudaMemsetAsync(b.look, 0, (size_t)s.nf_max * 8, st)) != cudaSuccess) return (int)e;
-  return (int)cudaMemsetAsync(b.cstart, 0, (P1 + 1) * 8, st);
-}
 }  // namespace kc
 
 struct kc_plan_s {
@@ -387,10 +393,6 @@ bool enqueue_job(const Job& j, uint8_t* ws, cudaStream_t st, kc::Meta* meta_dst,
   const kc::Buffers b = make_buffers(j, ws);
   if (!enqueue_copies(j, b, st, err)) return false;
   cudaError_t e;
-  if ((e = (cudaError_t)kc::clear_scratch(s, b, (void*)st)) != cudaSuccess) {
-    *err = std::string("clearing scratch: ") + cudaGetErrorString(e);
-    return false;
-  }
   int l = kc::launch_phase1(s, b, n_sms, (void*)st, mark);
   if (l >= 0) {
     const int l2 = kc::launch_phase2(s, b, n_sms, j.nf_max, (void*)st, mark);

@@ -24,6 +24,11 @@ constexpr uint64_t kTilesWanted = 4864;        // 16 waves of pass B's 2 blocks 
 constexpr int kPackThreads = 256;              // pass A: one code word per thread per sub-step
 constexpr int kMaxCoarseLog2 = 12;             // at most 4096 coarse partitions
 constexpr int kMaxFine = 4096;                 // at most this many fine partitions per coarse one
+// One-level partitioning (inputs of a single coarse partition): pass A counts the windows of
+// 2^6 .. 2^13 bins, about 8 to a fine partition, and its last block groups the bins into at
+// most this many fine partitions, which pass B writes directly.
+constexpr uint64_t kOneLevelFine = 3072;
+constexpr int kMinBinsLog2 = 6, kMaxBinsLog2 = 13;
 // bases per coarse partition aimed at when the plan sets no partition count
 constexpr uint64_t coarse_bases(int kw) { return kw == 1 ? (12ull << 20) : (6ull << 20); }
 // count kernel: threads per block and blocks per SM (one block of 1024 threads with
@@ -71,6 +76,8 @@ struct Meta {
   uint32_t fine_spill;  // the sampled fine layout overflowed a region: the exact fine split ran
   uint64_t ticket;      // phase-2 work counter
   uint64_t d_estimate;  // distinct keys estimated by the sketch
+  uint32_t done;        // blocks of pass A that have finished
+  uint32_t pad_;
   uint64_t sub_cycles[8];    // profiled plans only: ordering sub-steps (range, rank, scan, place, small sorts, big sorts, #big)
   uint64_t phase_cycles[8];  // profiled plans only: SM cycles per phase of k_count_emit, summed over CTAs
 };
@@ -100,6 +107,8 @@ struct Shape {
   int defer_all;        // nonzero (testing): every fine partition takes the deferred write-out
   int withhold;         // nonzero (testing): partition 0 never publishes its prefix
   int aggr;             // aggregation variants: kAggr* bits (single-count path only)
+  int one_level;        // nonzero: pass B writes the fine partitions directly (b1 = 0)
+  int bb;               // one-level: log2 of the bins that are grouped into fine partitions
 };
 constexpr int kAggrNoSmemBuckets = 1;  // pass B writes every key on its own (global atomic cursor)
 constexpr int kAggrWarpMerge = 2;      // the count kernel adds a warp's equal keys with one atomic
@@ -125,6 +134,8 @@ struct Buffers {
   uint64_t* out_keys;
   uint32_t* out_counts;
   Meta* meta;
+  uint32_t* bins;         // one-level: [2^bb] windows per bin (in cstart's memory)
+  uint16_t* bmap;         // one-level: [2^bb] fine partition of each bin
 };
 
 // One count of a batch: its shape and its buffers (inside the batch's scratch arena).
@@ -156,8 +167,8 @@ struct BatchPlan {
   uint32_t grid[16] = {};
 };
 enum BatchKernel {
-  BK_CLEAR, BK_CHECK, BK_TILE_FIRST, BK_PACK, BK_BUCKET_SCAN, BK_SCATTER, BK_FINE_PLAN, BK_FINE_HIST,
-  BK_FINE_SCAN, BK_FINE_SCATTER, BK_COUNT, BK_SCAN_DISTINCT, BK_COMPACT, BK_N
+  BK_PREPARE, BK_PACK, BK_PACK_ONE, BK_SCATTER, BK_SCATTER_ONE, BK_FINE_PLAN, BK_FINE_HIST, BK_FINE_SCAN, BK_FINE_SCATTER, BK_COUNT, BK_SCAN_DISTINCT,
+  BK_COMPACT, BK_FINISH_ONE, BK_N
 };
 
 // Called after every kernel launch with the kernel's name (used for per-kernel timing).
@@ -198,7 +209,7 @@ struct ShapeOpts {
   int tight_slack = 0;     // testing: sampled regions get no slack
 };
 struct Layout {  // byte offsets into the count's scratch block
-  size_t reads, offs, codes, inv, tf, cst, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
+  size_t reads, offs, codes, inv, tf, cst, bmap, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
   size_t total;
 };
 // Fills s and lay for L bases and n_reads reads; copy_reads / copy_offs: the scratch holds a
@@ -208,8 +219,4 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
 // The scratch-held buffers at ws (reads, offsets and outputs are the caller's to set when
 // they are not copies).
 Buffers layout_buffers(const Layout& lay, uint8_t* ws);
-// Enqueue the clears every count starts from on `stream` (a cudaStream_t); returns a
-// cudaError_t.
-int clear_scratch(const Shape& s, const Buffers& b, void* stream);
-
 }  // namespace kc

@@ -42,6 +42,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "kc_internal.h"
 
 namespace kc {
@@ -230,60 +232,73 @@ __device__ T block_exclusive_scan_pad(T* data, int n, T* warp_tmp) {
   return total;
 }
 
-// ------------------------------------------------------------------ input checks
-// Batched launches: the arrays a count needs zeroed (status record, fine histogram,
-// look-back words, sketch, partition starts) are cleared by one kernel for all counts.
-__global__ void k_clear_batch(BatchTab t) {
-  KC_BATCH_PROLOGUE(t);
-  const Shape& s = d.s;
-  const Buffers& b = d.b;
+// The last block of a launch (of a count's blocks, in a batched launch) to get here returns
+// true, with every other block's writes visible to L2 reads; all threads call it.
+__device__ __forceinline__ bool last_block(uint32_t* done, uint32_t nblk) {
+  __shared__ uint32_t last_s;
+  __syncwarp();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_s = atomicAdd(done, 1u) == nblk - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  return last_s != 0;
+}
+
+// ------------------------------------------------------------------ prepare
+// What a count needs cleared (status record, fine histogram, look-back words, sketch,
+// partition counts), and the first read whose start is >= the halo start of each tile (lower
+// bound in offsets): one launch where there were five clears and a kernel.
+__device__ __forceinline__ void prepare_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
   const uint64_t i0 = (uint64_t)bid * blockDim.x + threadIdx.x, stride = (uint64_t)nblk * blockDim.x;
   for (uint64_t i = i0; i < s.nf_max; i += stride) {
     b.fhist[i] = 0;
     b.look[i] = 0;
   }
   for (uint64_t i = i0; i < (uint64_t)kHllRegs; i += stride) b.hll[i] = 0;
-  for (uint64_t i = i0; i <= (1ull << s.b1); i += stride) b.cstart[i] = 0;
+  if (s.one_level) {
+    for (uint64_t i = i0; i < (1ull << s.bb); i += stride) b.bins[i] = 0;
+  } else {
+    for (uint64_t i = i0; i <= (1ull << s.b1); i += stride) b.cstart[i] = 0;
+  }
   for (uint64_t i = i0; i < sizeof(Meta) / 4; i += stride) reinterpret_cast<uint32_t*>(b.meta)[i] = 0;
+  // a warp per tile, 32 offsets compared at a time: 4 round trips for 1 M reads, not 20
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint64_t t = i0 >> 5; t < s.n_tiles; t += stride >> 5) {
+    const uint64_t pos = t * s.tile_words * kWordBases;
+    const uint64_t halo = pos >= 64 ? pos - 64 : 0;
+    uint64_t lo = 0, hi = s.n_reads;
+    while (lo < hi) {
+      const uint64_t len = hi - lo, p = len <= 32 ? lo + lane : lo + len / 33 * (lane + 1);
+      const uint32_t below = __popc(__ballot_sync(0xffffffffu, p < hi && b.offsets[p] < halo));
+      const uint64_t step = len <= 32 ? 1 : len / 33;
+      const uint64_t first = len <= 32 ? lo : lo + step;  // lane 0's position
+      if (len <= 32) {
+        lo = hi = lo + below;
+      } else {
+        if (below < 32) hi = first + step * below;
+        if (below > 0) lo = first + step * (below - 1) + 1;
+      }
+    }
+    if (lane == 0) b.tile_first[t] = lo;
+  }
+}
+__global__ void __launch_bounds__(256) k_prepare(Shape s, Buffers b) { prepare_body(s, b, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(256) k_prepare_batch(BatchTab t) {
+  KC_BATCH_PROLOGUE(t);
+  prepare_body(d.s, d.b, bid, nblk);
 }
 
-__device__ __forceinline__ void check_offsets_body(const uint64_t* offsets, uint64_t n_reads, uint64_t L, Meta* meta,
-                                                   uint32_t bid, uint32_t nblk) {
-  for (uint64_t i = bid * (uint64_t)blockDim.x + threadIdx.x; i < n_reads; i += (uint64_t)nblk * blockDim.x) {
-    if (offsets[i + 1] < offsets[i]) atomicOr(&meta->status, ST_BAD_OFFSETS);
-  }
-  if (bid == 0 && threadIdx.x == 0 && (offsets[0] != 0 || offsets[n_reads] != L))
-    atomicOr(&meta->status, ST_BAD_OFFSETS);
-}
-__global__ void k_check_offsets(const uint64_t* offsets, uint64_t n_reads, uint64_t L, Meta* meta) {
-  check_offsets_body(offsets, n_reads, L, meta, blockIdx.x, gridDim.x);
-}
-__global__ void k_check_offsets_batch(BatchTab t) {
-  KC_BATCH_PROLOGUE(t);
-  check_offsets_body(d.b.offsets, d.s.n_reads, d.s.L, d.b.meta, bid, nblk);
-}
-
-// first read whose start is >= the halo start of each tile (lower bound in offsets)
-__device__ __forceinline__ void tile_first_body(const uint64_t* offsets, const Shape& s, uint64_t* tile_first,
-                                                uint32_t bid) {
-  const uint64_t t = bid * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t n_reads = s.n_reads;
-  if (t >= s.n_tiles) return;
-  const uint64_t pos = t * s.tile_words * kWordBases;
-  const uint64_t halo = pos >= 64 ? pos - 64 : 0;
-  uint64_t lo = 0, hi = n_reads;
-  while (lo < hi) {
-    const uint64_t mid = lo + (hi - lo) / 2;
-    if (offsets[mid] < halo) lo = mid + 1; else hi = mid;
-  }
-  tile_first[t] = lo;
-}
-__global__ void k_tile_first(const uint64_t* offsets, Shape s, uint64_t* tile_first) {
-  tile_first_body(offsets, s, tile_first, blockIdx.x);
-}
-__global__ void k_tile_first_batch(BatchTab t) {
-  KC_BATCH_PROLOGUE(t);
-  tile_first_body(d.b.offsets, d.s, d.b.tile_first, bid);
+// Offsets start at 0, do not decrease and end at L: a share for each block of the last kernel
+// (no kernel indexes memory by an unchecked offset: bad ones only make the counts meaningless).
+__device__ __forceinline__ void check_offsets(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+  bool bad = false;
+  for (uint64_t i = bid * (uint64_t)blockDim.x + threadIdx.x; i < s.n_reads; i += (uint64_t)nblk * blockDim.x)
+    bad |= b.offsets[i + 1] < b.offsets[i];
+  if (bid == 0 && threadIdx.x == 0) bad |= b.offsets[0] != 0 || b.offsets[s.n_reads] != s.L;
+  if (bad) atomicOr(&b.meta->status, ST_BAD_OFFSETS);
 }
 
 // ------------------------------------------------------------------ phase 1 helpers
@@ -548,25 +563,141 @@ __device__ __forceinline__ void top_to_key(uint64_t c0, uint64_t c1, int k, u128
   key = k >= 64 ? c : c >> (128 - 2 * k);
 }
 
+// ------------------------------------------------------------------ distinct-key sketch
+__device__ __forceinline__ uint64_t key_hash(uint64_t key) { return key * 0x9E3779B97F4A7C15ull; }
+__device__ __forceinline__ uint64_t key_hash(u128 key) {
+  return ((uint64_t)key ^ ((uint64_t)(key >> 64) * 0xC2B2AE3D27D4EB4Full)) * 0x9E3779B97F4A7C15ull;
+}
+
+// A HyperLogLog over a 1/64 sample of the keys, chosen by the sum of the window's top forward
+// and reverse-complement words (its first and its last 16 bases: the words that its partition
+// is found from, the same on either strand).  The first bases alone would take or leave the
+// variants of a repeat together: on the repeat genome that estimate was 11% low.  A register
+// is read before it is raised: after the first few thousand keys hardly one still rises.
+__device__ __forceinline__ bool sketch_sampled(uint32_t f, uint32_t r) {
+  return ((f + r) * 0x9E3779B1u) >> (32 - kHllSampleLog2) == 0;
+}
+template <class K>
+__device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
+  const uint64_t h = key_hash(key);
+  const uint32_t reg = (uint32_t)(h >> (64 - kHllLog2));
+  const uint32_t v = (uint32_t)min(__clzll(h << kHllLog2) + 1, 64 - kHllLog2 + 1);
+  if (v > hll[reg]) atomicMax(&hll[reg], v);
+}
+
+// The keys a fine partition aims at, from the sketch of a count of K windows: fine_target
+// distinct keys, i.e. fine_target * K / D keys.  All threads of the block call it.
+__device__ double sketch_target(const uint32_t* hll, uint64_t K, uint32_t fine_target, Meta* meta) {
+  __shared__ float zsum_s[32], zeros_s[32];
+  __shared__ double target_s;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // HyperLogLog estimate over the 1/64 sample of the keys (read from L2: written by every SM)
+  float z = 0.f, zeros = 0.f;
+  for (int i = threadIdx.x; i < kHllRegs; i += blockDim.x) {
+    const uint32_t r = __ldcg(&hll[i]);
+    z += exp2f(-(float)r);
+    zeros += r == 0 ? 1.f : 0.f;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    z += __shfl_xor_sync(0xffffffffu, z, d);
+    zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
+  }
+  if (lane == 0) {
+    zsum_s[wid] = z;
+    zeros_s[wid] = zeros;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double zs = 0, zr = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      zs += zsum_s[w];
+      zr += zeros_s[w];
+    }
+    const double m = kHllRegs;
+    double e = 0.7213 / (1.0 + 1.079 / m) * m * m / zs;
+    if (e < 2.5 * m && zr > 0) e = m * log(m / zr);
+    const double d_est = e * kHllSample;
+    double dup = d_est > 1.0 ? (double)K / d_est : 1.0;
+    dup = dup < 1.0 ? 1.0 : (dup > 32.0 ? 32.0 : dup);
+    target_s = (double)fine_target * (0.9 * dup > 1.0 ? 0.9 * dup : 1.0);
+    meta->d_estimate = (uint64_t)d_est;
+  }
+  __syncthreads();
+  return target_s;
+}
+
 // ------------------------------------------------------------------ pass A
-// One code word per thread: convert, store, and histogram the coarse partitions of its 32
-// windows (keys are recomputed in pass B, which needs the partition offsets first).
-template <int KW>
-__device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b, uint32_t bid) {
+// Partition starts (also pass B's cursors) from the partitions' totals (added up in cstart by
+// all blocks), and the total number of windows.  One block; sc: P1 words.
+__device__ __forceinline__ void bucket_scan(const Shape& s, const Buffers& b, uint64_t* sc) {
+  __shared__ uint64_t wt[32];
+  const int P1 = 1 << s.b1;
+  for (int c = threadIdx.x; c < P1; c += blockDim.x) {
+    const uint64_t n = __ldcg(&b.cstart[c]);
+    sc[c] = n;
+    if (n > 0xffffffffull) atomicOr(&b.meta->status, ST_PARTITION_OVERFLOW);  // pass B keeps 32-bit cursors
+  }
+  __syncthreads();
+  const uint64_t K = block_exclusive_scan<uint64_t>(sc, P1, wt);
+  for (int c = threadIdx.x; c < P1; c += blockDim.x) b.cstart[c] = b.fcur[c] = sc[c];
+  if (threadIdx.x == 0) {
+    b.cstart[P1] = K;
+    b.meta->n_windows = K;
+  }
+}
+
+// One-level partitioning: the bins, in order, are grouped into fine partitions of about T keys
+// (T from the sketch): a bin belongs to the partition in which its first key falls when every
+// partition takes T, so a partition takes T keys, give or take a bin.  Writes the bins' map and
+// the partitions' starts (also pass B's cursors) and first range-map values; a partition that
+// no bin starts in is left empty.  One block; sc: 2^bb words, padded.
+__device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b, uint32_t* sc) {
+  __shared__ uint32_t wt[32];
+  const int NB = 1 << s.bb;
+  for (int i = threadIdx.x; i < NB; i += blockDim.x) sc[PAD(i)] = __ldcg(&b.bins[i]);
+  __syncthreads();
+  const uint32_t K = block_exclusive_scan_pad<uint32_t>(sc, NB, wt);  // below 2^24
+  const double target = sketch_target(b.hll, K, s.fine_target, b.meta);
+  const uint32_t T = max((uint32_t)target, (uint32_t)(K / s.nf_max) + 1u);
+  const uint32_t NF = sc[PAD(NB - 1)] / T + 1;  // the last bin's partition is the last: at most K / T + 1 <= nf_max
+  for (int i = threadIdx.x; i < NB; i += blockDim.x) {
+    const uint32_t p = sc[PAD(i)];
+    const int g = (int)(p / T), prev = i ? (int)(sc[PAD(i - 1)] / T) : -1;
+    b.bmap[i] = (uint16_t)g;
+    for (int q = prev + 1; q <= g; ++q) {
+      b.foff[q] = p;
+      b.fcur[q] = p;
+      b.flo[q] = (uint32_t)i << (32 - s.bb);
+    }
+  }
+  if (threadIdx.x == 0) {
+    b.foff[NF] = K;
+    b.flo[NF] = 0;  // so that the last partition ends at u = 2^32 - 1
+    b.meta->n_windows = K;
+    b.meta->n_fine = NF;
+  }
+}
+
+// One code word per thread: convert, store, and histogram the partitions of its 32 windows
+// (keys are computed in pass B, which needs the partition offsets first).  The last block turns
+// the partitions' totals into their starts.
+// ONE: the windows of every bin instead, and the distinct-key sketch, from which the last
+// block plans the fine partitions.
+template <int KW, bool ONE>
+__device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint64_t tile, uint32_t* hist_s) {
   typedef typename KeyT<KW>::T K;
-  extern __shared__ uint32_t hist_s[];  // [P1 + 32]: bins P1 + lane take the invalid windows
   __shared__ uint64_t code_s[kPackThreads + 2];
   __shared__ uint32_t inv_s[kPackThreads + 2];
   __shared__ uint32_t st_s[kPackThreads + 2];
   __shared__ uint64_t rcur_s, len_s;
   const int t = threadIdx.x;
-  const int P1 = 1 << s.b1;
-  const uint64_t tile = bid;
-  for (int c = t; c < P1 + 32; c += kPackThreads) hist_s[c] = 0;
+  const int bits = ONE ? s.bb : s.b1;
+  const int P1 = 1 << bits;
   if (t == 0) {
     rcur_s = b.tile_first[tile];
     // bases read: never past the end the offsets give (a base count that disagrees with
-    // them is reported by k_check_offsets; the reads buffer is not overrun meanwhile)
+    // them is reported by the last kernel; the reads buffer is not overrun meanwhile)
     const uint64_t e = b.offsets[s.n_reads];
     len_s = e < s.L ? e : s.L;
   }
@@ -610,55 +741,55 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
 #pragma unroll
       for (int i = 0; i < 32; ++i) {  // an invalid window goes to bin P1 + lane, never read: no branch
         uint32_t f, r;
-        const uint32_t c = coarse_field(umap(win_top32<KW, 32>(W, i, s.canonical, f, r), s.canonical), s.b1);
-        atomicAdd(&hist_s[((W.valid >> i) & 1u) ? c : (uint32_t)P1 + (t & 31)], 1u);
+        const uint32_t c = coarse_field(umap(win_top32<KW, 32>(W, i, s.canonical, f, r), s.canonical), bits);
+        const bool v = (W.valid >> i) & 1u;
+        atomicAdd(&hist_s[v ? c : (uint32_t)P1 + (t & 31)], 1u);
+        if constexpr (ONE) {
+          if (v && sketch_sampled(f, r)) {
+            uint64_t c0, c1;
+            K key;
+            win_top<KW, 32>(W, i, s.canonical, c0, c1);
+            top_to_key(c0, c1, s.k, key);
+            sketch_add(b.hll, key);
+          }
+        }
       }
     }
   }
   __syncthreads();
-  // the tile's counts, and the partitions' totals (cstart holds them until k_bucket_scan)
-  for (int c = t; c < P1; c += kPackThreads) {
-    const uint32_t n = hist_s[c];
-    b.hist[tile * P1 + c] = n;
-    if (n) atomicAdd(reinterpret_cast<unsigned long long*>(&b.cstart[c]), (unsigned long long)n);
+}
+template <int KW, bool ONE>
+__device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+  extern __shared__ __align__(16) uint32_t hist_s[];  // [P1 + 32]: bins P1 + lane take the invalid windows
+  const int t = threadIdx.x, P1 = 1 << (ONE ? s.bb : s.b1);
+  if (bid < s.n_tiles) {  // (an empty input has one block and no tile)
+    for (int c = t; c < P1 + 32; c += kPackThreads) hist_s[c] = 0;
+    if constexpr (ONE) {  // several tiles, so that the bins are added up less often
+      for (uint64_t tile = bid; tile < s.n_tiles; tile += nblk) pack_tile<KW, true>(s, b, tile, hist_s);
+      for (int c = t; c < P1; c += kPackThreads)
+        if (hist_s[c]) atomicAdd(&b.bins[c], hist_s[c]);
+    } else {
+      pack_tile<KW, false>(s, b, bid, hist_s);
+      // the tile's counts, and the partitions' totals (cstart holds them until bucket_scan)
+      for (int c = t; c < P1; c += kPackThreads) {
+        const uint32_t n = hist_s[c];
+        b.hist[(uint64_t)bid * P1 + c] = n;
+        if (n) atomicAdd(reinterpret_cast<unsigned long long*>(&b.cstart[c]), (unsigned long long)n);
+      }
+    }
   }
+  if (!last_block(&b.meta->done, nblk)) return;
+  if constexpr (ONE) one_level_plan(s, b, hist_s);
+  else bucket_scan(s, b, reinterpret_cast<uint64_t*>(hist_s));
 }
-template <int KW>
+template <int KW, bool ONE>
 __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count(Shape s, Buffers b) {
-  pack_count_body<KW>(s, b, blockIdx.x);
+  pack_count_body<KW, ONE>(s, b, blockIdx.x, gridDim.x);
 }
-template <int KW>
+template <int KW, bool ONE>
 __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  pack_count_body<KW>(d.s, d.b, bid);
-}
-
-// ------------------------------------------------------------------ scans
-// Partition starts (also pass B's cursors) from the partitions' totals, and the total number
-// of windows.  One block.
-__device__ __forceinline__ void bucket_scan_body(const uint64_t* ccount, uint64_t* cstart, unsigned long long* cursor,
-                                                 int P1, Meta* meta) {
-  extern __shared__ uint64_t sc[];  // [P1]
-  __shared__ uint64_t wt[32];
-  for (int c = threadIdx.x; c < P1; c += blockDim.x) {
-    const uint64_t n = ccount[c];
-    sc[c] = n;
-    if (n > 0xffffffffull) atomicOr(&meta->status, ST_PARTITION_OVERFLOW);  // pass B keeps 32-bit cursors
-  }
-  __syncthreads();
-  const uint64_t K = block_exclusive_scan<uint64_t>(sc, P1, wt);
-  for (int c = threadIdx.x; c < P1; c += blockDim.x) cstart[c] = cursor[c] = sc[c];
-  if (threadIdx.x == 0) {
-    cstart[P1] = K;
-    meta->n_windows = K;
-  }
-}
-__global__ void k_bucket_scan(const uint64_t* ccount, uint64_t* cstart, unsigned long long* cursor, int P1, Meta* meta) {
-  bucket_scan_body(ccount, cstart, cursor, P1, meta);
-}
-__global__ void k_bucket_scan_batch(BatchTab t) {
-  KC_BATCH_PROLOGUE(t);
-  bucket_scan_body(d.b.cstart, d.b.cstart, d.b.fcur, 1 << d.s.b1, d.b.meta);
+  pack_count_body<KW, ONE>(d.s, d.b, bid, nblk);
 }
 
 // Fine split of every coarse partition, after pass B: the distinct-key estimate (a sampled
@@ -668,44 +799,7 @@ __device__ __forceinline__ void fine_plan_body(const uint64_t* cstart, const uin
                             uint32_t* flo, int P1, int b1, uint32_t fine_target, uint32_t nf_max, Meta* meta) {
   extern __shared__ uint64_t fsc[];  // [P1]
   __shared__ uint64_t wt[32];
-  __shared__ float zsum_s[32], zeros_s[32];
-  __shared__ double target_s;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // HyperLogLog estimate over the 1/64 sample of the keys
-  float z = 0.f, zeros = 0.f;
-  for (int i = threadIdx.x; i < kHllRegs; i += blockDim.x) {
-    const uint32_t r = hll[i];
-    z += exp2f(-(float)r);
-    zeros += r == 0 ? 1.f : 0.f;
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    z += __shfl_xor_sync(0xffffffffu, z, d);
-    zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
-  }
-  if (lane == 0) {
-    zsum_s[wid] = z;
-    zeros_s[wid] = zeros;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double zs = 0, zr = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      zs += zsum_s[w];
-      zr += zeros_s[w];
-    }
-    const double m = kHllRegs;
-    double e = 0.7213 / (1.0 + 1.079 / m) * m * m / zs;
-    if (e < 2.5 * m && zr > 0) e = m * log(m / zr);
-    const double d_est = e * kHllSample;
-    const double K = (double)cstart[P1];
-    double dup = d_est > 1.0 ? K / d_est : 1.0;
-    dup = dup < 1.0 ? 1.0 : (dup > 32.0 ? 32.0 : dup);
-    target_s = (double)fine_target * (0.9 * dup > 1.0 ? 0.9 * dup : 1.0);
-    meta->d_estimate = (uint64_t)d_est;
-  }
-  __syncthreads();
-  const double target = target_s;
+  const double target = sketch_target(hll, cstart[P1], fine_target, meta);
   for (int c = threadIdx.x; c < P1; c += blockDim.x) {
     const uint64_t n = cstart[c + 1] - cstart[c];
     uint64_t m = (uint64_t)ceil((double)n / target);
@@ -748,28 +842,6 @@ __global__ void k_fine_plan_batch(BatchTab t) {
 }
 
 // ------------------------------------------------------------------ pass B
-__device__ __forceinline__ uint64_t key_hash(uint64_t key) { return key * 0x9E3779B97F4A7C15ull; }
-__device__ __forceinline__ uint64_t key_hash(u128 key) {
-  return ((uint64_t)key ^ ((uint64_t)(key >> 64) * 0xC2B2AE3D27D4EB4Full)) * 0x9E3779B97F4A7C15ull;
-}
-
-// The distinct-key sketch: a HyperLogLog over a 1/64 sample of the keys, chosen by the sum of
-// the window's top forward and reverse-complement words (its first and its last 16 bases: the
-// words that its partition is found from, the same on either strand).  The first bases alone
-// would take or leave the variants of a repeat together: on the repeat genome that estimate
-// was 11% low.  A register is read before it is raised: after the first few thousand keys
-// hardly one still rises.
-__device__ __forceinline__ bool sketch_sampled(uint32_t f, uint32_t r) {
-  return ((f + r) * 0x9E3779B1u) >> (32 - kHllSampleLog2) == 0;
-}
-template <class K>
-__device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
-  const uint64_t h = key_hash(key);
-  const uint32_t reg = (uint32_t)(h >> (64 - kHllLog2));
-  const uint32_t v = (uint32_t)min(__clzll(h << kHllLog2) + 1, 64 - kHllLog2 + 1);
-  if (v > hll[reg]) atomicMax(&hll[reg], v);
-}
-
 // Per sub-step, NT threads x WPT windows.  A window's partition comes from the top 32 bits of
 // its canonical value alone, and its rank inside the partition from a shared-memory atomic (a
 // counting sort's first step); after the block scan of the partition histogram the whole keys
@@ -779,9 +851,12 @@ __device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
 // a staged key's partition is found from the key again, so that three blocks fit an SM (80
 // registers, 73 KB).  With the keys held and the partitions kept in shared memory there were
 // two (128 registers) and it took 15.1 ms.
-// DIRECT (the aggregation ablation without per-block buckets): every valid window takes its
+// SC_DIRECT (the aggregation ablation without per-block buckets): every valid window takes its
 // slot with a global atomic on its partition's cursor and is written on its own.
-template <int KW, int NT, bool DIRECT = false>
+// SC_ONE (one-level partitioning): the partitions are the fine ones, found through the bins'
+// map, a sub-step reserves its run in each with one atomic, and the keys go to sbuf.
+enum { SC_COARSE, SC_DIRECT, SC_ONE };
+template <int KW, int NT, int MODE = SC_COARSE>
 __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, uint32_t bid) {
   typedef typename KeyT<KW>::T K;
   constexpr int WPT = KW == 1 ? 32 : 16;    // windows per thread
@@ -789,11 +864,13 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   constexpr int NW = NT / TPW;              // code words per sub-step
   constexpr int SUB = NT * WPT;             // windows per sub-step
   extern __shared__ __align__(16) uint8_t sm[];
-  const int P1 = 1 << s.b1;
+  constexpr bool DIRECT = MODE == SC_DIRECT, ONE = MODE == SC_ONE;
+  const int P1 = ONE ? (int)min(b.meta->n_fine, s.nf_max) : 1 << s.b1, PM = ONE ? (int)s.nf_max : P1;
   K* stage = reinterpret_cast<K*>(sm);                                                // [SUB]
   unsigned long long* cursor = reinterpret_cast<unsigned long long*>(stage + SUB);   // [P1] absolute write positions
-  uint32_t* hist = reinterpret_cast<uint32_t*>(cursor + P1);                            // [padded P1 + 32]
-  uint32_t* soff = hist + padded_len(P1 + 32);                                          // [padded P1 + 32]
+  uint32_t* hist = reinterpret_cast<uint32_t*>(cursor + (ONE ? 0 : P1));                // [padded PM + 32]
+  uint32_t* soff = hist + padded_len(PM + 32);                                          // [padded PM + 32]
+  uint16_t* map = reinterpret_cast<uint16_t*>(soff + padded_len(PM + 32));              // ONE: [2^bb]
   __shared__ uint64_t code_s[NW + 2];
   __shared__ uint32_t inv_s[NW + 2];
   __shared__ uint32_t st_s[NW + 2];
@@ -805,10 +882,14 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   for (int c = t; c < P1; c += NT) {
     // the tile's run in partition c, reserved at once (the order of the tiles' runs inside a
     // partition does not matter to any later step)
-    const uint32_t n = DIRECT ? 0u : b.hist[tile * P1 + c];
-    cursor[c] = n ? atomicAdd(&b.fcur[c], (unsigned long long)n) : 0ull;
+    if constexpr (!ONE) {
+      const uint32_t n = DIRECT ? 0u : b.hist[tile * P1 + c];
+      cursor[c] = n ? atomicAdd(&b.fcur[c], (unsigned long long)n) : 0ull;
+    }
     hist[PAD(c)] = 0;
   }
+  if constexpr (ONE)
+    for (int i = t; i < (1 << s.bb); i += NT) map[i] = b.bmap[i];
   if (t == 0) rcur_s = b.tile_first[tile];
   for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
@@ -845,7 +926,8 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     for (int i = 0; i < WPT; ++i) {
       uint32_t f, r;
       const uint32_t x = win_top32<KW, WPT>(W, i, s.canonical, f, r);
-      const uint32_t c = coarse_field(umap(x, s.canonical), s.b1);
+      uint32_t c = coarse_field(umap(x, s.canonical), ONE ? s.bb : s.b1);
+      if constexpr (ONE) c = map[c];
       const bool v = (valid >> i) & 1u;
       if constexpr (DIRECT) {
         if (v) {
@@ -861,12 +943,14 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
         const uint32_t cc = v ? c : (uint32_t)P1 + (t & 31);
         cr[i] = (cc << 16) | atomicAdd(&hist[PAD(cc)], 1u);  // bin below 2^13, rank below 2^13
       }
-      if (v && sketch_sampled(f, r)) {
-        uint64_t c0, c1;
-        K key;
-        win_top<KW, WPT>(W, i, s.canonical, c0, c1);
-        top_to_key(c0, c1, s.k, key);
-        sketch_add(b.hll, key);
+      if constexpr (!ONE) {
+        if (v && sketch_sampled(f, r)) {
+          uint64_t c0, c1;
+          K key;
+          win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+          top_to_key(c0, c1, s.k, key);
+          sketch_add(b.hll, key);
+        }
       }
     }
     if constexpr (DIRECT) continue;
@@ -879,8 +963,17 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     // pass A saw the same reads) is recorded and the sub-step not written.
     bool fits = true;
     for (int c = t; c < P1; c += NT) {
-      fits = fits && cursor[c] + hist[PAD(c)] <= s.cap;
-      cursor[c] -= soff[PAD(c)];
+      if constexpr (ONE) {  // (positions are below 2^24; hist holds cursor - soff until it is cleared)
+        const uint32_t n = hist[PAD(c)];
+        if (n) {
+          const uint64_t lim = b.foff[c + 1], at = atomicAdd(&b.fcur[c], (unsigned long long)n);
+          fits = fits && at + n <= lim;
+          hist[PAD(c)] = (uint32_t)at - soff[PAD(c)];
+        }
+      } else {
+        fits = fits && cursor[c] + hist[PAD(c)] <= s.cap;
+        cursor[c] -= soff[PAD(c)];
+      }
     }
 #pragma unroll
     for (int i = 0; i < WPT; ++i) {
@@ -897,33 +990,34 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     if (fits) {
       for (uint32_t i = t; i < n_sub; i += NT) {
         const K key = stage[i];
-        const uint32_t c = coarse_of(key, s.k, s.canonical, s.b1);  // same field as above, from the key
-        store_key(b.kbuf, cursor[c] + i, key);
+        const uint32_t c = coarse_of(key, s.k, s.canonical, ONE ? s.bb : s.b1);  // same field as above, from the key
+        if constexpr (ONE) store_key(b.sbuf, (uint32_t)(hist[PAD(map[c])] + i), key);
+        else store_key(b.kbuf, cursor[c] + i, key);
       }
     } else if (t == 0) {
       atomicOr(&b.meta->status, ST_INTERNAL);
     }
     __syncthreads();
     for (int c = t; c < P1; c += NT) {
-      cursor[c] += soff[PAD(c)] + hist[PAD(c)];
+      if constexpr (!ONE) cursor[c] += soff[PAD(c)] + hist[PAD(c)];
       hist[PAD(c)] = 0;
     }
   }
 }
-template <int KW, int NT>
+template <int KW, int NT, int MODE>
 __global__ void __launch_bounds__(NT, 3) k_scatter(Shape s, Buffers b) {
-  scatter_body<KW, NT>(s, b, blockIdx.x);
+  scatter_body<KW, NT, MODE>(s, b, blockIdx.x);
 }
 // Aggregation ablation: pass B writes every key on its own through the partition cursors.
 template <int KW>
 __global__ void __launch_bounds__(256, 2) k_scatter_direct(Shape s, Buffers b) {
-  scatter_body<KW, 256, true>(s, b, blockIdx.x);
+  scatter_body<KW, 256, SC_DIRECT>(s, b, blockIdx.x);
 }
 
-template <int KW, int NT>
+template <int KW, int NT, int MODE>
 __global__ void __launch_bounds__(NT, 3) k_scatter_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  scatter_body<KW, NT>(d.s, d.b, bid);
+  scatter_body<KW, NT, MODE>(d.s, d.b, bid);
 }
 
 // ------------------------------------------------------------------ phase 2: fine split
@@ -2232,29 +2326,75 @@ __global__ void __launch_bounds__(1024) k_scan_distinct_batch(BatchTab t) {
 // Move the runs of the deferred fine partitions from their input regions (keys in sbuf,
 // counts in kbuf as 32-bit words) to their output positions: one block per partition.
 template <int KW>
-__device__ __forceinline__ void compact_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+__device__ __forceinline__ void move_run(const Shape& s, const Buffers& b, uint64_t src, uint64_t dst, uint32_t d) {
   typedef typename KeyT<KW>::T K;
-  const uint64_t n_def = min(b.meta->n_deferred, s.nf_max);
   const uint32_t* cnt_src = reinterpret_cast<const uint32_t*>(b.kbuf);
+  if (src > s.cap_kb || d > s.cap_kb - src || dst > s.cap || d > s.cap - dst) {
+    if (threadIdx.x == 0) atomicOr(&b.meta->status, ST_INTERNAL);
+    return;
+  }
+  for (uint32_t i = threadIdx.x; i < d; i += blockDim.x) {
+    K key;
+    load_key(b.sbuf, src + i, key);
+    store_key(b.out_keys, dst + i, key);
+    b.out_counts[dst + i] = cnt_src[src + i];
+  }
+}
+template <int KW>
+__device__ __forceinline__ void compact_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+  check_offsets(s, b, bid, nblk);
+  const uint64_t n_def = min(b.meta->n_deferred, s.nf_max);
   for (uint64_t q = bid; q < n_def; q += nblk) {
     const uint64_t g = b.look[q];
     if (g >= min(b.meta->n_fine, s.nf_max)) {
       if (threadIdx.x == 0) atomicOr(&b.meta->status, ST_INTERNAL);
       continue;
     }
-    const uint32_t d = b.fhist[g] & 0x7fffffffu;
-    const uint64_t src = b.foff[g], dst = b.fcur[g];
-    if (src + d > s.cap_kb || dst + d > s.cap) {
-      if (threadIdx.x == 0) atomicOr(&b.meta->status, ST_INTERNAL);
-      continue;
-    }
-    for (uint32_t i = threadIdx.x; i < d; i += blockDim.x) {
-      K key;
-      load_key(b.sbuf, src + i, key);
-      store_key(b.out_keys, dst + i, key);
-      b.out_counts[dst + i] = cnt_src[src + i];
-    }
+    move_run<KW>(s, b, b.foff[g], b.fcur[g], b.fhist[g] & 0x7fffffffu);
   }
+}
+// One-level counts: the scan of the distinct counts and the moving of deferred runs in one
+// launch.  There are at most kOneLevelFine partitions, so every block scans all of them for
+// itself; the first one also checks the look-back words and records the total.
+template <int KW>
+__device__ __forceinline__ void finish_one_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+  __shared__ uint32_t pre[kOneLevelFine + kOneLevelFine / 32 + 1];
+  __shared__ uint32_t wt[32];
+  check_offsets(s, b, bid, nblk);
+  const int NF = (int)min(b.meta->n_fine, min(s.nf_max, kOneLevelFine));
+  for (int g = threadIdx.x; g < NF; g += blockDim.x) pre[PAD(g)] = b.fhist[g] & 0x7fffffffu;
+  __syncthreads();
+  const uint32_t D = block_exclusive_scan_pad<uint32_t>(pre, NF, wt);  // below 2^24
+  if (bid == 0) {
+    bool bad = false;
+    uint32_t n_def = 0;
+    for (int g = threadIdx.x; g < NF; g += blockDim.x) {
+      // a direct partition published its inclusive prefix, a deferred one its count
+      const uint32_t v = b.fhist[g], d = v & 0x7fffffffu;
+      bad |= ld_status(&b.look[g]) != (v >> 31 ? (kLookAgg | d) : (kLookIncl | ((uint64_t)pre[PAD(g)] + d)));
+      n_def += v >> 31;
+    }
+    if (threadIdx.x == 0) wt[0] = 0;
+    __syncthreads();
+    if (n_def) atomicAdd(&wt[0], n_def);
+    __syncthreads();
+    bad |= wt[0] != b.meta->n_deferred;
+    if (bad) atomicOr(&b.meta->status, ST_INTERNAL);
+    if (threadIdx.x == 0) b.meta->n_distinct = D;
+  }
+  for (int g = bid; g < NF; g += nblk) {
+    const uint32_t v = b.fhist[g];
+    if (v >> 31) move_run<KW>(s, b, b.foff[g], pre[PAD(g)], v & 0x7fffffffu);
+  }
+}
+template <int KW>
+__global__ void __launch_bounds__(256) k_finish_one(Shape s, Buffers b) {
+  finish_one_body<KW>(s, b, blockIdx.x, gridDim.x);
+}
+template <int KW>
+__global__ void __launch_bounds__(256) k_finish_one_batch(BatchTab t) {
+  KC_BATCH_PROLOGUE(t);
+  finish_one_body<KW>(d.s, d.b, bid, nblk);
 }
 template <int KW>
 __global__ void __launch_bounds__(256) k_compact(Shape s, Buffers b) {
@@ -2268,9 +2408,30 @@ __global__ void __launch_bounds__(256) k_compact_batch(BatchTab t) {
 
 // ------------------------------------------------------------------ launches
 constexpr size_t kScatterStaticSmem = 6144;  // pass B's static shared memory (batched form included), rounded up
-static size_t scatter_smem(int kw, int nt, int P1) {
-  const size_t sub = (size_t)nt * (kw == 1 ? 32 : 16);
-  return sub * (size_t)(kw * 8) + (size_t)P1 * 8 + 2 * padded_len(P1 + 32) * 4;
+static size_t scatter_smem(const Shape& s, int nt) {
+  const size_t sub = (size_t)nt * (s.kw == 1 ? 32 : 16) * s.kw * 8;
+  if (s.one_level) return sub + 2 * padded_len(s.nf_max + 32) * 4 + ((size_t)2 << s.bb);
+  const size_t P1 = (size_t)1 << s.b1;
+  return sub + P1 * 8 + 2 * padded_len(P1 + 32) * 4;
+}
+// clears (a thread per fine partition) and first reads (a warp per tile)
+static uint32_t prepare_blocks(const Shape& s, uint64_t most) {
+  const uint64_t want = std::max<uint64_t>((s.nf_max + 255) / 256, (s.n_tiles + 7) / 8) + 4;
+  return (uint32_t)(want < most ? want : most);
+}
+// pass A: one block per tile (one-level: at most one wave, 4 blocks on 152 SMs)
+static uint32_t pack_blocks(const Shape& s) {
+  return (uint32_t)std::max<uint64_t>(1, s.one_level ? std::min<uint64_t>(s.n_tiles, 608) : s.n_tiles);
+}
+// the last kernel: deferred runs to move (at most one per fine partition), offsets to check
+static uint32_t compact_blocks(const Shape& s, int n_sms) {
+  const uint64_t want = std::max<uint64_t>(s.nf_max / 8, s.n_reads / 2048) + 1, most = (uint64_t)n_sms * 8;
+  return (uint32_t)(want < most ? want : most);
+}
+// pass A: the histogram, and the last block's scan of the partitions' totals
+static size_t pack_smem(const Shape& s) {
+  const size_t P1 = (size_t)1 << s.b1;
+  return s.one_level ? padded_len(((size_t)1 << s.bb) + 32) * 4 : (P1 + 16) * 8;
 }
 static size_t fine_hist_smem(int P1) { return (size_t)(P1 + 1) * 8 + kFineLocalCap * 4 + 16; }
 static size_t fine_scatter_smem(int kw, int P1) {
@@ -2290,10 +2451,14 @@ int configure_kernels(int device) {
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)) != cudaSuccess) \
       return (int)e;                                                                                        \
   }
-  KC_SET(k_pack_count<1>);
-  KC_SET(k_pack_count<2>);
-  KC_SET((k_scatter<1, 256>));
-  KC_SET((k_scatter<2, 256>));
+  KC_SET((k_pack_count<1, false>));
+  KC_SET((k_pack_count<1, true>));
+  KC_SET((k_pack_count<2, false>));
+  KC_SET((k_pack_count<2, true>));
+  KC_SET((k_scatter<1, 256, SC_COARSE>));
+  KC_SET((k_scatter<1, 256, SC_ONE>));
+  KC_SET((k_scatter<2, 256, SC_COARSE>));
+  KC_SET((k_scatter<2, 256, SC_ONE>));
   KC_SET(k_scatter_direct<1>);
   KC_SET(k_scatter_direct<2>);
   KC_SET(k_fine_plan);
@@ -2305,11 +2470,14 @@ int configure_kernels(int device) {
   KC_SET(k_count_emit<2>);
   KC_SET((k_count_emit<1, true>));
   KC_SET((k_count_emit<2, true>));
-  KC_SET(k_bucket_scan);
-  KC_SET(k_pack_count_batch<1>);
-  KC_SET(k_pack_count_batch<2>);
-  KC_SET((k_scatter_batch<1, 256>));
-  KC_SET((k_scatter_batch<2, 256>));
+  KC_SET((k_pack_count_batch<1, false>));
+  KC_SET((k_pack_count_batch<1, true>));
+  KC_SET((k_pack_count_batch<2, false>));
+  KC_SET((k_pack_count_batch<2, true>));
+  KC_SET((k_scatter_batch<1, 256, SC_COARSE>));
+  KC_SET((k_scatter_batch<1, 256, SC_ONE>));
+  KC_SET((k_scatter_batch<2, 256, SC_COARSE>));
+  KC_SET((k_scatter_batch<2, 256, SC_ONE>));
   KC_SET(k_fine_plan_batch);
   KC_SET(k_fine_hist_batch<1>);
   KC_SET(k_fine_hist_batch<2>);
@@ -2317,7 +2485,6 @@ int configure_kernels(int device) {
   KC_SET(k_fine_scatter_batch<2>);
   KC_SET(k_count_emit_batch<1>);
   KC_SET(k_count_emit_batch<2>);
-  KC_SET(k_bucket_scan_batch);
 #undef KC_SET
   return 0;
 }
@@ -2333,22 +2500,19 @@ int configure_kernels(int device) {
 
 int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, const Marker& mark) {
   cudaStream_t st = (cudaStream_t)stream;
-  const int P1 = 1 << s.b1;
   int launches = 0;
-  if (s.n_reads > 0) {
-    const uint64_t want = (s.n_reads + 255) / 256, lim = (uint64_t)n_sms * 8;
-    const unsigned g = (unsigned)(want < lim ? want : lim);
-    k_check_offsets<<<g, 256, 0, st>>>(b.offsets, s.n_reads, s.L, b.meta);
-    ++launches;
-    KC_STEP("k_check_offsets");
-  }
-  if (s.n_tiles == 0) return launches;
-  k_tile_first<<<(unsigned)((s.n_tiles + 127) / 128), 128, 0, st>>>(b.offsets, s, b.tile_first);
+  k_prepare<<<prepare_blocks(s, (uint64_t)n_sms * 8), 256, 0, st>>>(s, b);
   ++launches;
-  KC_STEP("k_tile_first");
-  const size_t smA = (size_t)(P1 + 32) * 4;
-  if (s.kw == 1) k_pack_count<1><<<(unsigned)s.n_tiles, kPackThreads, smA, st>>>(s, b);
-  else k_pack_count<2><<<(unsigned)s.n_tiles, kPackThreads, smA, st>>>(s, b);
+  KC_STEP("k_prepare");
+  const unsigned gt = pack_blocks(s);
+  const size_t smA = pack_smem(s);
+  if (s.kw == 1) {
+    if (s.one_level) k_pack_count<1, true><<<gt, kPackThreads, smA, st>>>(s, b);
+    else k_pack_count<1, false><<<gt, kPackThreads, smA, st>>>(s, b);
+  } else {
+    if (s.one_level) k_pack_count<2, true><<<gt, kPackThreads, smA, st>>>(s, b);
+    else k_pack_count<2, false><<<gt, kPackThreads, smA, st>>>(s, b);
+  }
   ++launches;
   KC_STEP("k_pack_count");
   return launches;
@@ -2358,50 +2522,49 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
   cudaStream_t st = (cudaStream_t)stream;
   const int P1 = 1 << s.b1;
   int launches = 0;
-  // partition starts (cstart holds the per-partition totals added up by pass A; the scan
-  // reads them into shared memory before overwriting)
-  k_bucket_scan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.cstart, b.fcur, P1, b.meta);
-  ++launches;
-  KC_STEP("k_bucket_scan");
   if (s.n_tiles > 0) {
-    const size_t smB = scatter_smem(s.kw, 256, P1);
+    const size_t smB = scatter_smem(s, 256);
     if (smB + kScatterStaticSmem > s.smem_budget) return -(int)cudaErrorInvalidConfiguration;
     const unsigned gt = (unsigned)s.n_tiles;
     if (s.aggr & kAggrNoSmemBuckets) {
       if (s.kw == 1) k_scatter_direct<1><<<gt, 256, smB, st>>>(s, b);
       else k_scatter_direct<2><<<gt, 256, smB, st>>>(s, b);
     } else if (s.kw == 1) {
-      k_scatter<1, 256><<<gt, 256, smB, st>>>(s, b);
+      if (s.one_level) k_scatter<1, 256, SC_ONE><<<gt, 256, smB, st>>>(s, b);
+      else k_scatter<1, 256, SC_COARSE><<<gt, 256, smB, st>>>(s, b);
     } else {
-      k_scatter<2, 256><<<gt, 256, smB, st>>>(s, b);
+      if (s.one_level) k_scatter<2, 256, SC_ONE><<<gt, 256, smB, st>>>(s, b);
+      else k_scatter<2, 256, SC_COARSE><<<gt, 256, smB, st>>>(s, b);
     }
     ++launches;
     KC_STEP("k_scatter");
   }
-  k_fine_plan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.hll, b.fine_base, b.fine_m, b.flo, P1, s.b1, s.fine_target, nf_max,
-                                               b.meta);
-  ++launches;
-  KC_STEP("k_fine_plan");
-  const unsigned gf = (unsigned)(n_sms * 2);
-  // the fine split (sampled layout or exact); after a sampled one, the exact split again,
-  // whose kernels return at once unless a sampled region overflowed
-  for (int redo = 0; redo <= (s.fine_sampled ? 1 : 0); ++redo) {
-    if (redo) {
-      k_fine_redo_clear<<<(unsigned)n_sms, 1024, 0, st>>>(s, b);
+  if (!s.one_level) {
+    k_fine_plan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.hll, b.fine_base, b.fine_m, b.flo, P1, s.b1, s.fine_target,
+                                                 nf_max, b.meta);
+    ++launches;
+    KC_STEP("k_fine_plan");
+    const unsigned gf = (unsigned)(n_sms * 2);
+    // the fine split (sampled layout or exact); after a sampled one, the exact split again,
+    // whose kernels return at once unless a sampled region overflowed
+    for (int redo = 0; redo <= (s.fine_sampled ? 1 : 0); ++redo) {
+      if (redo) {
+        k_fine_redo_clear<<<(unsigned)n_sms, 1024, 0, st>>>(s, b);
+        ++launches;
+        KC_STEP("k_fine_redo_clear");
+      }
+      if (s.kw == 1) k_fine_hist<1><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
+      else k_fine_hist<2><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
       ++launches;
-      KC_STEP("k_fine_redo_clear");
+      KC_STEP(redo ? "k_fine_hist_redo" : "k_fine_hist");
+      k_fine_scan<<<1, 1024, 0, st>>>(s, b, redo);
+      ++launches;
+      KC_STEP(redo ? "k_fine_scan_redo" : "k_fine_scan");
+      if (s.kw == 1) k_fine_scatter<1><<<gf, kFineThreads, fine_scatter_smem(1, P1), st>>>(s, b, redo);
+      else k_fine_scatter<2><<<gf, kFineThreads, fine_scatter_smem(2, P1), st>>>(s, b, redo);
+      ++launches;
+      KC_STEP(redo ? "k_fine_scatter_redo" : "k_fine_scatter");
     }
-    if (s.kw == 1) k_fine_hist<1><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
-    else k_fine_hist<2><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
-    ++launches;
-    KC_STEP(redo ? "k_fine_hist_redo" : "k_fine_hist");
-    k_fine_scan<<<1, 1024, 0, st>>>(s, b, redo);
-    ++launches;
-    KC_STEP(redo ? "k_fine_scan_redo" : "k_fine_scan");
-    if (s.kw == 1) k_fine_scatter<1><<<gf, kFineThreads, fine_scatter_smem(1, P1), st>>>(s, b, redo);
-    else k_fine_scatter<2><<<gf, kFineThreads, fine_scatter_smem(2, P1), st>>>(s, b, redo);
-    ++launches;
-    KC_STEP(redo ? "k_fine_scatter_redo" : "k_fine_scatter");
   }
   const size_t smC = count_kernel_smem(s.kw, s.bT_max, s.tail);
   if (s.aggr & kAggrWarpMerge) {
@@ -2414,11 +2577,18 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
   }
   ++launches;
   KC_STEP("k_count_emit");
+  if (s.one_level) {
+    if (s.kw == 1) k_finish_one<1><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
+    else k_finish_one<2><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
+    ++launches;
+    KC_STEP("k_finish_one");
+    return launches;
+  }
   k_scan_distinct<<<1, 1024, 0, st>>>(s, b);
   ++launches;
   KC_STEP("k_scan_distinct");
-  if (s.kw == 1) k_compact<1><<<(unsigned)(n_sms * 8), 256, 0, st>>>(s, b);
-  else k_compact<2><<<(unsigned)(n_sms * 8), 256, 0, st>>>(s, b);
+  if (s.kw == 1) k_compact<1><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
+  else k_compact<2><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
   ++launches;
   KC_STEP("k_compact");
   return launches;
@@ -2428,19 +2598,23 @@ uint32_t batch_blocks(BatchKernel k, const Shape& s, int n_sms, uint64_t bases_t
   auto clampu = [](uint64_t v, uint64_t lo, uint64_t hi) { return (uint32_t)(v < lo ? lo : (v > hi ? hi : v)); };
   const uint64_t nsm = (uint64_t)n_sms;
   switch (k) {
-    case BK_CLEAR: return clampu((s.nf_max + 2047) / 2048, 1, 32);
-    case BK_CHECK: return clampu((s.n_reads + 255) / 256, 1, 64);
-    case BK_TILE_FIRST: return (uint32_t)((s.n_tiles + 127) / 128);
-    case BK_PACK: return (uint32_t)s.n_tiles;
-    case BK_SCATTER: return (uint32_t)s.n_tiles;
+    case BK_PREPARE: return prepare_blocks(s, 64);
+    case BK_PACK: return s.one_level ? 0u : pack_blocks(s);
+    case BK_PACK_ONE: return s.one_level ? pack_blocks(s) : 0u;
+    case BK_SCATTER: return s.one_level ? 0u : (uint32_t)s.n_tiles;
+    case BK_SCATTER_ONE: return s.one_level ? (uint32_t)s.n_tiles : 0u;
+    case BK_FINE_PLAN:
+    case BK_FINE_SCAN: return s.one_level ? 0u : 1u;
     case BK_FINE_HIST:
-    case BK_FINE_SCATTER: return clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
+    case BK_FINE_SCATTER: return s.one_level ? 0u : clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
     case BK_COUNT: {
       const double share = bases_total ? (double)s.L / (double)bases_total : 1.0;
       return clampu((uint64_t)(2.0 * (double)nsm * share + 0.999), 1, nsm * kCountBlocksPerSM);
     }
-    case BK_COMPACT: return clampu(s.nf_max / 8, 1, 8 * nsm);
-    default: return 1u;  // one block per count: bucket scan, fine plan, fine scan, scan of distinct counts
+    case BK_SCAN_DISTINCT: return s.one_level ? 0u : 1u;
+    case BK_COMPACT: return s.one_level ? 0u : compact_blocks(s, n_sms);
+    case BK_FINISH_ONE: return s.one_level ? compact_blocks(s, n_sms) : 0u;
+    default: return 1u;
   }
 }
 
@@ -2458,28 +2632,39 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
     ++launches;                   \
     KC_STEP(name);                \
   }
-  KC_BLAUNCH(BK_CLEAR, (k_clear_batch<<<bp.grid[BK_CLEAR], 256, 0, st>>>(tab(BK_CLEAR))), "k_clear_batch");
-  KC_BLAUNCH(BK_CHECK, (k_check_offsets_batch<<<bp.grid[BK_CHECK], 256, 0, st>>>(tab(BK_CHECK))), "k_check_offsets");
-  KC_BLAUNCH(BK_TILE_FIRST, (k_tile_first_batch<<<bp.grid[BK_TILE_FIRST], 128, 0, st>>>(tab(BK_TILE_FIRST))),
-             "k_tile_first");
-  if (bp.kw == 1) {
-    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<1><<<bp.grid[BK_PACK], kPackThreads, (size_t)(P1 + 32) * 4, st>>>(tab(BK_PACK))),
-               "k_pack_count");
-  } else {
-    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<2><<<bp.grid[BK_PACK], kPackThreads, (size_t)(P1 + 32) * 4, st>>>(tab(BK_PACK))),
-               "k_pack_count");
+  // shared memory: the most that any count of the launch asks for
+  size_t smA[2] = {}, smB[2] = {};
+  for (int q = 0; q < bp.n; ++q) {
+    const Shape& s = bp.host[q].s;
+    smA[s.one_level != 0] = std::max(smA[s.one_level != 0], pack_smem(s));
+    smB[s.one_level != 0] = std::max(smB[s.one_level != 0], scatter_smem(s, 256));
   }
-  KC_BLAUNCH(BK_BUCKET_SCAN,
-             (k_bucket_scan_batch<<<bp.grid[BK_BUCKET_SCAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_BUCKET_SCAN))),
-             "k_bucket_scan");
-  if (bp.grid[BK_SCATTER]) {
-    const size_t smB = scatter_smem(bp.kw, 256, P1);
-    if (smB + kScatterStaticSmem > s0.smem_budget) return -(int)cudaErrorInvalidConfiguration;
-    const unsigned g = bp.grid[BK_SCATTER];
-    if (bp.kw == 1) k_scatter_batch<1, 256><<<g, 256, smB, st>>>(tab(BK_SCATTER));
-    else k_scatter_batch<2, 256><<<g, 256, smB, st>>>(tab(BK_SCATTER));
-    ++launches;
-    KC_STEP("k_scatter");
+  if (std::max(smB[0], smB[1]) + kScatterStaticSmem > s0.smem_budget) return -(int)cudaErrorInvalidConfiguration;
+  KC_BLAUNCH(BK_PREPARE, (k_prepare_batch<<<bp.grid[BK_PREPARE], 256, 0, st>>>(tab(BK_PREPARE))), "k_prepare");
+  if (bp.kw == 1) {
+    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<1, false><<<bp.grid[BK_PACK], kPackThreads, smA[0], st>>>(tab(BK_PACK))),
+               "k_pack_count");
+    KC_BLAUNCH(BK_PACK_ONE,
+               (k_pack_count_batch<1, true><<<bp.grid[BK_PACK_ONE], kPackThreads, smA[1], st>>>(tab(BK_PACK_ONE))),
+               "k_pack_count");
+    KC_BLAUNCH(BK_SCATTER,
+               (k_scatter_batch<1, 256, SC_COARSE><<<bp.grid[BK_SCATTER], 256, smB[0], st>>>(tab(BK_SCATTER))),
+               "k_scatter");
+    KC_BLAUNCH(BK_SCATTER_ONE,
+               (k_scatter_batch<1, 256, SC_ONE><<<bp.grid[BK_SCATTER_ONE], 256, smB[1], st>>>(tab(BK_SCATTER_ONE))),
+               "k_scatter");
+  } else {
+    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<2, false><<<bp.grid[BK_PACK], kPackThreads, smA[0], st>>>(tab(BK_PACK))),
+               "k_pack_count");
+    KC_BLAUNCH(BK_PACK_ONE,
+               (k_pack_count_batch<2, true><<<bp.grid[BK_PACK_ONE], kPackThreads, smA[1], st>>>(tab(BK_PACK_ONE))),
+               "k_pack_count");
+    KC_BLAUNCH(BK_SCATTER,
+               (k_scatter_batch<2, 256, SC_COARSE><<<bp.grid[BK_SCATTER], 256, smB[0], st>>>(tab(BK_SCATTER))),
+               "k_scatter");
+    KC_BLAUNCH(BK_SCATTER_ONE,
+               (k_scatter_batch<2, 256, SC_ONE><<<bp.grid[BK_SCATTER_ONE], 256, smB[1], st>>>(tab(BK_SCATTER_ONE))),
+               "k_scatter");
   }
   KC_BLAUNCH(BK_FINE_PLAN, (k_fine_plan_batch<<<bp.grid[BK_FINE_PLAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_FINE_PLAN))),
              "k_fine_plan");
@@ -2527,8 +2712,12 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
              "k_scan_distinct");
   if (bp.kw == 1) {
     KC_BLAUNCH(BK_COMPACT, (k_compact_batch<1><<<bp.grid[BK_COMPACT], 256, 0, st>>>(tab(BK_COMPACT))), "k_compact");
+    KC_BLAUNCH(BK_FINISH_ONE, (k_finish_one_batch<1><<<bp.grid[BK_FINISH_ONE], 256, 0, st>>>(tab(BK_FINISH_ONE))),
+               "k_finish_one");
   } else {
     KC_BLAUNCH(BK_COMPACT, (k_compact_batch<2><<<bp.grid[BK_COMPACT], 256, 0, st>>>(tab(BK_COMPACT))), "k_compact");
+    KC_BLAUNCH(BK_FINISH_ONE, (k_finish_one_batch<2><<<bp.grid[BK_FINISH_ONE], 256, 0, st>>>(tab(BK_FINISH_ONE))),
+               "k_finish_one");
   }
 #undef KC_BLAUNCH
   return launches;

@@ -137,9 +137,6 @@ extern "C" kc_status kc_count_noalloc(const uint8_t* reads, const uint64_t* offs
   b.out_keys = out_keys;
   b.out_counts = out_counts;
 
-  // the array keeps the previous call's contents: clear what the kernels expect at zero
-  if ((e = (cudaError_t)kc::clear_scratch(s, b, (void*)strm)) != cudaSuccess)
-    return nfail(KC_ECUDA, std::string("kc_count_noalloc: clearing scratch: ") + cudaGetErrorString(e));
   kc::Marker none;
   int launches = kc::launch_phase1(s, b, ds->n_sms, (void*)strm, none);
   if (launches >= 0) {

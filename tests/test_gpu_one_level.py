@@ -1,0 +1,71 @@
+"""Inputs of a single coarse partition are partitioned once (pass A plans the fine partitions,
+pass B writes them).  The result is compared with the oracle and with the general two-level
+path, which a plan that asks for a partition count takes."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def counters(torch_cuda):
+    from paper_2505_04431_gb300 import KmerCounter
+    made = {name: KmerCounter(**kw) for name, kw in (
+        ("one", {}), ("two", {"n_partitions_hint": 1}), ("one deferred", {"defer_all": True}),
+        ("one, small tables", {"table_slots_max": 1024}))}
+    yield made
+    for c in made.values():
+        c.close()
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    return torch
+
+
+def check(torch, counters, reads, offsets, k, canonical):
+    want_k, want_c, want_n = oracle.count(reads, offsets, k, canonical)
+    r = torch.from_numpy(reads).cuda()
+    o = torch.from_numpy(offsets.view(np.int64)).cuda()
+    for name, c in counters.items():
+        res = c.count(r, o, k, canonical)
+        keys, counts = res.to_numpy()
+        n = res.n_valid_windows
+        res.free()
+        assert n == want_n and np.array_equal(keys, want_k) and np.array_equal(counts, want_c), name
+        assert (c.stats()["kernel_launches"] == 5) == (name != "two"), name
+
+
+# one read start to a few tiles of 8192 bases, with the lengths around a tile's edge
+@pytest.mark.parametrize("bases", [1, 64, 8191, 8192, 8193, 16383, 70_001, 400_000])
+@pytest.mark.parametrize("k,canonical", [(5, True), (21, False), (31, True), (32, True), (33, False), (63, True)])
+def test_one_level_sizes(torch_cuda, counters, bases, k, canonical):
+    rng = np.random.default_rng(bases * 100 + k)
+    reads, offsets = synth.random_reads(rng, max(1, bases // 100), 200)
+    reads, offsets = reads[:bases], np.minimum(offsets, bases).astype(np.uint64)
+    offsets[-1] = len(reads)
+    check(torch_cuda, counters, reads, offsets, k, canonical)
+
+
+@pytest.mark.parametrize("k", [31, 63])
+def test_one_level_uneven_bins(torch_cuda, counters, k):
+    # 14 000 distinct keys under one 15-base prefix (one bin, larger than any table), a last
+    # bin that holds many keys, and ordinary reads around them
+    rng = np.random.default_rng(k)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    n = 14_000
+    clump = acgt[rng.integers(0, 4, (n, k))]
+    clump[:, :15] = ord("A")
+    last = acgt[rng.integers(0, 4, (3000, k))]
+    last[:, :16] = ord("T")
+    rest = acgt[rng.integers(0, 4, (500, k))]
+    reads = np.ascontiguousarray(np.concatenate([rest, clump, last, rest])).reshape(-1)
+    offsets = np.arange(0, len(reads) + 1, k, dtype=np.uint64)
+    check(torch_cuda, counters, reads, offsets, k, False)
+    assert counters["one"].stats()["n_overflow_fine"] > 0
