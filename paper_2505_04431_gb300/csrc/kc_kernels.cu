@@ -302,24 +302,37 @@ __device__ __forceinline__ void check_offsets(const Shape& s, const Buffers& b, 
 }
 
 // ------------------------------------------------------------------ phase 1 helpers
-// ASCII -> codes for 32 bytes given as 8 little-endian words.
+// ASCII -> codes for 32 bytes given as 8 little-endian words.  The 2-bit codes of a word's four
+// bytes are gathered by one multiplication (their products fall on bits of their own), and a
+// byte is a base iff it is, in lower case, the letter of its code (looked up for four bytes by
+// one byte permutation): a third of the instructions of comparing each byte with each letter.
+// The bytes that are not are picked out only in words that have one.
 __device__ __forceinline__ void pack32(const uint32_t w[8], uint64_t& code, uint32_t& inv) {
-  uint64_t c = 0;
-  uint32_t v = 0;
+  uint32_t p[8], any = 0;
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const uint32_t x = w[m];
-    const uint32_t c4 = ((x >> 1) ^ (x >> 2)) & 0x03030303u;  // A0 C1 G2 T3 (either case)
-    const uint32_t g = ((c4 << 6) & 0xC0u) | ((c4 >> 4) & 0x30u) | ((c4 >> 14) & 0x0Cu) | ((c4 >> 24) & 0x03u);
-    c |= (uint64_t)g << (56 - 8 * m);
-    const uint32_t lc = x | 0x20202020u;
-    const uint32_t ok = __vcmpeq4(lc, 0x61616161u) | __vcmpeq4(lc, 0x63636363u) | __vcmpeq4(lc, 0x67676767u) |
-                        __vcmpeq4(lc, 0x74747474u);
-    const uint32_t bad = ~ok & 0x80808080u;
-    v |= (((bad >> 7) & 1u) | ((bad >> 14) & 2u) | ((bad >> 21) & 4u) | ((bad >> 28) & 8u)) << (4 * m);
+    const uint32_t c4 = ((x >> 1) ^ (x >> 2)) & 0x03030303u;  // A0 C1 G2 T3 (either case), one per byte
+    p[m] = c4 * 0x40100401u;                                   // the four codes in the top byte, first base on top
+    const uint32_t n4 = c4 | (c4 >> 4);                        // two selectors in bytes 0 and 2
+    const uint32_t letters = __byte_perm(0x74676361u, 0, __byte_perm(n4, 0, 0x4420));  // "acgt"
+    any |= letters ^ (x | 0x20202020u);
   }
-  code = c;
-  inv = v;
+  const uint32_t hi = __byte_perm(__byte_perm(p[3], p[2], 0x0073), __byte_perm(p[1], p[0], 0x0073), 0x5410);
+  const uint32_t lo = __byte_perm(__byte_perm(p[7], p[6], 0x0073), __byte_perm(p[5], p[4], 0x0073), 0x5410);
+  code = ((uint64_t)hi << 32) | lo;
+  inv = 0;
+  if (any) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const uint32_t x = w[m];
+      const uint32_t c4 = ((x >> 1) ^ (x >> 2)) & 0x03030303u;
+      const uint32_t n4 = c4 | (c4 >> 4);
+      const uint32_t d = __byte_perm(0x74676361u, 0, __byte_perm(n4, 0, 0x4420)) ^ (x | 0x20202020u);
+      const uint32_t bad = (((d & 0x7f7f7f7fu) + 0x7f7f7f7fu) | d) & 0x80808080u;  // top bit of each nonzero byte
+      inv |= (((bad >> 7) & 1u) | ((bad >> 14) & 2u) | ((bad >> 21) & 4u) | ((bad >> 28) & 8u)) << (4 * m);
+    }
+  }
 }
 
 // Convert code word w (bases 32w .. 32w+31) straight from the reads.
@@ -371,6 +384,10 @@ __device__ void build_starts(const uint64_t* offsets, uint64_t n_reads, uint64_t
   if (t == 0) *rcur_s += adv;
 }
 
+// Variants of the phase-1 kernels: canonical keys and forward keys of k >= 16, whose top 32
+// bits need no mask, and any k < 16.
+enum { V_SHORT, V_CANON, V_FORWARD };
+
 // The range map: coarse partition, fine partition are bit fields of a 32-bit value u,
 // non-decreasing in the key.  x = top 32 bits of the 2k-bit key; canonical keys are the
 // min of two near-independent uniforms (density 2(1-x)), so u = 1 - (1-x)^2 (its
@@ -386,6 +403,12 @@ __device__ __forceinline__ uint32_t umap(uint32_t x, int canonical) {
 __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t s) { return __funnelshift_rc(x, 0u, s); }
 // the coarse field of u: its top b1 bits (none for b1 = 0)
 __device__ __forceinline__ uint32_t coarse_field(uint32_t u, int b1) { return shr_clamp(u, 32 - b1); }
+// The same field counted from its far end (2^b1 - 1 - field), one instruction cheaper: the
+// order of the partitions inside one block's shared arrays.
+__device__ __forceinline__ uint32_t coarse_field_rev(uint32_t x, int canonical, int b1) {
+  const uint32_t y = ~x;
+  return shr_clamp(canonical ? __umulhi(y, y) : y, 32 - b1);
+}
 template <class K>
 __device__ __forceinline__ uint32_t coarse_of(K key, int k, int canonical, int b1) {
   return coarse_field(umap(top32_of(key, k), canonical), b1);
@@ -548,9 +571,9 @@ __device__ __forceinline__ uint32_t top32_shl(uint64_t a, uint64_t b, int sh) {
 // shifts.  The smaller of the forward and reverse-complement top words is the canonical
 // value's top word: where the top words differ they decide which value is smaller, and
 // where they tie both values share them.
-template <int KW, int WPT>
+template <int KW, int WPT, int VAR>
 __device__ __forceinline__ uint32_t win_top32(const Win& W, int i, int canonical, uint32_t& f, uint32_t& r) {
-  const uint32_t m = (uint32_t)(W.m0 >> 32);
+  const uint32_t m = VAR == V_SHORT ? (uint32_t)(W.m0 >> 32) : ~0u;
   f = top32_shl(W.s0, W.s1, 2 * i) & m;
   r = top32_shl(W.r0, W.r1, 2 * (WPT - 1 - i)) & m;
   return canonical ? min(f, r) : f;
@@ -628,6 +651,10 @@ __device__ double sketch_target(const uint32_t* hll, uint64_t K, uint32_t fine_t
 }
 
 // ------------------------------------------------------------------ pass A
+// Add 1 to the shared word at address a if p is not 0.
+__device__ __forceinline__ void red_shared_if(uint32_t a, uint32_t p) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t@q red.shared.add.u32 [%0], 1;\n\t}" ::"r"(a), "r"(p) : "memory");
+}
 // Partition starts (also pass B's cursors) from the partitions' totals (added up in cstart by
 // all blocks), and the total number of windows.  One block; sc: P1 words.
 __device__ __forceinline__ void bucket_scan(const Shape& s, const Buffers& b, uint64_t* sc) {
@@ -681,10 +708,14 @@ __device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b,
 
 // One code word per thread: convert, store, and histogram the partitions of its 32 windows
 // (keys are computed in pass B, which needs the partition offsets first).  The last block turns
-// the partitions' totals into their starts.
+// the partitions' totals into their starts.  Bound by the ALU (86% busy at 2.4 G windows): a
+// window takes two funnel shifts, a minimum, the range map and one predicated reduction, with
+// no masks (variants by k and mode) and no select for invalid windows, and a word's bytes are
+// converted by multiplications and byte permutations; 2.95 ms, where masks, selects and
+// byte-by-byte comparisons took 4.44.
 // ONE: the windows of every bin instead, and the distinct-key sketch, from which the last
 // block plans the fine partitions.
-template <int KW, bool ONE>
+template <int KW, bool ONE, int VAR>
 __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint64_t tile, uint32_t* hist_s) {
   typedef typename KeyT<KW>::T K;
   __shared__ uint64_t code_s[kPackThreads + 2];
@@ -693,7 +724,8 @@ __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint
   __shared__ uint64_t rcur_s, len_s;
   const int t = threadIdx.x;
   const int bits = ONE ? s.bb : s.b1;
-  const int P1 = 1 << bits;
+  const int canonical = VAR == V_SHORT ? s.canonical : VAR == V_CANON;
+  const uint32_t hist_a = (uint32_t)__cvta_generic_to_shared(hist_s);
   if (t == 0) {
     rcur_s = b.tile_first[tile];
     // bases read: never past the end the offsets give (a base count that disagrees with
@@ -739,16 +771,16 @@ __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint
       const uint32_t vm = valid_mask(inv_s[t], inv_s[t + 1], inv, st_s[t], st_s[t + 1], st_s[t + 2], s.k);
       win_setup<KW, 32>(code_s[t], code_s[t + 1], code, vm, 0, s.k, W);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {  // an invalid window goes to bin P1 + lane, never read: no branch
+      for (int i = 0; i < 32; ++i) {
         uint32_t f, r;
-        const uint32_t c = coarse_field(umap(win_top32<KW, 32>(W, i, s.canonical, f, r), s.canonical), bits);
-        const bool v = (W.valid >> i) & 1u;
-        atomicAdd(&hist_s[v ? c : (uint32_t)P1 + (t & 31)], 1u);
+        const uint32_t c = coarse_field_rev(win_top32<KW, 32, VAR>(W, i, canonical, f, r), canonical, bits);
+        const uint32_t v = W.valid & (1u << i);
+        red_shared_if(hist_a + 4 * c, v);  // predicated: no branch, no bin for the invalid windows
         if constexpr (ONE) {
           if (v && sketch_sampled(f, r)) {
             uint64_t c0, c1;
             K key;
-            win_top<KW, 32>(W, i, s.canonical, c0, c1);
+            win_top<KW, 32>(W, i, canonical, c0, c1);
             top_to_key(c0, c1, s.k, key);
             sketch_add(b.hll, key);
           }
@@ -758,21 +790,21 @@ __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint
   }
   __syncthreads();
 }
-template <int KW, bool ONE>
+template <int KW, bool ONE, int VAR>
 __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
-  extern __shared__ __align__(16) uint32_t hist_s[];  // [P1 + 32]: bins P1 + lane take the invalid windows
+  extern __shared__ __align__(16) uint32_t hist_s[];  // [P1], partitions from the last to the first
   const int t = threadIdx.x, P1 = 1 << (ONE ? s.bb : s.b1);
   if (bid < s.n_tiles) {  // (an empty input has one block and no tile)
-    for (int c = t; c < P1 + 32; c += kPackThreads) hist_s[c] = 0;
+    for (int c = t; c < P1; c += kPackThreads) hist_s[c] = 0;
     if constexpr (ONE) {  // several tiles, so that the bins are added up less often
-      for (uint64_t tile = bid; tile < s.n_tiles; tile += nblk) pack_tile<KW, true>(s, b, tile, hist_s);
+      for (uint64_t tile = bid; tile < s.n_tiles; tile += nblk) pack_tile<KW, true, VAR>(s, b, tile, hist_s);
       for (int c = t; c < P1; c += kPackThreads)
-        if (hist_s[c]) atomicAdd(&b.bins[c], hist_s[c]);
+        if (hist_s[c]) atomicAdd(&b.bins[P1 - 1 - c], hist_s[c]);
     } else {
-      pack_tile<KW, false>(s, b, bid, hist_s);
+      pack_tile<KW, false, VAR>(s, b, bid, hist_s);
       // the tile's counts, and the partitions' totals (cstart holds them until bucket_scan)
       for (int c = t; c < P1; c += kPackThreads) {
-        const uint32_t n = hist_s[c];
+        const uint32_t n = hist_s[P1 - 1 - c];
         b.hist[(uint64_t)bid * P1 + c] = n;
         if (n) atomicAdd(reinterpret_cast<unsigned long long*>(&b.cstart[c]), (unsigned long long)n);
       }
@@ -782,14 +814,14 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
   if constexpr (ONE) one_level_plan(s, b, hist_s);
   else bucket_scan(s, b, reinterpret_cast<uint64_t*>(hist_s));
 }
-template <int KW, bool ONE>
+template <int KW, bool ONE, int VAR>
 __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count(Shape s, Buffers b) {
-  pack_count_body<KW, ONE>(s, b, blockIdx.x, gridDim.x);
+  pack_count_body<KW, ONE, VAR>(s, b, blockIdx.x, gridDim.x);
 }
-template <int KW, bool ONE>
+template <int KW, bool ONE, int VAR>
 __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  pack_count_body<KW, ONE>(d.s, d.b, bid, nblk);
+  pack_count_body<KW, ONE, VAR>(d.s, d.b, bid, nblk);
 }
 
 // Fine split of every coarse partition, after pass B: the distinct-key estimate (a sampled
@@ -846,7 +878,7 @@ __global__ void k_fine_plan_batch(BatchTab t) {
 // its canonical value alone, and its rank inside the partition from a shared-memory atomic (a
 // counting sort's first step); after the block scan of the partition histogram the whole keys
 // are computed, go to their partition's run in the staging buffer, and the runs leave in
-// order.  Bound by instruction issue and latency, not by HBM (19.2 GB written in 12.3 ms at 2.4 G
+// order.  Bound by instruction issue and latency, not by HBM (19.2 GB written in 11.9 ms at 2.4 G
 // windows): no key is kept in registers across the scan (each is computed once, after it) and
 // a staged key's partition is found from the key again, so that three blocks fit an SM (80
 // registers, 73 KB).  With the keys held and the partitions kept in shared memory there were
@@ -856,7 +888,7 @@ __global__ void k_fine_plan_batch(BatchTab t) {
 // SC_ONE (one-level partitioning): the partitions are the fine ones, found through the bins'
 // map, a sub-step reserves its run in each with one atomic, and the keys go to sbuf.
 enum { SC_COARSE, SC_DIRECT, SC_ONE };
-template <int KW, int NT, int MODE = SC_COARSE>
+template <int KW, int NT, int MODE, int VAR>
 __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, uint32_t bid) {
   typedef typename KeyT<KW>::T K;
   constexpr int WPT = KW == 1 ? 32 : 16;    // windows per thread
@@ -865,6 +897,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   constexpr int SUB = NT * WPT;             // windows per sub-step
   extern __shared__ __align__(16) uint8_t sm[];
   constexpr bool DIRECT = MODE == SC_DIRECT, ONE = MODE == SC_ONE;
+  const int canonical = VAR == V_SHORT ? s.canonical : VAR == V_CANON;
   const int P1 = ONE ? (int)min(b.meta->n_fine, s.nf_max) : 1 << s.b1, PM = ONE ? (int)s.nf_max : P1;
   K* stage = reinterpret_cast<K*>(sm);                                                // [SUB]
   unsigned long long* cursor = reinterpret_cast<unsigned long long*>(stage + SUB);   // [P1] absolute write positions
@@ -883,13 +916,14 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     // the tile's run in partition c, reserved at once (the order of the tiles' runs inside a
     // partition does not matter to any later step)
     if constexpr (!ONE) {
-      const uint32_t n = DIRECT ? 0u : b.hist[tile * P1 + c];
-      cursor[c] = n ? atomicAdd(&b.fcur[c], (unsigned long long)n) : 0ull;
+      const int p = P1 - 1 - c;  // shared arrays: partitions from the last to the first
+      const uint32_t n = DIRECT ? 0u : b.hist[tile * P1 + p];
+      cursor[c] = n ? atomicAdd(&b.fcur[p], (unsigned long long)n) : 0ull;
     }
     hist[PAD(c)] = 0;
   }
   if constexpr (ONE)
-    for (int i = t; i < (1 << s.bb); i += NT) map[i] = b.bmap[i];
+    for (int i = t; i < (1 << s.bb); i += NT) map[i] = b.bmap[(1 << s.bb) - 1 - i];
   if (t == 0) rcur_s = b.tile_first[tile];
   for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
@@ -925,17 +959,17 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
 #pragma unroll
     for (int i = 0; i < WPT; ++i) {
       uint32_t f, r;
-      const uint32_t x = win_top32<KW, WPT>(W, i, s.canonical, f, r);
-      uint32_t c = coarse_field(umap(x, s.canonical), ONE ? s.bb : s.b1);
+      const uint32_t x = win_top32<KW, WPT, VAR>(W, i, canonical, f, r);
+      uint32_t c = coarse_field_rev(x, canonical, ONE ? s.bb : s.b1);
       if constexpr (ONE) c = map[c];
       const bool v = (valid >> i) & 1u;
       if constexpr (DIRECT) {
         if (v) {
           uint64_t c0, c1;
           K key;
-          win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+          win_top<KW, WPT>(W, i, canonical, c0, c1);
           top_to_key(c0, c1, s.k, key);
-          const unsigned long long pos = atomicAdd(&b.fcur[c], 1ull);
+          const unsigned long long pos = atomicAdd(&b.fcur[P1 - 1 - c], 1ull);
           if (pos < s.cap) store_key(b.kbuf, pos, key);
           else atomicOr(&b.meta->status, ST_INTERNAL);
         }
@@ -947,7 +981,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
         if (v && sketch_sampled(f, r)) {
           uint64_t c0, c1;
           K key;
-          win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+          win_top<KW, WPT>(W, i, canonical, c0, c1);
           top_to_key(c0, c1, s.k, key);
           sketch_add(b.hll, key);
         }
@@ -981,7 +1015,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
       // one window invalid, at most SUB - 1 are valid) and the write-out never reads
       uint64_t c0, c1;
       K key;
-      win_top<KW, WPT>(W, i, s.canonical, c0, c1);
+      win_top<KW, WPT>(W, i, canonical, c0, c1);
       top_to_key(c0, c1, s.k, key);
       const uint32_t pos = (valid & (1u << i)) ? soff[PAD(cr[i] >> 16)] + (cr[i] & 0xffffu) : (uint32_t)(SUB - 1);
       stage[pos] = key;
@@ -990,7 +1024,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     if (fits) {
       for (uint32_t i = t; i < n_sub; i += NT) {
         const K key = stage[i];
-        const uint32_t c = coarse_of(key, s.k, s.canonical, ONE ? s.bb : s.b1);  // same field as above, from the key
+        const uint32_t c = coarse_field_rev(top32_of(key, s.k), canonical, ONE ? s.bb : s.b1);  // as above, from the key
         if constexpr (ONE) store_key(b.sbuf, (uint32_t)(hist[PAD(map[c])] + i), key);
         else store_key(b.kbuf, cursor[c] + i, key);
       }
@@ -1004,20 +1038,20 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     }
   }
 }
-template <int KW, int NT, int MODE>
+template <int KW, int NT, int MODE, int VAR>
 __global__ void __launch_bounds__(NT, 3) k_scatter(Shape s, Buffers b) {
-  scatter_body<KW, NT, MODE>(s, b, blockIdx.x);
+  scatter_body<KW, NT, MODE, VAR>(s, b, blockIdx.x);
 }
 // Aggregation ablation: pass B writes every key on its own through the partition cursors.
 template <int KW>
 __global__ void __launch_bounds__(256, 2) k_scatter_direct(Shape s, Buffers b) {
-  scatter_body<KW, 256, SC_DIRECT>(s, b, blockIdx.x);
+  scatter_body<KW, 256, SC_DIRECT, V_SHORT>(s, b, blockIdx.x);
 }
 
-template <int KW, int NT, int MODE>
+template <int KW, int NT, int MODE, int VAR>
 __global__ void __launch_bounds__(NT, 3) k_scatter_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  scatter_body<KW, NT, MODE>(d.s, d.b, bid);
+  scatter_body<KW, NT, MODE, VAR>(d.s, d.b, bid);
 }
 
 // ------------------------------------------------------------------ phase 2: fine split
@@ -2451,14 +2485,20 @@ int configure_kernels(int device) {
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)) != cudaSuccess) \
       return (int)e;                                                                                        \
   }
-  KC_SET((k_pack_count<1, false>));
-  KC_SET((k_pack_count<1, true>));
-  KC_SET((k_pack_count<2, false>));
-  KC_SET((k_pack_count<2, true>));
-  KC_SET((k_scatter<1, 256, SC_COARSE>));
-  KC_SET((k_scatter<1, 256, SC_ONE>));
-  KC_SET((k_scatter<2, 256, SC_COARSE>));
-  KC_SET((k_scatter<2, 256, SC_ONE>));
+#define KC_SET_PHASE1(KW, VAR)                              \
+  KC_SET((k_pack_count<KW, false, VAR>));                   \
+  KC_SET((k_pack_count<KW, true, VAR>));                    \
+  KC_SET((k_pack_count_batch<KW, false, VAR>));             \
+  KC_SET((k_pack_count_batch<KW, true, VAR>));              \
+  KC_SET((k_scatter<KW, 256, SC_COARSE, VAR>));             \
+  KC_SET((k_scatter<KW, 256, SC_ONE, VAR>));                \
+  KC_SET((k_scatter_batch<KW, 256, SC_COARSE, VAR>));       \
+  KC_SET((k_scatter_batch<KW, 256, SC_ONE, VAR>))
+  KC_SET_PHASE1(1, V_SHORT);
+  KC_SET_PHASE1(1, V_CANON);
+  KC_SET_PHASE1(1, V_FORWARD);
+  KC_SET_PHASE1(2, V_CANON);
+  KC_SET_PHASE1(2, V_FORWARD);
   KC_SET(k_scatter_direct<1>);
   KC_SET(k_scatter_direct<2>);
   KC_SET(k_fine_plan);
@@ -2470,14 +2510,6 @@ int configure_kernels(int device) {
   KC_SET(k_count_emit<2>);
   KC_SET((k_count_emit<1, true>));
   KC_SET((k_count_emit<2, true>));
-  KC_SET((k_pack_count_batch<1, false>));
-  KC_SET((k_pack_count_batch<1, true>));
-  KC_SET((k_pack_count_batch<2, false>));
-  KC_SET((k_pack_count_batch<2, true>));
-  KC_SET((k_scatter_batch<1, 256, SC_COARSE>));
-  KC_SET((k_scatter_batch<1, 256, SC_ONE>));
-  KC_SET((k_scatter_batch<2, 256, SC_COARSE>));
-  KC_SET((k_scatter_batch<2, 256, SC_ONE>));
   KC_SET(k_fine_plan_batch);
   KC_SET(k_fine_hist_batch<1>);
   KC_SET(k_fine_hist_batch<2>);
@@ -2498,6 +2530,21 @@ int configure_kernels(int device) {
     mark(name);                                         \
   } while (0)
 
+// CALL(key words, variant) for a count's key width, k and mode.
+#define KC_PHASE1_VARIANT(s, CALL)                         \
+  do {                                                     \
+    if ((s).kw == 2) {                                     \
+      if ((s).canonical) { CALL(2, V_CANON); }             \
+      else { CALL(2, V_FORWARD); }                         \
+    } else if ((s).k < 16) {                               \
+      CALL(1, V_SHORT);                                    \
+    } else if ((s).canonical) {                            \
+      CALL(1, V_CANON);                                    \
+    } else {                                               \
+      CALL(1, V_FORWARD);                                  \
+    }                                                      \
+  } while (0)
+
 int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, const Marker& mark) {
   cudaStream_t st = (cudaStream_t)stream;
   int launches = 0;
@@ -2506,13 +2553,11 @@ int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, con
   KC_STEP("k_prepare");
   const unsigned gt = pack_blocks(s);
   const size_t smA = pack_smem(s);
-  if (s.kw == 1) {
-    if (s.one_level) k_pack_count<1, true><<<gt, kPackThreads, smA, st>>>(s, b);
-    else k_pack_count<1, false><<<gt, kPackThreads, smA, st>>>(s, b);
-  } else {
-    if (s.one_level) k_pack_count<2, true><<<gt, kPackThreads, smA, st>>>(s, b);
-    else k_pack_count<2, false><<<gt, kPackThreads, smA, st>>>(s, b);
-  }
+#define KC_PACK(KW, VAR)                                                                  \
+  if (s.one_level) k_pack_count<KW, true, VAR><<<gt, kPackThreads, smA, st>>>(s, b);      \
+  else k_pack_count<KW, false, VAR><<<gt, kPackThreads, smA, st>>>(s, b)
+  KC_PHASE1_VARIANT(s, KC_PACK);
+#undef KC_PACK
   ++launches;
   KC_STEP("k_pack_count");
   return launches;
@@ -2529,12 +2574,12 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     if (s.aggr & kAggrNoSmemBuckets) {
       if (s.kw == 1) k_scatter_direct<1><<<gt, 256, smB, st>>>(s, b);
       else k_scatter_direct<2><<<gt, 256, smB, st>>>(s, b);
-    } else if (s.kw == 1) {
-      if (s.one_level) k_scatter<1, 256, SC_ONE><<<gt, 256, smB, st>>>(s, b);
-      else k_scatter<1, 256, SC_COARSE><<<gt, 256, smB, st>>>(s, b);
     } else {
-      if (s.one_level) k_scatter<2, 256, SC_ONE><<<gt, 256, smB, st>>>(s, b);
-      else k_scatter<2, 256, SC_COARSE><<<gt, 256, smB, st>>>(s, b);
+#define KC_SCATTER(KW, VAR)                                                       \
+  if (s.one_level) k_scatter<KW, 256, SC_ONE, VAR><<<gt, 256, smB, st>>>(s, b);   \
+  else k_scatter<KW, 256, SC_COARSE, VAR><<<gt, 256, smB, st>>>(s, b)
+      KC_PHASE1_VARIANT(s, KC_SCATTER);
+#undef KC_SCATTER
     }
     ++launches;
     KC_STEP("k_scatter");
@@ -2641,31 +2686,20 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
   }
   if (std::max(smB[0], smB[1]) + kScatterStaticSmem > s0.smem_budget) return -(int)cudaErrorInvalidConfiguration;
   KC_BLAUNCH(BK_PREPARE, (k_prepare_batch<<<bp.grid[BK_PREPARE], 256, 0, st>>>(tab(BK_PREPARE))), "k_prepare");
-  if (bp.kw == 1) {
-    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<1, false><<<bp.grid[BK_PACK], kPackThreads, smA[0], st>>>(tab(BK_PACK))),
-               "k_pack_count");
-    KC_BLAUNCH(BK_PACK_ONE,
-               (k_pack_count_batch<1, true><<<bp.grid[BK_PACK_ONE], kPackThreads, smA[1], st>>>(tab(BK_PACK_ONE))),
-               "k_pack_count");
-    KC_BLAUNCH(BK_SCATTER,
-               (k_scatter_batch<1, 256, SC_COARSE><<<bp.grid[BK_SCATTER], 256, smB[0], st>>>(tab(BK_SCATTER))),
-               "k_scatter");
-    KC_BLAUNCH(BK_SCATTER_ONE,
-               (k_scatter_batch<1, 256, SC_ONE><<<bp.grid[BK_SCATTER_ONE], 256, smB[1], st>>>(tab(BK_SCATTER_ONE))),
-               "k_scatter");
-  } else {
-    KC_BLAUNCH(BK_PACK, (k_pack_count_batch<2, false><<<bp.grid[BK_PACK], kPackThreads, smA[0], st>>>(tab(BK_PACK))),
-               "k_pack_count");
-    KC_BLAUNCH(BK_PACK_ONE,
-               (k_pack_count_batch<2, true><<<bp.grid[BK_PACK_ONE], kPackThreads, smA[1], st>>>(tab(BK_PACK_ONE))),
-               "k_pack_count");
-    KC_BLAUNCH(BK_SCATTER,
-               (k_scatter_batch<2, 256, SC_COARSE><<<bp.grid[BK_SCATTER], 256, smB[0], st>>>(tab(BK_SCATTER))),
-               "k_scatter");
-    KC_BLAUNCH(BK_SCATTER_ONE,
-               (k_scatter_batch<2, 256, SC_ONE><<<bp.grid[BK_SCATTER_ONE], 256, smB[1], st>>>(tab(BK_SCATTER_ONE))),
-               "k_scatter");
-  }
+#define KC_PHASE1(KW, VAR)                                                                                          \
+  KC_BLAUNCH(BK_PACK, (k_pack_count_batch<KW, false, VAR><<<bp.grid[BK_PACK], kPackThreads, smA[0], st>>>(tab(BK_PACK))), \
+             "k_pack_count");                                                                                      \
+  KC_BLAUNCH(BK_PACK_ONE,                                                                                          \
+             (k_pack_count_batch<KW, true, VAR><<<bp.grid[BK_PACK_ONE], kPackThreads, smA[1], st>>>(tab(BK_PACK_ONE))), \
+             "k_pack_count");                                                                                      \
+  KC_BLAUNCH(BK_SCATTER,                                                                                           \
+             (k_scatter_batch<KW, 256, SC_COARSE, VAR><<<bp.grid[BK_SCATTER], 256, smB[0], st>>>(tab(BK_SCATTER))), \
+             "k_scatter");                                                                                         \
+  KC_BLAUNCH(BK_SCATTER_ONE,                                                                                       \
+             (k_scatter_batch<KW, 256, SC_ONE, VAR><<<bp.grid[BK_SCATTER_ONE], 256, smB[1], st>>>(tab(BK_SCATTER_ONE))), \
+             "k_scatter")
+  KC_PHASE1_VARIANT(s0, KC_PHASE1);  // (all counts of a batch have the same k and mode)
+#undef KC_PHASE1
   KC_BLAUNCH(BK_FINE_PLAN, (k_fine_plan_batch<<<bp.grid[BK_FINE_PLAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_FINE_PLAN))),
              "k_fine_plan");
   // the fine split; then, for counts with a sampled layout, the exact split again (each
