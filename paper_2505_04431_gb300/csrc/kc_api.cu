@@ -192,6 +192,12 @@ struct kc_plan_s {
   size_t smem_per_sm = 0;
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  // kc_count's read-backs (the offsets' ends, the status record): pinned, so that the copies
+  // are not staged by the driver
+  struct ReadBack {
+    uint64_t ends[2];
+    kc::Meta meta;
+  }* rb = nullptr;
   // batched counts: scratch arena of a group of counts, device and pinned host tables
   void* bws = nullptr;
   size_t bws_bytes = 0;
@@ -257,6 +263,8 @@ void dev_free_on(kc_plan_s* p, void* ptr, cudaStream_t st) {
   if (p->free_) p->free_(ptr, (void*)st, p->ctx);
   else cudaFreeAsync(ptr, st);
 }
+// (a result's counts lie behind its keys in one allocation)
+size_t counts_at(size_t key_bytes) { return align_up(key_bytes, 256); }
 void* dev_alloc(kc_plan_s* p, size_t bytes) { return dev_alloc_on(p, bytes, p->stream); }
 void dev_free(kc_plan_s* p, void* ptr) { dev_free_on(p, ptr, p->stream); }
 
@@ -355,6 +363,13 @@ void plan_job(const kc_plan_s* p, const uint8_t* reads, const uint64_t* offsets,
   j.ws_bytes = j.lay.total;
   j.out_key_bytes = j.s.cap * j.s.kw * 8;
   j.out_cnt_bytes = j.s.cap * 4;
+}
+
+// One allocation for a count's keys and, behind them, its counts; false if there is none.
+bool alloc_outputs(kc_plan_s* p, Job& j) {
+  j.okeys = dev_alloc(p, counts_at(j.out_key_bytes) + j.out_cnt_bytes);
+  j.ocnts = j.okeys ? (uint8_t*)j.okeys + counts_at(j.out_key_bytes) : nullptr;
+  return j.okeys != nullptr;
 }
 
 // The buffers of one count with scratch at `ws` and its outputs at j.okeys / j.ocnts.
@@ -483,7 +498,6 @@ void retire(kc_plan_s* p, uint64_t id, AsyncJob* a, bool drop) {
       release_owner(p, a->owner);
     } else {
       dev_free(p, a->j.okeys);
-      dev_free(p, a->j.ocnts);
     }
   }
   if (a->ev) cudaEventDestroy(a->ev);
@@ -736,6 +750,12 @@ kc_status kc_plan(const kc_plan_opts* opts, kc_plan_t* out) {
       }
     }
   }
+  if ((e = cudaMallocHost((void**)&p->rb, sizeof(*p->rb))) != cudaSuccess) {
+    if (p->profile)
+      for (int i = 0; i <= kc_plan_s::kMaxMarks; ++i) cudaEventDestroy(p->ev[i]);
+    delete p;
+    return cuda_fail(e, "kc_plan: pinned read-back buffer");
+  }
   *out = p;
   return KC_OK;
 }
@@ -751,6 +771,7 @@ kc_status kc_plan_destroy(kc_plan_t p) {
     retire(p, it->first, it->second, true);
   }
   if (p->pinned) cudaFreeHost(p->pinned);
+  cudaFreeHost(p->rb);
   if (p->btab_host) cudaFreeHost(p->btab_host);
   if (p->bmeta) cudaFreeHost(p->bmeta);
   for (auto& st : p->stg) {
@@ -793,8 +814,7 @@ kc_status kc_free(kc_plan_t p, kc_result* r) {
   if (r->_owner) {  // a result of a batched group: the group's buffers go with its last result
     release_owner(p, (GroupOwner*)r->_owner);
   } else {
-    dev_free(p, r->keys);
-    dev_free(p, r->counts);
+    dev_free(p, r->keys);  // the counts lie in the same block
   }
   memset(r, 0, sizeof(*r));
   return KC_OK;
@@ -850,10 +870,14 @@ kc_status kc_count(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, u
   const bool off_dev = is_device_ptr(offsets);
   uint64_t first = 0, L = 0;
   if (off_dev) {
-    if ((e = cudaMemcpyAsync(&first, offsets, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&L, offsets + n_reads, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(&p->rb->ends[0], offsets, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&p->rb->ends[1], offsets + n_reads, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(st)) != cudaSuccess) {
+      cudaStreamSynchronize(st);  // no copy into the buffer is left behind
       return cuda_fail(e, "kc_count: reading offsets");
+    }
+    first = p->rb->ends[0];
+    L = p->rb->ends[1];
   } else {  // their order is checked on the device (k_check_offsets), as for device offsets
     first = offsets[0];
     L = offsets[n_reads];
@@ -874,18 +898,12 @@ kc_status kc_count(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, u
     p->ws = w;
     p->ws_bytes = j.ws_bytes;
   }
-  j.okeys = dev_alloc(p, j.out_key_bytes);
-  j.ocnts = j.okeys ? dev_alloc(p, j.out_cnt_bytes) : nullptr;
-  if (!j.okeys || !j.ocnts) {
-    dev_free(p, j.okeys);
-    return fail(KC_ENOMEM, "kc_count: result allocation failed");
-  }
+  if (!alloc_outputs(p, j)) return fail(KC_ENOMEM, "kc_count: result allocation failed");
   // on any error: let the launched work finish before its buffers go back to the allocator
   auto bail = [&](kc_status stc, const std::string& msg) {
     cudaStreamSynchronize(st);
     cudaGetLastError();
     dev_free(p, j.okeys);
-    dev_free(p, j.ocnts);
     return fail(stc, msg);
   };
 
@@ -900,7 +918,7 @@ kc_status kc_count(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, u
     mark.fn = debug_mark;
     mark.ctx = p;
   }
-  kc::Meta m{};
+  kc::Meta& m = p->rb->meta;
   int launches = 0;
   std::string err;
   if (!enqueue_job(j, (uint8_t*)p->ws, st, &m, mark, p->n_sms, &launches, &err)) return bail(KC_ECUDA, "kc_count: " + err);
@@ -979,10 +997,7 @@ kc_status kc_count_batch(kc_plan_t p, uint32_t n_samples, const uint8_t* const* 
   auto release = [&](kc_status stc, const std::string& msg) {
     cudaStreamSynchronize(p->stream);
     cudaGetLastError();
-    for (uint32_t i : gp.alone) {
-      dev_free(p, jobs[i].okeys);
-      dev_free(p, jobs[i].ocnts);
-    }
+    for (uint32_t i : gp.alone) dev_free(p, jobs[i].okeys);
     for (GroupOwner* o : owners)
       if (o) {
         dev_free(p, o->keys);
@@ -997,9 +1012,7 @@ kc_status kc_count_batch(kc_plan_t p, uint32_t n_samples, const uint8_t* const* 
   uint32_t launches = 0;
   for (uint32_t i : gp.alone) {
     Job& j = jobs[i];
-    j.okeys = dev_alloc(p, j.out_key_bytes);
-    j.ocnts = j.okeys ? dev_alloc(p, j.out_cnt_bytes) : nullptr;
-    if (!j.okeys || !j.ocnts) return release(KC_ENOMEM, "kc_count_batch: result allocation failed");
+    if (!alloc_outputs(p, j)) return release(KC_ENOMEM, "kc_count_batch: result allocation failed");
     int nl = 0;
     if (!enqueue_job(j, (uint8_t*)p->ws, p->stream, &metas[i], none, p->n_sms, &nl, &err))
       return release(KC_ECUDA, "kc_count_batch: " + err);
@@ -1107,10 +1120,7 @@ kc_status kc_submit(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, 
     }
     p->ws_bytes = a->j.ws_bytes;
   }
-  a->j.okeys = dev_alloc(p, a->j.out_key_bytes);
-  a->j.ocnts = a->j.okeys ? dev_alloc(p, a->j.out_cnt_bytes) : nullptr;
-  if (!a->j.okeys || !a->j.ocnts) {
-    dev_free(p, a->j.okeys);
+  if (!alloc_outputs(p, a->j)) {
     drop_unsubmitted(p, a);
     return fail(KC_ENOMEM, "kc_submit: result allocation failed");
   }
@@ -1197,10 +1207,7 @@ kc_status kc_submit_batch(kc_plan_t p, uint32_t n_samples, const uint8_t* const*
   auto release = [&](kc_status stc, const std::string& msg) {
     cudaStreamSynchronize(p->stream);
     cudaGetLastError();
-    for (uint32_t i : gp.alone) {
-      dev_free(p, jobs[i].okeys);
-      dev_free(p, jobs[i].ocnts);
-    }
+    for (uint32_t i : gp.alone) dev_free(p, jobs[i].okeys);
     for (GroupOwner* o : owners)
       if (o) {
         dev_free(p, o->keys);
@@ -1214,9 +1221,7 @@ kc_status kc_submit_batch(kc_plan_t p, uint32_t n_samples, const uint8_t* const*
   uint32_t launches = 0;
   for (uint32_t i : gp.alone) {
     Job& j = jobs[i];
-    j.okeys = dev_alloc(p, j.out_key_bytes);
-    j.ocnts = j.okeys ? dev_alloc(p, j.out_cnt_bytes) : nullptr;
-    if (!j.okeys || !j.ocnts) return release(KC_ENOMEM, "kc_submit_batch: result allocation failed");
+    if (!alloc_outputs(p, j)) return release(KC_ENOMEM, "kc_submit_batch: result allocation failed");
     int nl = 0;
     if (!enqueue_job(j, (uint8_t*)p->ws, p->stream, &p->pinned[made[i]->slot], none, p->n_sms, &nl, &err))
       return release(KC_ECUDA, "kc_submit_batch: " + err);
