@@ -92,9 +92,13 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   s.fine_target = ft < 16 ? 16u : (uint32_t)ft;
   s.cap = L > 0 ? L : 1;
   // sum over partitions of ceil(n_c / target), target >= fine_target: at most K / ft + P1
-  const uint64_t nf_bound = s.cap / s.fine_target + P1 + 1;
+  // (more where the plan rounds the partitions up to a whole number per SM: at most one more
+  // per SM, of kMinFineKeys keys at least)
+  const uint64_t nf_target = s.cap / s.fine_target;
+  const uint64_t nf_waves = std::min<uint64_t>(nf_target + (uint64_t)o.n_sms, s.cap / kMinFineKeys);
   const uint64_t nf_lim = P1 * kMaxFine;
-  s.nf_max = nf_bound < nf_lim ? nf_bound : nf_lim;
+  s.nf_max = std::min(std::max(nf_target, nf_waves) + P1 + 1, nf_lim);
+  s.n_sms = o.n_sms;
   // Inputs that would be a single coarse partition (12 Mi bases of 64-bit keys, 6 Mi of 128-bit
   // keys) are partitioned once: pass A already knows the windows per bin and the sketch, so
   // pass B can write the fine partitions, and the fine split's kernels and its pass over the
@@ -110,7 +114,7 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   // in all, and at least 16 keys each); a layout that does not fit falls back to the exact one
   s.fine_sampled = o.allow_sampled && (o.force_sampled || L >= kFineSampledMinBases) ? 1 : 0;
   s.tight_slack = o.tight_slack;
-  s.cap_kb = s.fine_sampled ? s.cap + s.cap / 4 + s.nf_max * 64 : s.cap;
+  s.cap_kb = s.fine_sampled ? s.cap + s.cap / 4 + std::min(nf_target + P1 + 1, nf_lim) * 64 : s.cap;
   s.smem_budget = o.smem_optin;
   s.spin_limit = o.withhold ? kTestSpinLimit : kLookbackSpinLimit;
   s.count_limit = o.low_count_limit ? kTestCountLimit : 0xffffffffu;
@@ -127,9 +131,9 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   };
   lay.reads = take(copy_reads ? L + 16 : 0);
   lay.offs = take(copy_offs ? (n_reads + 1) * 8 : 0);
-  lay.codes = take(s.n_words * 8);
+  // flo of the two-level path is written after pass B has read the codes
+  lay.codes = take(std::max<uint64_t>(s.n_words * 8, s.one_level ? 0 : (nf + 1) * 4));
   lay.inv = take(s.n_words * 4);
-  lay.tf = take(s.n_tiles * 8);
   const uint64_t bins = s.one_level ? 1ull << s.bb : 0;
   lay.cst = take(std::max<uint64_t>((P1 + 1) * 8, bins * 4));
   lay.bmap = take(bins * 2);
@@ -138,14 +142,19 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.hll = take((size_t)kHllRegs * 4);
   lay.fh = take(nf * 4);
   lay.fo = take((nf + 1) * 8);
-  lay.flo = take((nf + 1) * 4);
+  lay.flo = s.one_level ? take((nf + 1) * 4) : lay.codes;
   lay.fc = take(nf * 8);
   lay.look = take(nf * 8);
   // one-level: no coarse-grouped keys, only the counts of deferred runs
-  lay.kbuf = take(s.one_level ? s.cap * 4 : s.cap_kb * s.kw * 8);
-  const uint64_t hist_bytes = s.one_level ? 0 : s.n_tiles * P1 * 4;  // pass A's histogram lies in sbuf's memory
+  // Phase 1's tables lie in the memory of the keys array that it does not write: each tile's
+  // first read in kbuf (one-level) or sbuf, and behind that pass A's histogram in sbuf
+  const uint64_t tf_bytes = (s.n_tiles * 8 + 255) / 256 * 256;
+  lay.kbuf = take(s.one_level ? std::max<uint64_t>(s.cap * 4, tf_bytes) : s.cap_kb * s.kw * 8);
+  const uint64_t hist_bytes = s.one_level ? 0 : tf_bytes + s.n_tiles * P1 * 4;
   lay.sbuf = take(std::max<uint64_t>(s.cap_kb * s.kw * 8, hist_bytes));
   lay.meta = take(sizeof(Meta));
+  lay.tf = s.one_level ? lay.kbuf : lay.sbuf;
+  lay.hist = lay.sbuf + tf_bytes;
   lay.total = at;
   return (uint32_t)nf;
 }
@@ -157,7 +166,7 @@ Buffers layout_buffers(const Layout& lay, uint8_t* ws) {
   b.codes64 = (uint64_t*)(ws + lay.codes);
   b.inv32 = (uint32_t*)(ws + lay.inv);
   b.tile_first = (uint64_t*)(ws + lay.tf);
-  b.hist = (uint32_t*)(ws + lay.sbuf);
+  b.hist = (uint32_t*)(ws + lay.hist);
   b.cstart = (uint64_t*)(ws + lay.cst);
   b.bins = (uint32_t*)(ws + lay.cst);
   b.bmap = (uint16_t*)(ws + lay.bmap);
@@ -334,6 +343,7 @@ kc::ShapeOpts shape_opts(const kc_plan_s* p) {
   o.slots_max = p->slots_max;
   o.smem_optin = p->smem_optin;
   o.smem_per_sm = p->smem_per_sm;
+  o.n_sms = p->n_sms;
   o.profile = p->profile ? 1 : 0;
   o.defer_all = p->defer_all ? 1 : 0;
   o.withhold = p->withhold ? 1 : 0;
@@ -522,7 +532,7 @@ void drop_unsubmitted(kc_plan_s* p, AsyncJob* a) {
 struct Group {
   std::vector<uint32_t> idx;
   std::vector<size_t> ws_off, key_off, cnt_off;
-  size_t ws = 0, keys = 0, cnts = 0, tab = 0;
+  size_t ws = 0, keys = 0, cnts = 0, tab = 0, metas = 0;
   uint64_t bases = 0;
 };
 struct GroupPlan {
@@ -581,7 +591,8 @@ bool plan_groups(const kc_plan_s* p, const std::vector<Job>& jobs, GroupPlan& gp
       }
       words += (n + 1) + sum;
     }
-    g.tab = align_up(n * sizeof(kc::BatchDesc), 256) + align_up(words * 4, 256);
+    g.metas = align_up(n * sizeof(kc::Meta), 256);
+    g.tab = align_up(n * sizeof(kc::BatchDesc), 256) + align_up(words * 4, 256) + g.metas;
     gp.tab_total += g.tab;
     gp.tab_max = std::max(gp.tab_max, g.tab);
   }
@@ -603,13 +614,19 @@ bool enqueue_group(kc_plan_s* p, std::vector<Job>& jobs, const Group& g, GroupOw
     return false;
   }
   kc::BatchDesc* hd = (kc::BatchDesc*)h;
+  // the group's status records lie side by side behind its tables, so that they come back in
+  // one copy (32 small counts: 32 copies of 2 us each)
+  kc::Meta* dmeta = (kc::Meta*)(dv + g.tab - g.metas);
   int P1_max = 1;
   for (uint32_t q = 0; q < n; ++q) {
     Job& j = jobs[g.idx[q]];
     j.okeys = (uint8_t*)o->keys + g.key_off[q];
     j.ocnts = (uint8_t*)o->counts + g.cnt_off[q];
     hd[q].s = j.s;
+    // the count's share of the SMs: its fine partitions fill those, not all of them
+    hd[q].s.n_sms = (int)std::max<uint64_t>(1, (uint64_t)p->n_sms * j.L / std::max<uint64_t>(g.bases, 1));
     hd[q].b = make_buffers(j, (uint8_t*)p->bws + g.ws_off[q]);
+    hd[q].b.meta = dmeta + q;
     P1_max = std::max(P1_max, j.P1);
     if (!enqueue_copies(j, hd[q].b, p->stream, err)) {
       *stc = KC_ECUDA;
@@ -644,7 +661,7 @@ bool enqueue_group(kc_plan_s* p, std::vector<Job>& jobs, const Group& g, GroupOw
     dw += n + 1 + at;
   }
   cudaError_t e;
-  if ((e = cudaMemcpyAsync(dv, h, g.tab, cudaMemcpyHostToDevice, p->stream)) != cudaSuccess) {
+  if ((e = cudaMemcpyAsync(dv, h, g.tab - g.metas, cudaMemcpyHostToDevice, p->stream)) != cudaSuccess) {
     *stc = KC_ECUDA;
     *err = std::string("copying tables: ") + cudaGetErrorString(e);
     return false;
@@ -657,13 +674,16 @@ bool enqueue_group(kc_plan_s* p, std::vector<Job>& jobs, const Group& g, GroupOw
     return false;
   }
   *launches += (uint32_t)nl;
-  for (uint32_t q = 0; q < n; ++q)
-    if ((e = cudaMemcpyAsync(meta_dst[q], hd[q].b.meta, sizeof(kc::Meta), cudaMemcpyDeviceToHost, p->stream)) !=
+  for (uint32_t q = 0, m; q < n; q += m) {  // records whose destinations lie side by side too: one copy
+    for (m = 1; q + m < n && meta_dst[q + m] == meta_dst[q] + m; ++m) {
+    }
+    if ((e = cudaMemcpyAsync(meta_dst[q], dmeta + q, m * sizeof(kc::Meta), cudaMemcpyDeviceToHost, p->stream)) !=
         cudaSuccess) {
       *stc = KC_ECUDA;
       *err = cudaGetErrorString(e);
       return false;
     }
+  }
   return true;
 }
 

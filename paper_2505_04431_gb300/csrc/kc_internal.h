@@ -28,7 +28,8 @@ constexpr int kMaxFine = 4096;                 // at most this many fine partiti
 // 2^6 .. 2^13 bins, about 8 to a fine partition, and its last block groups the bins into at
 // most this many fine partitions, which pass B writes directly.
 constexpr uint64_t kOneLevelFine = 3072;
-constexpr int kMinBinsLog2 = 6, kMaxBinsLog2 = 13;
+constexpr int kMinBinsLog2 = 10, kMaxBinsLog2 = 13;
+constexpr uint32_t kMinFineKeys = 512;         // smaller fine partitions are not made to fill the SMs
 // bases per coarse partition aimed at when the plan sets no partition count
 constexpr uint64_t coarse_bases(int kw) { return kw == 1 ? (12ull << 20) : (6ull << 20); }
 // count kernel: threads per block and blocks per SM (one block of 1024 threads with
@@ -109,6 +110,7 @@ struct Shape {
   int aggr;             // aggregation variants: kAggr* bits (single-count path only)
   int one_level;        // nonzero: pass B writes the fine partitions directly (b1 = 0)
   int bb;               // one-level: log2 of the bins that are grouped into fine partitions
+  int n_sms;
 };
 constexpr int kAggrNoSmemBuckets = 1;  // pass B writes every key on its own (global atomic cursor)
 constexpr int kAggrWarpMerge = 2;      // the count kernel adds a warp's equal keys with one atomic
@@ -118,7 +120,7 @@ struct Buffers {
   const uint64_t* offsets;
   uint64_t* codes64;
   uint32_t* inv32;
-  uint64_t* tile_first;   // first read index whose start is >= the tile's halo start
+  uint64_t* tile_first;   // first read index whose start is >= the tile's halo start (in a keys array's memory)
   uint32_t* hist;         // [n_tiles][P1], in sbuf's memory
   uint64_t* cstart;       // [P1 + 1] coarse partition starts
   uint32_t* fine_base;    // [P1 + 1] first fine index of each coarse partition
@@ -203,13 +205,14 @@ struct ShapeOpts {
   uint32_t slots_max = 0;   // largest count table (slots) or 0
   size_t smem_optin = 0;
   size_t smem_per_sm = 0;   // shared memory of one SM (for the count blocks it holds)
+  int n_sms = 0;
   int profile = 0, defer_all = 0, withhold = 0, low_count_limit = 0, aggr = 0;
   int allow_sampled = 0;   // a single count: the fine layout may be sized from a sample
   int force_sampled = 0;   // testing: sampled at any size
   int tight_slack = 0;     // testing: sampled regions get no slack
 };
 struct Layout {  // byte offsets into the count's scratch block
-  size_t reads, offs, codes, inv, tf, cst, bmap, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
+  size_t reads, offs, codes, inv, tf, hist, cst, bmap, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
   size_t total;
 };
 // Fills s and lay for L bases and n_reads reads; copy_reads / copy_offs: the scratch holds a

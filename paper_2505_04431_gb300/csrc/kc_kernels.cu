@@ -609,8 +609,11 @@ __device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
 }
 
 // The keys a fine partition aims at, from the sketch of a count of K windows: fine_target
-// distinct keys, i.e. fine_target * K / D keys.  All threads of the block call it.
-__device__ double sketch_target(const uint32_t* hll, uint64_t K, uint32_t fine_target, Meta* meta) {
+// distinct keys, i.e. fine_target * K / D keys; where that gives an SM few partitions, as much
+// less as makes them a whole number (one partition too many for a last wave costs a small
+// count a wave: 10 M bases had 497 for 152 SMs, and 0.2 M bases 11).  `extra`: partitions that
+// come on top of K / target.  All threads of the block call it.
+__device__ double sketch_target(const uint32_t* hll, uint64_t K, const Shape& s, uint32_t extra, Meta* meta) {
   __shared__ float zsum_s[32], zeros_s[32];
   __shared__ double target_s;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -632,18 +635,25 @@ __device__ double sketch_target(const uint32_t* hll, uint64_t K, uint32_t fine_t
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double zs = 0, zr = 0;
+    float zs = 0, zr = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
       zs += zsum_s[w];
       zr += zeros_s[w];
     }
-    const double m = kHllRegs;
-    double e = 0.7213 / (1.0 + 1.079 / m) * m * m / zs;
-    if (e < 2.5 * m && zr > 0) e = m * log(m / zr);
-    const double d_est = e * kHllSample;
-    double dup = d_est > 1.0 ? (double)K / d_est : 1.0;
-    dup = dup < 1.0 ? 1.0 : (dup > 32.0 ? 32.0 : dup);
-    target_s = (double)fine_target * (0.9 * dup > 1.0 ? 0.9 * dup : 1.0);
+    // (single precision: the estimate is good to 3%, and double precision is slow here)
+    const float m = kHllRegs;
+    float e = 0.7213f / (1.0f + 1.079f / m) * m * m / zs;
+    if (e < 2.5f * m && zr > 0) e = m * logf(m / zr);
+    const float d_est = e * (float)kHllSample;
+    float dup = d_est > 1.0f ? (float)K / d_est : 1.0f;
+    dup = fminf(fmaxf(dup, 1.0f), 32.0f);
+    float target = (float)s.fine_target * fmaxf(0.9f * dup, 1.0f);
+    const float per_sm = ceilf(((float)K / target + (float)extra) / (float)s.n_sms);
+    if (per_sm <= 16.0f) {
+      const float parts = per_sm * (float)s.n_sms - (float)extra;
+      target = fminf(target, fmaxf((float)K / parts + 1.0f, (float)kMinFineKeys));
+    }
+    target_s = target;
     meta->d_estimate = (uint64_t)d_est;
   }
   __syncthreads();
@@ -685,8 +695,8 @@ __device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b,
   for (int i = threadIdx.x; i < NB; i += blockDim.x) sc[PAD(i)] = __ldcg(&b.bins[i]);
   __syncthreads();
   const uint32_t K = block_exclusive_scan_pad<uint32_t>(sc, NB, wt);  // below 2^24
-  const double target = sketch_target(b.hll, K, s.fine_target, b.meta);
-  const uint32_t T = max((uint32_t)target, (uint32_t)(K / s.nf_max) + 1u);
+  const double target = sketch_target(b.hll, K, s, 0, b.meta);
+  const uint32_t T = max((uint32_t)ceil(target), (uint32_t)(K / s.nf_max) + 1u);
   const uint32_t NF = sc[PAD(NB - 1)] / T + 1;  // the last bin's partition is the last: at most K / T + 1 <= nf_max
   for (int i = threadIdx.x; i < NB; i += blockDim.x) {
     const uint32_t p = sc[PAD(i)];
@@ -827,11 +837,15 @@ __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count_ba
 // Fine split of every coarse partition, after pass B: the distinct-key estimate (a sampled
 // HyperLogLog filled by pass B) gives the duplication factor K / D, and a fine partition
 // aims at fine_target distinct keys, i.e. fine_target * K / D keys.  One block.
-__device__ __forceinline__ void fine_plan_body(const uint64_t* cstart, const uint32_t* hll, uint32_t* fine_base, uint32_t* fine_m,
-                            uint32_t* flo, int P1, int b1, uint32_t fine_target, uint32_t nf_max, Meta* meta) {
+__device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b) {
+  const uint64_t* cstart = b.cstart;
+  uint32_t *fine_base = b.fine_base, *fine_m = b.fine_m, *flo = b.flo;
+  const int P1 = 1 << s.b1, b1 = s.b1;
+  const uint32_t nf_max = (uint32_t)s.nf_max;
+  Meta* meta = b.meta;
   extern __shared__ uint64_t fsc[];  // [P1]
   __shared__ uint64_t wt[32];
-  const double target = sketch_target(hll, cstart[P1], fine_target, meta);
+  const double target = sketch_target(b.hll, cstart[P1], s, P1, meta);
   for (int c = threadIdx.x; c < P1; c += blockDim.x) {
     const uint64_t n = cstart[c + 1] - cstart[c];
     uint64_t m = (uint64_t)ceil((double)n / target);
@@ -863,14 +877,10 @@ __device__ __forceinline__ void fine_plan_body(const uint64_t* cstart, const uin
     if (NF > nf_max) atomicOr(&meta->status, ST_INTERNAL);
   }
 }
-__global__ void k_fine_plan(const uint64_t* cstart, const uint32_t* hll, uint32_t* fine_base, uint32_t* fine_m,
-                            uint32_t* flo, int P1, int b1, uint32_t fine_target, uint32_t nf_max, Meta* meta) {
-  fine_plan_body(cstart, hll, fine_base, fine_m, flo, P1, b1, fine_target, nf_max, meta);
-}
+__global__ void k_fine_plan(Shape s, Buffers b) { fine_plan_body(s, b); }
 __global__ void k_fine_plan_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  fine_plan_body(d.b.cstart, d.b.hll, d.b.fine_base, d.b.fine_m, d.b.flo, 1 << d.s.b1, d.s.b1, d.s.fine_target,
-                 (uint32_t)d.s.nf_max, d.b.meta);
+  fine_plan_body(d.s, d.b);
 }
 
 // ------------------------------------------------------------------ pass B
@@ -2585,8 +2595,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     KC_STEP("k_scatter");
   }
   if (!s.one_level) {
-    k_fine_plan<<<1, 1024, (size_t)P1 * 8, st>>>(b.cstart, b.hll, b.fine_base, b.fine_m, b.flo, P1, s.b1, s.fine_target,
-                                                 nf_max, b.meta);
+    k_fine_plan<<<1, 1024, (size_t)P1 * 8, st>>>(s, b);
     ++launches;
     KC_STEP("k_fine_plan");
     const unsigned gf = (unsigned)(n_sms * 2);

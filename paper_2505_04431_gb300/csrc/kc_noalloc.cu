@@ -126,6 +126,7 @@ extern "C" kc_status kc_count_noalloc(const uint8_t* reads, const uint64_t* offs
   kc::ShapeOpts so;
   so.smem_optin = ds->smem_optin;
   so.smem_per_sm = ds->smem_per_sm;
+  so.n_sms = ds->n_sms;
   kc::Shape s{};
   kc::Layout lay{};
   kc::make_shape(so, L, n_reads, k, canonical, false, false, s, lay);
