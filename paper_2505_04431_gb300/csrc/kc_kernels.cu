@@ -50,6 +50,28 @@ namespace kc {
 
 typedef unsigned __int128 u128;
 
+// The kernels of a single count are launched so that each may be set up while the one before it
+// still runs (programmatic dependent launch); a kernel first waits for that one's end and its
+// writes.  12 launches 2 us apart were 4% of a count of 21 M bases (565 -> 546 us), 2% at 45 M
+// (1079 -> 1059).  Letting the next kernel's blocks onto the SMs early, before the last one's
+// have ended, cost more than it gave (50.9 -> 52.4 ms at 3 G bases), and so did this form for
+// the batched launches (32 small samples 932 -> 951 us), which stay as they are.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+static void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Batched launches: each block finds its count (one table load), copies the count's
 // descriptor to shared memory and runs the kernel body for that count.
 __device__ __forceinline__ void batch_locate(const BatchTab& t, BatchDesc& d_s, uint32_t& bid_s, uint32_t& nblk_s) {
@@ -285,7 +307,7 @@ __device__ __forceinline__ void prepare_body(const Shape& s, const Buffers& b, u
     if (lane == 0) b.tile_first[t] = lo;
   }
 }
-__global__ void __launch_bounds__(256) k_prepare(Shape s, Buffers b) { prepare_body(s, b, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(256) k_prepare(Shape s, Buffers b) { pdl_wait(); prepare_body(s, b, blockIdx.x, gridDim.x); }
 __global__ void __launch_bounds__(256) k_prepare_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
   prepare_body(d.s, d.b, bid, nblk);
@@ -826,6 +848,7 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
 }
 template <int KW, bool ONE, int VAR>
 __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count(Shape s, Buffers b) {
+  pdl_wait();
   pack_count_body<KW, ONE, VAR>(s, b, blockIdx.x, gridDim.x);
 }
 template <int KW, bool ONE, int VAR>
@@ -877,7 +900,7 @@ __device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b)
     if (NF > nf_max) atomicOr(&meta->status, ST_INTERNAL);
   }
 }
-__global__ void k_fine_plan(Shape s, Buffers b) { fine_plan_body(s, b); }
+__global__ void k_fine_plan(Shape s, Buffers b) { pdl_wait(); fine_plan_body(s, b); }
 __global__ void k_fine_plan_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
   fine_plan_body(d.s, d.b);
@@ -1050,11 +1073,13 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
 }
 template <int KW, int NT, int MODE, int VAR>
 __global__ void __launch_bounds__(NT, 3) k_scatter(Shape s, Buffers b) {
+  pdl_wait();
   scatter_body<KW, NT, MODE, VAR>(s, b, blockIdx.x);
 }
 // Aggregation ablation: pass B writes every key on its own through the partition cursors.
 template <int KW>
 __global__ void __launch_bounds__(256, 2) k_scatter_direct(Shape s, Buffers b) {
+  pdl_wait();
   scatter_body<KW, 256, SC_DIRECT, V_SHORT>(s, b, blockIdx.x);
 }
 
@@ -1196,6 +1221,7 @@ __device__ __forceinline__ void fine_hist_body(const Shape& s, const Buffers& b,
 }
 template <int KW>
 __global__ void __launch_bounds__(kFineThreads, 2) k_fine_hist(Shape s, Buffers b, int redo) {
+  pdl_wait();
   fine_hist_body<KW>(s, b, blockIdx.x, gridDim.x, redo != 0);
 }
 template <int KW>
@@ -1290,10 +1316,11 @@ __device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b
     if (sampled && carry_s > sh.cap_kb) b.meta->fine_spill = 1;
   }
 }
-__global__ void k_fine_scan(Shape sh, Buffers b, int redo) { fine_scan_body(sh, b, redo != 0); }
+__global__ void k_fine_scan(Shape sh, Buffers b, int redo) { pdl_wait(); fine_scan_body(sh, b, redo != 0); }
 
 // Before the exact fine split runs again (a sampled region overflowed): a fresh histogram.
 __global__ void k_fine_redo_clear(Shape sh, Buffers b) {
+  pdl_wait();
   if (!b.meta->fine_spill) return;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < sh.nf_max; i += (uint64_t)gridDim.x * blockDim.x)
     b.fhist[i] = 0;
@@ -1457,6 +1484,7 @@ __device__ __forceinline__ void fine_scatter_body(const Shape& s, const Buffers&
 }
 template <int KW>
 __global__ void __launch_bounds__(kFineThreads, 2) k_fine_scatter(Shape s, Buffers b, int redo) {
+  pdl_wait();
   fine_scatter_body<KW>(s, b, blockIdx.x, gridDim.x, redo != 0);
 }
 template <int KW>
@@ -2261,6 +2289,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
 }
 template <int KW, bool MERGE = false>
 __global__ void __launch_bounds__(kCountThreads, kCountBlocksPerSM) k_count_emit(Shape s, Buffers b) {
+  pdl_wait();
   count_emit_body<KW, MERGE>(s, b);
 }
 template <int KW>
@@ -2361,7 +2390,7 @@ __device__ __forceinline__ void scan_distinct_body(const Shape& sh, const Buffer
     if (dcarry_s != b.meta->n_deferred) atomicOr(&b.meta->status, ST_INTERNAL);
   }
 }
-__global__ void __launch_bounds__(1024) k_scan_distinct(Shape sh, Buffers b) { scan_distinct_body(sh, b); }
+__global__ void __launch_bounds__(1024) k_scan_distinct(Shape sh, Buffers b) { pdl_wait(); scan_distinct_body(sh, b); }
 __global__ void __launch_bounds__(1024) k_scan_distinct_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
   scan_distinct_body(d.s, d.b);
@@ -2433,6 +2462,7 @@ __device__ __forceinline__ void finish_one_body(const Shape& s, const Buffers& b
 }
 template <int KW>
 __global__ void __launch_bounds__(256) k_finish_one(Shape s, Buffers b) {
+  pdl_wait();
   finish_one_body<KW>(s, b, blockIdx.x, gridDim.x);
 }
 template <int KW>
@@ -2442,6 +2472,7 @@ __global__ void __launch_bounds__(256) k_finish_one_batch(BatchTab t) {
 }
 template <int KW>
 __global__ void __launch_bounds__(256) k_compact(Shape s, Buffers b) {
+  pdl_wait();
   compact_body<KW>(s, b, blockIdx.x, gridDim.x);
 }
 template <int KW>
@@ -2558,14 +2589,14 @@ int configure_kernels(int device) {
 int launch_phase1(const Shape& s, const Buffers& b, int n_sms, void* stream, const Marker& mark) {
   cudaStream_t st = (cudaStream_t)stream;
   int launches = 0;
-  k_prepare<<<prepare_blocks(s, (uint64_t)n_sms * 8), 256, 0, st>>>(s, b);
+  pdl_launch(k_prepare, prepare_blocks(s, (uint64_t)n_sms * 8), 256, 0, st, s, b);
   ++launches;
   KC_STEP("k_prepare");
   const unsigned gt = pack_blocks(s);
   const size_t smA = pack_smem(s);
 #define KC_PACK(KW, VAR)                                                                  \
-  if (s.one_level) k_pack_count<KW, true, VAR><<<gt, kPackThreads, smA, st>>>(s, b);      \
-  else k_pack_count<KW, false, VAR><<<gt, kPackThreads, smA, st>>>(s, b)
+  if (s.one_level) pdl_launch(k_pack_count<KW, true, VAR>, gt, kPackThreads, smA, st, s, b);      \
+  else pdl_launch(k_pack_count<KW, false, VAR>, gt, kPackThreads, smA, st, s, b)
   KC_PHASE1_VARIANT(s, KC_PACK);
 #undef KC_PACK
   ++launches;
@@ -2582,12 +2613,12 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     if (smB + kScatterStaticSmem > s.smem_budget) return -(int)cudaErrorInvalidConfiguration;
     const unsigned gt = (unsigned)s.n_tiles;
     if (s.aggr & kAggrNoSmemBuckets) {
-      if (s.kw == 1) k_scatter_direct<1><<<gt, 256, smB, st>>>(s, b);
-      else k_scatter_direct<2><<<gt, 256, smB, st>>>(s, b);
+      if (s.kw == 1) pdl_launch(k_scatter_direct<1>, gt, 256, smB, st, s, b);
+      else pdl_launch(k_scatter_direct<2>, gt, 256, smB, st, s, b);
     } else {
 #define KC_SCATTER(KW, VAR)                                                       \
-  if (s.one_level) k_scatter<KW, 256, SC_ONE, VAR><<<gt, 256, smB, st>>>(s, b);   \
-  else k_scatter<KW, 256, SC_COARSE, VAR><<<gt, 256, smB, st>>>(s, b)
+  if (s.one_level) pdl_launch(k_scatter<KW, 256, SC_ONE, VAR>, gt, 256, smB, st, s, b);   \
+  else pdl_launch(k_scatter<KW, 256, SC_COARSE, VAR>, gt, 256, smB, st, s, b)
       KC_PHASE1_VARIANT(s, KC_SCATTER);
 #undef KC_SCATTER
     }
@@ -2595,7 +2626,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     KC_STEP("k_scatter");
   }
   if (!s.one_level) {
-    k_fine_plan<<<1, 1024, (size_t)P1 * 8, st>>>(s, b);
+    pdl_launch(k_fine_plan, 1, 1024, (size_t)P1 * 8, st, s, b);
     ++launches;
     KC_STEP("k_fine_plan");
     const unsigned gf = (unsigned)(n_sms * 2);
@@ -2603,46 +2634,46 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     // whose kernels return at once unless a sampled region overflowed
     for (int redo = 0; redo <= (s.fine_sampled ? 1 : 0); ++redo) {
       if (redo) {
-        k_fine_redo_clear<<<(unsigned)n_sms, 1024, 0, st>>>(s, b);
+        pdl_launch(k_fine_redo_clear, (unsigned)n_sms, 1024, 0, st, s, b);
         ++launches;
         KC_STEP("k_fine_redo_clear");
       }
-      if (s.kw == 1) k_fine_hist<1><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
-      else k_fine_hist<2><<<gf, kFineThreads, fine_hist_smem(P1), st>>>(s, b, redo);
+      if (s.kw == 1) pdl_launch(k_fine_hist<1>, gf, kFineThreads, fine_hist_smem(P1), st, s, b, redo);
+      else pdl_launch(k_fine_hist<2>, gf, kFineThreads, fine_hist_smem(P1), st, s, b, redo);
       ++launches;
       KC_STEP(redo ? "k_fine_hist_redo" : "k_fine_hist");
-      k_fine_scan<<<1, 1024, 0, st>>>(s, b, redo);
+      pdl_launch(k_fine_scan, 1, 1024, 0, st, s, b, redo);
       ++launches;
       KC_STEP(redo ? "k_fine_scan_redo" : "k_fine_scan");
-      if (s.kw == 1) k_fine_scatter<1><<<gf, kFineThreads, fine_scatter_smem(1, P1), st>>>(s, b, redo);
-      else k_fine_scatter<2><<<gf, kFineThreads, fine_scatter_smem(2, P1), st>>>(s, b, redo);
+      if (s.kw == 1) pdl_launch(k_fine_scatter<1>, gf, kFineThreads, fine_scatter_smem(1, P1), st, s, b, redo);
+      else pdl_launch(k_fine_scatter<2>, gf, kFineThreads, fine_scatter_smem(2, P1), st, s, b, redo);
       ++launches;
       KC_STEP(redo ? "k_fine_scatter_redo" : "k_fine_scatter");
     }
   }
   const size_t smC = count_kernel_smem(s.kw, s.bT_max, s.tail);
   if (s.aggr & kAggrWarpMerge) {
-    if (s.kw == 1) k_count_emit<1, true><<<(unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st>>>(s, b);
-    else k_count_emit<2, true><<<(unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st>>>(s, b);
+    if (s.kw == 1) pdl_launch(k_count_emit<1, true>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
+    else pdl_launch(k_count_emit<2, true>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
   } else if (s.kw == 1) {
-    k_count_emit<1><<<(unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st>>>(s, b);
+    pdl_launch(k_count_emit<1>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
   } else {
-    k_count_emit<2><<<(unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st>>>(s, b);
+    pdl_launch(k_count_emit<2>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
   }
   ++launches;
   KC_STEP("k_count_emit");
   if (s.one_level) {
-    if (s.kw == 1) k_finish_one<1><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
-    else k_finish_one<2><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
+    if (s.kw == 1) pdl_launch(k_finish_one<1>, compact_blocks(s, n_sms), 256, 0, st, s, b);
+    else pdl_launch(k_finish_one<2>, compact_blocks(s, n_sms), 256, 0, st, s, b);
     ++launches;
     KC_STEP("k_finish_one");
     return launches;
   }
-  k_scan_distinct<<<1, 1024, 0, st>>>(s, b);
+  pdl_launch(k_scan_distinct, 1, 1024, 0, st, s, b);
   ++launches;
   KC_STEP("k_scan_distinct");
-  if (s.kw == 1) k_compact<1><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
-  else k_compact<2><<<compact_blocks(s, n_sms), 256, 0, st>>>(s, b);
+  if (s.kw == 1) pdl_launch(k_compact<1>, compact_blocks(s, n_sms), 256, 0, st, s, b);
+  else pdl_launch(k_compact<2>, compact_blocks(s, n_sms), 256, 0, st, s, b);
   ++launches;
   KC_STEP("k_compact");
   return launches;
