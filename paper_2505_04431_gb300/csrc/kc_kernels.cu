@@ -857,53 +857,45 @@ __global__ void __launch_bounds__(kPackThreads, KW == 1 ? 4 : 2) k_pack_count_ba
   pack_count_body<KW, ONE, VAR>(d.s, d.b, bid, nblk);
 }
 
-// Fine split of every coarse partition, after pass B: the distinct-key estimate (a sampled
-// HyperLogLog filled by pass B) gives the duplication factor K / D, and a fine partition
-// aims at fine_target distinct keys, i.e. fine_target * K / D keys.  One block.
-__device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b) {
-  const uint64_t* cstart = b.cstart;
-  uint32_t *fine_base = b.fine_base, *fine_m = b.fine_m, *flo = b.flo;
-  const int P1 = 1 << s.b1, b1 = s.b1;
-  const uint32_t nf_max = (uint32_t)s.nf_max;
-  Meta* meta = b.meta;
-  extern __shared__ uint64_t fsc[];  // [P1]
-  __shared__ uint64_t wt[32];
-  const double target = sketch_target(b.hll, cstart[P1], s, P1, meta);
-  for (int c = threadIdx.x; c < P1; c += blockDim.x) {
-    const uint64_t n = cstart[c + 1] - cstart[c];
-    uint64_t m = (uint64_t)ceil((double)n / target);
-    m = m < 1 ? 1 : (m > (uint64_t)kMaxFine ? (uint64_t)kMaxFine : m);
-    fine_m[c] = (uint32_t)m;
-    fsc[c] = m;
-  }
+// Fine split of every coarse partition, after pass B: the distinct-key estimate (filled by pass
+// B) gives the keys a fine partition aims at, and coarse partition c is cut into
+// m_c = ceil(n_c / target).  One block per coarse partition; each finds the number of fine
+// partitions before its own for itself (a block of one launch for all took 98 us for 100 K
+// fine partitions and 219 us for 221 K, this takes 9 and 11).
+__device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b, uint32_t c) {
+  extern __shared__ uint32_t fsc[];  // [padded P1]
+  __shared__ uint32_t wt[32];
+  const int P1 = 1 << s.b1;
+  const uint32_t T = (uint32_t)ceil(sketch_target(b.hll, b.cstart[P1], s, P1, b.meta));
+  auto parts = [&](uint64_t n) -> uint32_t {  // (n is below 2^32)
+    const uint32_t m = n ? ((uint32_t)n - 1) / T + 1 : 1;
+    return m < (uint32_t)kMaxFine ? m : (uint32_t)kMaxFine;
+  };
+  for (int i = threadIdx.x; i < P1; i += blockDim.x) fsc[PAD(i)] = parts(b.cstart[i + 1] - b.cstart[i]);
   __syncthreads();
-  const uint64_t NF = block_exclusive_scan<uint64_t>(fsc, P1, wt);
-  for (int c = threadIdx.x; c < P1; c += blockDim.x) fine_base[c] = (uint32_t)fsc[c];
-  // fine partition g = fsc[c] + f holds the values u of coarse field c whose low part
-  // v = u mod 2^(32 - b1) has floor(v m / 2^(32 - b1)) = f, i.e. v >= ceil(f 2^(32 - b1) / m);
-  // one thread per fine partition, its coarse partition found by binary search in fsc
-  const uint64_t w = 1ull << (32 - b1);
-  for (uint64_t g = threadIdx.x; g < NF && g < nf_max; g += blockDim.x) {
-    int lo = 0, hi = P1 - 1;  // last c with fsc[c] <= g
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (fsc[mid] <= g) lo = mid;
-      else hi = mid - 1;
-    }
-    const uint64_t m = fine_m[lo], f = g - fsc[lo];
-    flo[g] = (uint32_t)((uint64_t)lo << (32 - b1)) + (uint32_t)((f * w + m - 1) / m);
-  }
+  const uint32_t NF = block_exclusive_scan_pad<uint32_t>(fsc, P1, wt);
+  const uint32_t base = fsc[PAD(c)], nf_max = (uint32_t)s.nf_max;
+  const uint64_t m = parts(b.cstart[c + 1] - b.cstart[c]);
+  // fine partition f of c holds the values u of coarse field c whose low part v = u mod
+  // 2^(32 - b1) has floor(v m / 2^(32 - b1)) = f, i.e. v >= ceil(f 2^(32 - b1) / m)
+  const uint64_t w = 1ull << (32 - s.b1);
+  for (uint64_t f = threadIdx.x; f < m && base + f < nf_max; f += blockDim.x)
+    b.flo[base + f] = (uint32_t)((uint64_t)c << (32 - s.b1)) + (uint32_t)((f * w + m - 1) / m);
   if (threadIdx.x == 0) {
-    if (NF <= nf_max) flo[NF] = 0;  // so that the last partition ends at u = 2^32 - 1
-    fine_base[P1] = (uint32_t)NF;
-    meta->n_fine = NF <= nf_max ? NF : 0;  // later kernels never index past nf_max
-    if (NF > nf_max) atomicOr(&meta->status, ST_INTERNAL);
+    b.fine_base[c] = base;
+    b.fine_m[c] = (uint32_t)m;
+    if ((int)c == P1 - 1) {
+      if (NF <= nf_max) b.flo[NF] = 0;  // so that the last partition ends at u = 2^32 - 1
+      b.fine_base[P1] = NF;
+      b.meta->n_fine = NF <= nf_max ? NF : 0;  // later kernels never index past nf_max
+      if (NF > nf_max) atomicOr(&b.meta->status, ST_INTERNAL);
+    }
   }
 }
-__global__ void k_fine_plan(Shape s, Buffers b) { pdl_wait(); fine_plan_body(s, b); }
-__global__ void k_fine_plan_batch(BatchTab t) {
+__global__ void __launch_bounds__(256) k_fine_plan(Shape s, Buffers b) { pdl_wait(); fine_plan_body(s, b, blockIdx.x); }
+__global__ void __launch_bounds__(256) k_fine_plan_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  fine_plan_body(d.s, d.b);
+  fine_plan_body(d.s, d.b, bid);
 }
 
 // ------------------------------------------------------------------ pass B
@@ -1238,14 +1230,12 @@ __device__ __forceinline__ uint64_t sampled_below(uint64_t x) {
   return (x / per) * kFineChunk + (r < (uint64_t)kFineChunk ? r : (uint64_t)kFineChunk);
 }
 
-// Region of fine partition g in a sampled layout: its estimated size (its sampled count
-// scaled by its coarse partition's keys over that partition's sampled keys) plus 5.5
-// standard deviations of that estimate and 16 keys; never more than its coarse partition.
-// Too small a sample gives the whole coarse partition.
-__device__ __forceinline__ uint64_t fine_region(const Shape& sh, const Buffers& b, uint64_t g) {
-  const uint32_t c = sh.b1 ? b.flo[g] >> (32 - sh.b1) : 0u;
-  const uint64_t a = b.cstart[c], e = b.cstart[c + 1];
-  const uint64_t n_c = e - a, s_c = sampled_below(e) - sampled_below(a);
+// Region of fine partition g of coarse partition c in a sampled layout: its estimated size (its
+// sampled count scaled by c's n_c keys over its s_c sampled keys) plus 5.5 standard deviations
+// of that estimate and 16 keys; never more than its coarse partition.  Too small a sample
+// gives the whole coarse partition.
+__device__ __forceinline__ uint64_t fine_region(const Shape& sh, const Buffers& b, uint64_t g, uint64_t n_c,
+                                                uint64_t s_c, uint32_t m_c) {
   if (s_c < 1024) return n_c;
   const float f = (float)n_c / (float)s_c, cnt = (float)b.fhist[g];
   float slack = sh.tight_slack ? 0.f : 5.5f * f * sqrtf(cnt + 1.f) + 16.f;
@@ -1253,70 +1243,80 @@ __device__ __forceinline__ uint64_t fine_region(const Shape& sh, const Buffers& 
   // come many at a time (a read inside an array holds each of them 20 times and more), so its
   // sampled count varies more than a random sample's: an eighth on top.  (Without it, 72 M
   // windows with 3% satellite arrays took the exact split again in most counts, 225 to 350 us.)
-  if (!sh.tight_slack && cnt * (float)b.fine_m[c] > 4.f * (float)s_c) slack += 0.125f * f * cnt;
+  if (!sh.tight_slack && cnt * (float)m_c > 4.f * (float)s_c) slack += 0.125f * f * cnt;
   const uint64_t r = (uint64_t)(cnt * f + slack) + (sh.tight_slack ? 0 : 1);
   return r < n_c ? r : n_c;
 }
+// Room of a coarse partition in a sampled layout: its keys, a quarter and 64 per fine
+// partition; as much as its regions take where the sample is too small.
+__device__ __forceinline__ uint64_t coarse_room(uint64_t n_c, uint64_t s_c, uint32_t m_c) {
+  return s_c < 1024 ? n_c * m_c : n_c + n_c / 4 + 64ull * m_c;
+}
 
-// Exclusive scan of the fine partitions' sizes (exact histogram) or regions (sampled
-// layout) into their starts (one block of 1024 threads).  A sampled layout that does not fit
-// the keys arrays is given up at once (the exact split follows).
-__device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b, bool redo = false) {
+// Starts of the fine partitions of coarse partition c: an exclusive scan of their sizes (exact
+// histogram) from c's own start, or of their regions (sampled layout) from the end of the room
+// of the coarse partitions before.  One block of 256 threads per coarse partition (one block
+// for all took 203 us for 100 K fine partitions and 430 us for 221 K, this takes 10 and 12).
+// Regions that pass their coarse partition's room, or rooms that pass the keys arrays, are
+// given up at once (the exact split follows).
+__device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b, uint32_t c, bool redo = false) {
   __shared__ uint64_t wt[32];
-  __shared__ uint64_t carry_s;
   if (redo && !b.meta->fine_spill) return;
   const bool sampled = sh.fine_sampled && !redo;
+  const int P1 = 1 << sh.b1, t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
   const uint64_t NF = min(b.meta->n_fine, sh.nf_max);
-  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wid = t >> 5;
-  if (t == 0) carry_s = 0;
-  __syncthreads();
-  for (uint64_t base = 0; base < NF; base += (uint64_t)nt * 8) {
-    uint64_t v[8];
-    uint64_t s = 0;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const uint64_t i = base + (uint64_t)t * 8 + m;
-      v[m] = i < NF ? (sampled ? fine_region(sh, b, i) : (uint64_t)b.fhist[i]) : 0;
-      s += v[m];
-    }
-    uint64_t x = s;
+  const uint64_t g0 = b.fine_base[c];
+  const uint32_t m = b.fine_m[c];
+  if (g0 + m > NF) return;  // (a plan that failed)
+  auto block_sum = [&](uint64_t x, uint64_t& before) -> uint64_t {  // the total; `before`: of the threads before
+    uint64_t y = x;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t y = __shfl_up_sync(0xffffffffu, x, d);
-      if (lane >= d) x += y;
-    }
-    if (lane == 31) wt[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      uint64_t w = wt[lane];
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xffffffffu, w, d);
-        if (lane >= d) w += y;
-      }
-      wt[lane] = w;
+      const uint64_t z = __shfl_up_sync(0xffffffffu, y, d);
+      if (lane >= d) y += z;
     }
     __syncthreads();
-    uint64_t run = carry_s + x - s + (wid ? wt[wid - 1] : 0);
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const uint64_t i = base + (uint64_t)t * 8 + m;
-      if (i < NF) {
-        b.foff[i] = run;
-        b.fcur[i] = run;
-      }
-      run += v[m];
+    if (lane == 31) wt[wid] = y;
+    __syncthreads();
+    uint64_t total = 0, prev = 0;
+    for (int w = 0; w < nw; ++w) {
+      if (w < wid) prev += wt[w];
+      total += wt[w];
     }
-    __syncthreads();
-    if (t == 0) carry_s += wt[31];
-    __syncthreads();
+    before = prev + y - x;
+    return total;
+  };
+  const uint64_t a = b.cstart[c], e = b.cstart[c + 1], n_c = e - a, s_c = sampled_below(e) - sampled_below(a);
+  uint64_t base = a, room = n_c, skip;
+  if (sampled) {
+    uint64_t x = 0;
+    for (uint32_t i = t; i < c; i += blockDim.x) {
+      const uint64_t p = b.cstart[i], q = b.cstart[i + 1];
+      x += coarse_room(q - p, sampled_below(q) - sampled_below(p), b.fine_m[i]);
+    }
+    base = block_sum(x, skip);
+    room = coarse_room(n_c, s_c, m);
+  }
+  const uint32_t per = (m + blockDim.x - 1) / blockDim.x, lo = min(m, t * per), hi = min(m, lo + per);
+  uint64_t sum = 0, run;
+  for (uint32_t i = lo; i < hi; ++i)
+    sum += sampled ? fine_region(sh, b, g0 + i, n_c, s_c, m) : (uint64_t)b.fhist[g0 + i];
+  const uint64_t total = block_sum(sum, run);
+  run += base;
+  for (uint32_t i = lo; i < hi; ++i) {
+    b.foff[g0 + i] = run;
+    b.fcur[g0 + i] = run;
+    run += sampled ? fine_region(sh, b, g0 + i, n_c, s_c, m) : (uint64_t)b.fhist[g0 + i];
   }
   if (t == 0) {
-    b.foff[NF] = carry_s;
-    if (sampled && carry_s > sh.cap_kb) b.meta->fine_spill = 1;
+    if ((int)c == P1 - 1) b.foff[NF] = base + room;
+    if (sampled && (total > room || base + room > sh.cap_kb)) b.meta->fine_spill = 1;
   }
 }
-__global__ void k_fine_scan(Shape sh, Buffers b, int redo) { pdl_wait(); fine_scan_body(sh, b, redo != 0); }
+__global__ void __launch_bounds__(256) k_fine_scan(Shape sh, Buffers b, int redo) {
+  pdl_wait();
+  fine_scan_body(sh, b, blockIdx.x, redo != 0);
+}
 
 // Before the exact fine split runs again (a sampled region overflowed): a fresh histogram.
 __global__ void k_fine_redo_clear(Shape sh, Buffers b) {
@@ -1325,15 +1325,15 @@ __global__ void k_fine_redo_clear(Shape sh, Buffers b) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < sh.nf_max; i += (uint64_t)gridDim.x * blockDim.x)
     b.fhist[i] = 0;
 }
-__global__ void k_fine_scan_batch(BatchTab t, int redo) {
+__global__ void __launch_bounds__(256) k_fine_scan_batch(BatchTab t, int redo) {
   KC_BATCH_PROLOGUE(t);
-  fine_scan_body(d.s, d.b, redo != 0);
+  fine_scan_body(d.s, d.b, bid, redo != 0);
 }
-// (the fine scan's table: one block per count)
+// (the fine scan's table: one block per coarse partition)
 __global__ void k_fine_redo_clear_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
   if (!d.b.meta->fine_spill) return;
-  for (uint64_t i = threadIdx.x; i < d.s.nf_max; i += blockDim.x) d.b.fhist[i] = 0;
+  for (uint64_t i = bid * (uint64_t)blockDim.x + threadIdx.x; i < d.s.nf_max; i += (uint64_t)nblk * blockDim.x) d.b.fhist[i] = 0;
 }
 
 // Exclusive scan of in[0, n) into out[0, n) (all threads of the block, n <= 4 * blockDim);
@@ -2299,101 +2299,101 @@ __global__ void __launch_bounds__(kCountThreads, kCountBlocksPerSM) k_count_emit
 }
 
 // ------------------------------------------------------------------ final: offsets of the runs
-// Exclusive scan of the distinct counts of the fine partitions (one block of 1024
-// threads): fcur[g] = first output position of partition g, n_distinct = the total.  The
-// look-back words are checked against it, and the deferred partitions are listed (in
-// increasing order) at the front of the spent look-back array for k_compact.
-__device__ __forceinline__ void scan_distinct_body(const Shape& sh, const Buffers& b) {
+// Exclusive scan of the distinct counts of the fine partitions: fcur[g] = first output position
+// of partition g, n_distinct = the total.  The look-back words are checked against it, and the
+// deferred partitions are listed in flo (dead by now) for k_compact.  Every block adds up the
+// counts before its own share for itself (they are read from L2; one block for all took 139 us
+// for 100 K partitions and 214 us for 221 K, this takes 18 and 27).
+__device__ __forceinline__ void scan_distinct_body(const Shape& sh, const Buffers& b, uint32_t bid, uint32_t nblk) {
   __shared__ uint64_t wt[32];
   __shared__ uint32_t wd[32];
-  __shared__ uint64_t carry_s;
-  __shared__ uint32_t dcarry_s;
   const uint64_t NF = min(b.meta->n_fine, sh.nf_max);
-  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wid = t >> 5;
-  if (t == 0) {
-    carry_s = 0;
-    dcarry_s = 0;
-  }
-  __syncthreads();
-  bool bad = false;
-  for (uint64_t base = 0; base < NF; base += (uint64_t)nt * 8) {
-    uint32_t v[8];
-    unsigned long long lk[8];
-    uint64_t s = 0;
-    uint32_t nd = 0;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const uint64_t i = base + (uint64_t)t * 8 + m;
-      v[m] = i < NF ? b.fhist[i] : 0;
-      lk[m] = i < NF ? ld_status(&b.look[i]) : 0;
-      s += v[m] & 0x7fffffffu;
-      nd += v[m] >> 31;
-    }
-    uint64_t x = s;
-    uint32_t y = nd;
+  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wid = t >> 5, nw = nt >> 5;
+  const uint64_t share = (NF + nblk - 1) / nblk, start = min(NF, bid * share), end = min(NF, start + share);
+  // sums over the block of (distinct, deferred), and the sums of the threads before
+  auto block_sum = [&](uint64_t& x, uint32_t& y, uint64_t& before_x, uint32_t& before_y) {
+    uint64_t p = x;
+    uint32_t q = y;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t xs = __shfl_up_sync(0xffffffffu, x, d);
-      const uint32_t ys = __shfl_up_sync(0xffffffffu, y, d);
+      const uint64_t xs = __shfl_up_sync(0xffffffffu, p, d);
+      const uint32_t ys = __shfl_up_sync(0xffffffffu, q, d);
       if (lane >= d) {
-        x += xs;
-        y += ys;
+        p += xs;
+        q += ys;
       }
     }
+    __syncthreads();
     if (lane == 31) {
-      wt[wid] = x;
-      wd[wid] = y;
+      wt[wid] = p;
+      wd[wid] = q;
     }
-    __syncthreads();  // also: every look-back word of this chunk has been read
-    if (wid == 0) {
-      uint64_t w = wt[lane];
-      uint32_t z = wd[lane];
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint64_t ws = __shfl_up_sync(0xffffffffu, w, d);
-        const uint32_t zs = __shfl_up_sync(0xffffffffu, z, d);
-        if (lane >= d) {
-          w += ws;
-          z += zs;
-        }
+    __syncthreads();
+    before_x = p - x;
+    before_y = q - y;
+    x = y = 0;
+    for (int w = 0; w < nw; ++w) {
+      if (w < wid) {
+        before_x += wt[w];
+        before_y += wd[w];
       }
-      wt[lane] = w;
-      wd[lane] = z;
+      x += wt[w];
+      y += wd[w];
     }
-    __syncthreads();
-    uint64_t run = carry_s + x - s + (wid ? wt[wid - 1] : 0);
-    uint32_t drun = dcarry_s + y - nd + (wid ? wd[wid - 1] : 0);
+  };
+  uint64_t carry = 0, skip_x;
+  uint32_t dcarry = 0, skip_y;
+  // the partitions before the share, four 16-byte loads in flight per thread
+  const uint4* f4 = reinterpret_cast<const uint4*>(b.fhist);
+  for (uint64_t i = t; i < start / 4; i += 4ull * nt) {
+    uint4 v[4];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const uint64_t i = base + (uint64_t)t * 8 + m;
-      if (i < NF) {
-        const uint64_t d = v[m] & 0x7fffffffu;
-        const bool deferred = v[m] >> 31;
-        // a direct partition published its inclusive prefix, a deferred one its count
-        const uint64_t want = deferred ? (kLookAgg | d) : (kLookIncl | (run + d));
-        bad |= lk[m] != want;
-        b.fcur[i] = run;
-        if (deferred) b.look[drun++] = i;
-        run += d;
-      }
+    for (int m = 0; m < 4; ++m) v[m] = i + (uint64_t)m * nt < start / 4 ? f4[i + (uint64_t)m * nt] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      carry += (uint64_t)(v[m].x & 0x7fffffffu) + (v[m].y & 0x7fffffffu) + (v[m].z & 0x7fffffffu) + (v[m].w & 0x7fffffffu);
+      dcarry += (v[m].x >> 31) + (v[m].y >> 31) + (v[m].z >> 31) + (v[m].w >> 31);
     }
-    __syncthreads();
-    if (t == 0) {
-      carry_s += wt[31];
-      dcarry_s += wd[31];
-    }
-    __syncthreads();
+  }
+  if (t < (int)(start & 3)) {  // an empty share after the last partition starts anywhere
+    const uint32_t v = b.fhist[(start & ~3ull) + t];
+    carry += v & 0x7fffffffu;
+    dcarry += v >> 31;
+  }
+  block_sum(carry, dcarry, skip_x, skip_y);
+  const uint64_t per = (end - start + nt - 1) / nt, lo = min(end, start + t * per), hi = min(end, lo + per);
+  uint64_t s = 0, run;
+  uint32_t nd = 0, drun;
+  for (uint64_t i = lo; i < hi; ++i) {
+    s += b.fhist[i] & 0x7fffffffu;
+    nd += b.fhist[i] >> 31;
+  }
+  block_sum(s, nd, run, drun);
+  run += carry;
+  drun += dcarry;
+  bool bad = false;
+  for (uint64_t i = lo; i < hi; ++i) {
+    const uint64_t d = b.fhist[i] & 0x7fffffffu;
+    const bool deferred = b.fhist[i] >> 31;
+    // a direct partition published its inclusive prefix, a deferred one its count
+    bad |= ld_status(&b.look[i]) != (deferred ? (kLookAgg | d) : (kLookIncl | (run + d)));
+    b.fcur[i] = run;
+    if (deferred) b.flo[drun++] = (uint32_t)i;
+    run += d;
   }
   if (bad) atomicOr(&b.meta->status, ST_INTERNAL);
-  if (t == 0) {
-    b.meta->n_distinct = carry_s;
-    if (dcarry_s != b.meta->n_deferred) atomicOr(&b.meta->status, ST_INTERNAL);
+  if (bid == nblk - 1 && t == 0) {
+    b.meta->n_distinct = carry + s;
+    if (dcarry + nd != b.meta->n_deferred) atomicOr(&b.meta->status, ST_INTERNAL);
   }
 }
-__global__ void __launch_bounds__(1024) k_scan_distinct(Shape sh, Buffers b) { pdl_wait(); scan_distinct_body(sh, b); }
+__global__ void __launch_bounds__(1024) k_scan_distinct(Shape sh, Buffers b) {
+  pdl_wait();
+  scan_distinct_body(sh, b, blockIdx.x, gridDim.x);
+}
 __global__ void __launch_bounds__(1024) k_scan_distinct_batch(BatchTab t) {
   KC_BATCH_PROLOGUE(t);
-  scan_distinct_body(d.s, d.b);
+  scan_distinct_body(d.s, d.b, bid, nblk);
 }
 
 // Move the runs of the deferred fine partitions from their input regions (keys in sbuf,
@@ -2418,7 +2418,7 @@ __device__ __forceinline__ void compact_body(const Shape& s, const Buffers& b, u
   check_offsets(s, b, bid, nblk);
   const uint64_t n_def = min(b.meta->n_deferred, s.nf_max);
   for (uint64_t q = bid; q < n_def; q += nblk) {
-    const uint64_t g = b.look[q];
+    const uint64_t g = b.flo[q];
     if (g >= min(b.meta->n_fine, s.nf_max)) {
       if (threadIdx.x == 0) atomicOr(&b.meta->status, ST_INTERNAL);
       continue;
@@ -2497,6 +2497,11 @@ static uint32_t prepare_blocks(const Shape& s, uint64_t most) {
 // pass A: one block per tile (one-level: at most one wave, 4 blocks on 152 SMs)
 static uint32_t pack_blocks(const Shape& s) {
   return (uint32_t)std::max<uint64_t>(1, s.one_level ? std::min<uint64_t>(s.n_tiles, 608) : s.n_tiles);
+}
+// the scan of the distinct counts: a share of about 4096 fine partitions each
+static uint32_t scan_blocks(const Shape& s) {
+  const uint64_t want = s.nf_max / 4096 + 1;
+  return (uint32_t)(want < 128 ? want : 128);
 }
 // the last kernel: deferred runs to move (at most one per fine partition), offsets to check
 static uint32_t compact_blocks(const Shape& s, int n_sms) {
@@ -2626,7 +2631,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     KC_STEP("k_scatter");
   }
   if (!s.one_level) {
-    pdl_launch(k_fine_plan, 1, 1024, (size_t)P1 * 8, st, s, b);
+    pdl_launch(k_fine_plan, P1, 256, padded_len(P1) * 4, st, s, b);
     ++launches;
     KC_STEP("k_fine_plan");
     const unsigned gf = (unsigned)(n_sms * 2);
@@ -2642,7 +2647,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
       else pdl_launch(k_fine_hist<2>, gf, kFineThreads, fine_hist_smem(P1), st, s, b, redo);
       ++launches;
       KC_STEP(redo ? "k_fine_hist_redo" : "k_fine_hist");
-      pdl_launch(k_fine_scan, 1, 1024, 0, st, s, b, redo);
+      pdl_launch(k_fine_scan, P1, 256, 0, st, s, b, redo);
       ++launches;
       KC_STEP(redo ? "k_fine_scan_redo" : "k_fine_scan");
       if (s.kw == 1) pdl_launch(k_fine_scatter<1>, gf, kFineThreads, fine_scatter_smem(1, P1), st, s, b, redo);
@@ -2669,7 +2674,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     KC_STEP("k_finish_one");
     return launches;
   }
-  pdl_launch(k_scan_distinct, 1, 1024, 0, st, s, b);
+  pdl_launch(k_scan_distinct, scan_blocks(s), 1024, 0, st, s, b);
   ++launches;
   KC_STEP("k_scan_distinct");
   if (s.kw == 1) pdl_launch(k_compact<1>, compact_blocks(s, n_sms), 256, 0, st, s, b);
@@ -2689,14 +2694,14 @@ uint32_t batch_blocks(BatchKernel k, const Shape& s, int n_sms, uint64_t bases_t
     case BK_SCATTER: return s.one_level ? 0u : (uint32_t)s.n_tiles;
     case BK_SCATTER_ONE: return s.one_level ? (uint32_t)s.n_tiles : 0u;
     case BK_FINE_PLAN:
-    case BK_FINE_SCAN: return s.one_level ? 0u : 1u;
+    case BK_FINE_SCAN: return s.one_level ? 0u : 1u << s.b1;
     case BK_FINE_HIST:
     case BK_FINE_SCATTER: return s.one_level ? 0u : clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
     case BK_COUNT: {
       const double share = bases_total ? (double)s.L / (double)bases_total : 1.0;
       return clampu((uint64_t)(2.0 * (double)nsm * share + 0.999), 1, nsm * kCountBlocksPerSM);
     }
-    case BK_SCAN_DISTINCT: return s.one_level ? 0u : 1u;
+    case BK_SCAN_DISTINCT: return s.one_level ? 0u : scan_blocks(s);
     case BK_COMPACT: return s.one_level ? 0u : compact_blocks(s, n_sms);
     case BK_FINISH_ONE: return s.one_level ? compact_blocks(s, n_sms) : 0u;
     default: return 1u;
@@ -2740,7 +2745,7 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
              "k_scatter")
   KC_PHASE1_VARIANT(s0, KC_PHASE1);  // (all counts of a batch have the same k and mode)
 #undef KC_PHASE1
-  KC_BLAUNCH(BK_FINE_PLAN, (k_fine_plan_batch<<<bp.grid[BK_FINE_PLAN], 1024, (size_t)P1 * 8, st>>>(tab(BK_FINE_PLAN))),
+  KC_BLAUNCH(BK_FINE_PLAN, (k_fine_plan_batch<<<bp.grid[BK_FINE_PLAN], 256, padded_len(P1) * 4, st>>>(tab(BK_FINE_PLAN))),
              "k_fine_plan");
   // the fine split; then, for counts with a sampled layout, the exact split again (each
   // count's blocks return at once unless its sampled regions overflowed)
@@ -2759,7 +2764,7 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
                      tab(BK_FINE_HIST), redo)),
                  redo ? "k_fine_hist_redo" : "k_fine_hist");
     }
-    KC_BLAUNCH(BK_FINE_SCAN, (k_fine_scan_batch<<<bp.grid[BK_FINE_SCAN], 1024, 0, st>>>(tab(BK_FINE_SCAN), redo)),
+    KC_BLAUNCH(BK_FINE_SCAN, (k_fine_scan_batch<<<bp.grid[BK_FINE_SCAN], 256, 0, st>>>(tab(BK_FINE_SCAN), redo)),
                redo ? "k_fine_scan_redo" : "k_fine_scan");
     if (bp.kw == 1) {
       KC_BLAUNCH(BK_FINE_SCATTER,

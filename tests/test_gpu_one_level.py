@@ -69,3 +69,24 @@ def test_one_level_uneven_bins(torch_cuda, counters, k):
     offsets = np.arange(0, len(reads) + 1, k, dtype=np.uint64)
     check(torch_cuda, counters, reads, offsets, k, False)
     assert counters["one"].stats()["n_overflow_fine"] > 0
+
+
+# Two-level counts: the plan and the scans take one block per coarse partition, and the scan of
+# the distinct counts one per 4096 possible fine partitions (of which repeats leave few)
+@pytest.mark.parametrize("hint,slots,genome", [(1, 64, 700), (2, 64, 5000), (64, 64, 60_000), (4096, 0, 3000)])
+def test_two_level_plan_and_scans(torch_cuda, hint, slots, genome):
+    from paper_2505_04431_gb300 import KmerCounter
+    rng = np.random.default_rng(hint + genome)
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    g = acgt[rng.integers(0, 4, genome)]
+    starts = rng.integers(0, genome - 100, 6000)
+    reads = np.ascontiguousarray(g[starts[:, None] + np.arange(100)]).reshape(-1)
+    offsets = np.arange(0, len(reads) + 1, 100, dtype=np.uint64)
+    want_k, want_c, _ = oracle.count(reads, offsets, 31, True)
+    for kw in ({}, {"defer_all": True}, {"test_fine_sampled": True}):
+        c = KmerCounter(n_partitions_hint=hint, table_slots_max=slots, **kw)
+        res = c.count(torch_cuda.from_numpy(reads).cuda(), torch_cuda.from_numpy(offsets.view(np.int64)).cuda(), 31, True)
+        keys, counts = res.to_numpy()
+        res.free()
+        c.close()
+        assert np.array_equal(keys, want_k) and np.array_equal(counts, want_c), kw
