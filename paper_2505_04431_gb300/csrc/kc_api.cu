@@ -107,9 +107,20 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   // small that there would be more fine partitions than pass B stages in shared memory.
   s.one_level = L > 0 && b1 == 0 && !o.p_hint && !o.force_sampled && !(o.aggr & kAggrNoSmemBuckets) &&
                 s.nf_max <= kOneLevelFine;
+  // Up to 48 Mi bases of 64-bit keys, repeats may leave as few fine partitions: pass A counts
+  // bins and fills the sketch for these too, and its last block takes one level if at most
+  // kEitherFine partitions come out (45 M bases of a 30x genome: 1824; kernels 867 -> 747 us, 21 M
+  // bases 447 -> 379), two if not (20 M bases of noisy long reads: 830 -> 895 us, the price of
+  // having looked).
+  // (128-bit keys: 20 M bases 567 -> 534 us, but 25 M of noisy long reads, which take two levels
+  // after all, 1476 -> 1565: they stay with two.)
+  if (!s.one_level && b1 > 0 && s.kw == 1 && L < kEitherBases && !o.p_hint && !o.force_sampled &&
+      !(o.aggr & kAggrNoSmemBuckets))
+    s.one_level = kEitherLevel;
   // bins of at most 5/8 of a fine partition, even if every base starts a distinct key: a
   // partition takes its target and up to a bin more, within the 3/4 load a table is ordered with
   s.bb = std::min(kMaxBinsLog2, std::max(kMinBinsLog2, ceil_log2_u64(8 * s.cap / (5 * s.fine_target) + 1)));
+  if (s.one_level == kEitherLevel) s.bb = kMaxBinsLog2;
   // a sampled fine layout: regions hold their estimate plus slack (about a fifth of the keys
   // in all, and at least 16 keys each); a layout that does not fit falls back to the exact one
   s.fine_sampled = o.allow_sampled && (o.force_sampled || L >= kFineSampledMinBases) ? 1 : 0;
@@ -132,9 +143,10 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.reads = take(copy_reads ? L + 16 : 0);
   lay.offs = take(copy_offs ? (n_reads + 1) * 8 : 0);
   // flo of the two-level path is written after pass B has read the codes
-  lay.codes = take(std::max<uint64_t>(s.n_words * 8, s.one_level ? 0 : (nf + 1) * 4));
+  const bool one = s.one_level == kOneLevel, either = s.one_level == kEitherLevel;
+  lay.codes = take(std::max<uint64_t>(s.n_words * 8, one ? 0 : (nf + 1) * 4));
   lay.inv = take(s.n_words * 4);
-  const uint64_t bins = s.one_level ? 1ull << s.bb : 0;
+  const uint64_t bins = one ? 1ull << s.bb : 0;
   lay.cst = take(std::max<uint64_t>((P1 + 1) * 8, bins * 4));
   lay.bmap = take(bins * 2);
   lay.fb = take((P1 + 1) * 4);
@@ -142,19 +154,28 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   lay.hll = take((size_t)kHllRegs * 4);
   lay.fh = take(nf * 4);
   lay.fo = take((nf + 1) * 8);
-  lay.flo = s.one_level ? take((nf + 1) * 4) : lay.codes;
+  lay.flo = one ? take((nf + 1) * 4) : lay.codes;
   lay.fc = take(nf * 8);
   lay.look = take(nf * 8);
   // one-level: no coarse-grouped keys, only the counts of deferred runs
   // Phase 1's tables lie in the memory of the keys array that it does not write: each tile's
   // first read in kbuf (one-level) or sbuf, and behind that pass A's histogram in sbuf
   const uint64_t tf_bytes = (s.n_tiles * 8 + 255) / 256 * 256;
-  lay.kbuf = take(s.one_level ? std::max<uint64_t>(s.cap * 4, tf_bytes) : s.cap_kb * s.kw * 8);
-  const uint64_t hist_bytes = s.one_level ? 0 : tf_bytes + s.n_tiles * P1 * 4;
+  lay.kbuf = take(one ? std::max<uint64_t>(s.cap * 4, tf_bytes) : s.cap_kb * s.kw * 8);
+  const uint64_t hist_bytes = one ? 0 : tf_bytes + s.n_tiles * P1 * 4;
   lay.sbuf = take(std::max<uint64_t>(s.cap_kb * s.kw * 8, hist_bytes));
   lay.meta = take(sizeof(Meta));
   lay.tf = s.one_level ? lay.kbuf : lay.sbuf;
+  lay.tf2 = lay.sbuf;
   lay.hist = lay.sbuf + tf_bytes;
+  lay.bins = lay.cst;
+  if (either) {  // (each keys array holds 100 MB and more here)
+    lay.bmap = lay.kbuf + tf_bytes;
+    lay.bmap2 = lay.sbuf + tf_bytes;
+    lay.bins = lay.bmap + ((size_t)2 << s.bb);
+  } else {
+    lay.bmap2 = lay.bmap;
+  }
   lay.total = at;
   return (uint32_t)nf;
 }
@@ -168,7 +189,9 @@ Buffers layout_buffers(const Layout& lay, uint8_t* ws) {
   b.tile_first = (uint64_t*)(ws + lay.tf);
   b.hist = (uint32_t*)(ws + lay.hist);
   b.cstart = (uint64_t*)(ws + lay.cst);
-  b.bins = (uint32_t*)(ws + lay.cst);
+  b.bins = (uint32_t*)(ws + lay.bins);
+  b.bmap2 = (uint16_t*)(ws + lay.bmap2);
+  b.tile_first2 = (uint64_t*)(ws + lay.tf2);
   b.bmap = (uint16_t*)(ws + lay.bmap);
   b.fine_base = (uint32_t*)(ws + lay.fb);
   b.fine_m = (uint32_t*)(ws + lay.fm);

@@ -25,9 +25,14 @@ constexpr int kPackThreads = 256;              // pass A: one code word per thre
 constexpr int kMaxCoarseLog2 = 12;             // at most 4096 coarse partitions
 constexpr int kMaxFine = 4096;                 // at most this many fine partitions per coarse one
 // One-level partitioning (inputs of a single coarse partition): pass A counts the windows of
-// 2^6 .. 2^13 bins, about 8 to a fine partition, and its last block groups the bins into at
-// most this many fine partitions, which pass B writes directly.
+// 2^10 .. 2^13 bins and its last block groups the bins into at most this many fine partitions,
+// which pass B writes directly.
 constexpr uint64_t kOneLevelFine = 3072;
+// Larger inputs below these bases take either path: one level if their repeats leave at most
+// this many fine partitions (four bins each), decided by pass A's last block.
+constexpr uint64_t kEitherBases = 48ull << 20;
+constexpr uint32_t kEitherFine = 2048;
+enum { kTwoLevel, kOneLevel, kEitherLevel };   // Shape::one_level
 constexpr int kMinBinsLog2 = 10, kMaxBinsLog2 = 13;
 constexpr uint32_t kMinFineKeys = 512;         // smaller fine partitions are not made to fill the SMs
 // bases per coarse partition aimed at when the plan sets no partition count
@@ -78,7 +83,7 @@ struct Meta {
   uint64_t ticket;      // phase-2 work counter
   uint64_t d_estimate;  // distinct keys estimated by the sketch
   uint32_t done;        // blocks of pass A that have finished
-  uint32_t pad_;
+  uint32_t one;         // either-level counts: 1 = pass B writes the fine partitions
   uint64_t sub_cycles[8];    // profiled plans only: ordering sub-steps (range, rank, scan, place, small sorts, big sorts, #big)
   uint64_t phase_cycles[8];  // profiled plans only: SM cycles per phase of k_count_emit, summed over CTAs
 };
@@ -108,7 +113,7 @@ struct Shape {
   int defer_all;        // nonzero (testing): every fine partition takes the deferred write-out
   int withhold;         // nonzero (testing): partition 0 never publishes its prefix
   int aggr;             // aggregation variants: kAggr* bits (single-count path only)
-  int one_level;        // nonzero: pass B writes the fine partitions directly (b1 = 0)
+  int one_level;        // kOneLevel: pass B writes the fine partitions directly (b1 = 0); kEitherLevel
   int bb;               // one-level: log2 of the bins that are grouped into fine partitions
   int n_sms;
 };
@@ -138,6 +143,8 @@ struct Buffers {
   Meta* meta;
   uint32_t* bins;         // one-level: [2^bb] windows per bin (in cstart's memory)
   uint16_t* bmap;         // one-level: [2^bb] fine partition of each bin
+  uint16_t* bmap2;        // either-level counts that take two: coarse partition of each bin, and the tiles' first
+  uint64_t* tile_first2;  // reads (bmap, bins and tile_first lie in kbuf's memory then, these in sbuf's)
 };
 
 // One count of a batch: its shape and its buffers (inside the batch's scratch arena).
@@ -212,7 +219,7 @@ struct ShapeOpts {
   int tight_slack = 0;     // testing: sampled regions get no slack
 };
 struct Layout {  // byte offsets into the count's scratch block
-  size_t reads, offs, codes, inv, tf, hist, cst, bmap, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
+  size_t reads, offs, codes, inv, tf, tf2, hist, cst, bins, bmap, bmap2, fb, fm, hll, fh, fo, flo, fc, look, kbuf, sbuf, meta;
   size_t total;
 };
 // Fills s and lay for L bases and n_reads reads; copy_reads / copy_offs: the scratch holds a

@@ -304,7 +304,10 @@ __device__ __forceinline__ void prepare_body(const Shape& s, const Buffers& b, u
         if (below > 0) lo = first + step * (below - 1) + 1;
       }
     }
-    if (lane == 0) b.tile_first[t] = lo;
+    if (lane == 0) {
+      b.tile_first[t] = lo;
+      if (s.one_level == kEitherLevel) b.tile_first2[t] = lo;
+    }
   }
 }
 __global__ void __launch_bounds__(256) k_prepare(Shape s, Buffers b) { pdl_wait(); prepare_body(s, b, blockIdx.x, gridDim.x); }
@@ -714,12 +717,24 @@ __device__ __forceinline__ void bucket_scan(const Shape& s, const Buffers& b, ui
 __device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b, uint32_t* sc) {
   __shared__ uint32_t wt[32];
   const int NB = 1 << s.bb;
+#pragma unroll 8
   for (int i = threadIdx.x; i < NB; i += blockDim.x) sc[PAD(i)] = __ldcg(&b.bins[i]);
   __syncthreads();
-  const uint32_t K = block_exclusive_scan_pad<uint32_t>(sc, NB, wt);  // below 2^24
+  const uint32_t K = block_exclusive_scan_pad<uint32_t>(sc, NB, wt);  // below 2^26
   const double target = sketch_target(b.hll, K, s, 0, b.meta);
   const uint32_t T = max((uint32_t)ceil(target), (uint32_t)(K / s.nf_max) + 1u);
   const uint32_t NF = sc[PAD(NB - 1)] / T + 1;  // the last bin's partition is the last: at most K / T + 1 <= nf_max
+  const bool either = s.one_level == kEitherLevel;
+  if (either && NF > kEitherFine) {  // two levels: the coarse partitions are the bins' top bits
+    const int P1 = 1 << s.b1, per = NB >> s.b1;
+    for (int i = threadIdx.x; i < NB; i += blockDim.x) b.bmap2[i] = (uint16_t)(i / per);
+    for (int c = threadIdx.x; c < P1; c += blockDim.x) b.cstart[c] = b.fcur[c] = sc[PAD(c * per)];
+    if (threadIdx.x == 0) {
+      b.cstart[P1] = K;
+      b.meta->n_windows = K;
+    }
+    return;
+  }
   for (int i = threadIdx.x; i < NB; i += blockDim.x) {
     const uint32_t p = sc[PAD(i)];
     const int g = (int)(p / T), prev = i ? (int)(sc[PAD(i - 1)] / T) : -1;
@@ -727,12 +742,13 @@ __device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b,
     for (int q = prev + 1; q <= g; ++q) {
       b.foff[q] = p;
       b.fcur[q] = p;
-      b.flo[q] = (uint32_t)i << (32 - s.bb);
+      if (!either) b.flo[q] = (uint32_t)i << (32 - s.bb);  // (either: after pass B, in the codes' memory)
     }
   }
   if (threadIdx.x == 0) {
     b.foff[NF] = K;
-    b.flo[NF] = 0;  // so that the last partition ends at u = 2^32 - 1
+    if (!either) b.flo[NF] = 0;  // so that the last partition ends at u = 2^32 - 1
+    b.meta->one = 1;
     b.meta->n_windows = K;
     b.meta->n_fine = NF;
   }
@@ -830,8 +846,10 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
     for (int c = t; c < P1; c += kPackThreads) hist_s[c] = 0;
     if constexpr (ONE) {  // several tiles, so that the bins are added up less often
       for (uint64_t tile = bid; tile < s.n_tiles; tile += nblk) pack_tile<KW, true, VAR>(s, b, tile, hist_s);
-      for (int c = t; c < P1; c += kPackThreads)
+      for (int i = t; i < P1; i += kPackThreads) {  // (each block starts elsewhere: all end together)
+        const int c = (i + bid * 13 * kPackThreads) & (P1 - 1);
         if (hist_s[c]) atomicAdd(&b.bins[P1 - 1 - c], hist_s[c]);
+      }
     } else {
       pack_tile<KW, false, VAR>(s, b, bid, hist_s);
       // the tile's counts, and the partitions' totals (cstart holds them until bucket_scan)
@@ -866,6 +884,12 @@ __device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b,
   extern __shared__ uint32_t fsc[];  // [padded P1]
   __shared__ uint32_t wt[32];
   const int P1 = 1 << s.b1;
+  if (s.one_level && b.meta->one) {  // planned before pass B; what is left is the partitions' first values
+    for (int i = c * blockDim.x + threadIdx.x; i < (1 << s.bb); i += P1 * blockDim.x)
+      for (int q = i ? b.bmap[i - 1] + 1 : 0; q <= b.bmap[i]; ++q) b.flo[q] = (uint32_t)i << (32 - s.bb);
+    if (c == 0 && threadIdx.x == 0) b.flo[min(b.meta->n_fine, s.nf_max)] = 0;
+    return;
+  }
   const uint32_t T = (uint32_t)ceil(sketch_target(b.hll, b.cstart[P1], s, P1, b.meta));
   auto parts = [&](uint64_t n) -> uint32_t {  // (n is below 2^32)
     const uint32_t m = n ? ((uint32_t)n - 1) / T + 1 : 1;
@@ -923,7 +947,9 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   extern __shared__ __align__(16) uint8_t sm[];
   constexpr bool DIRECT = MODE == SC_DIRECT, ONE = MODE == SC_ONE;
   const int canonical = VAR == V_SHORT ? s.canonical : VAR == V_CANON;
-  const int P1 = ONE ? (int)min(b.meta->n_fine, s.nf_max) : 1 << s.b1, PM = ONE ? (int)s.nf_max : P1;
+  const bool fine = ONE && b.meta->one;  // (ONE without: an either-level count that takes two)
+  const int PM = ONE ? (s.one_level == kEitherLevel ? (int)kEitherFine : (int)s.nf_max) : 1 << s.b1;
+  const int P1 = fine ? (int)min(b.meta->n_fine, (uint64_t)PM) : 1 << s.b1;
   K* stage = reinterpret_cast<K*>(sm);                                                // [SUB]
   unsigned long long* cursor = reinterpret_cast<unsigned long long*>(stage + SUB);   // [P1] absolute write positions
   uint32_t* hist = reinterpret_cast<uint32_t*>(cursor + (ONE ? 0 : P1));                // [padded PM + 32]
@@ -948,8 +974,8 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     hist[PAD(c)] = 0;
   }
   if constexpr (ONE)
-    for (int i = t; i < (1 << s.bb); i += NT) map[i] = b.bmap[(1 << s.bb) - 1 - i];
-  if (t == 0) rcur_s = b.tile_first[tile];
+    for (int i = t; i < (1 << s.bb); i += NT) map[i] = (fine ? b.bmap : b.bmap2)[(1 << s.bb) - 1 - i];
+  if (t == 0) rcur_s = (ONE && !fine ? b.tile_first2 : b.tile_first)[tile];
   for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
     if (j0 >= s.n_words) break;
@@ -1022,10 +1048,10 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     // pass A saw the same reads) is recorded and the sub-step not written.
     bool fits = true;
     for (int c = t; c < P1; c += NT) {
-      if constexpr (ONE) {  // (positions are below 2^24; hist holds cursor - soff until it is cleared)
+      if constexpr (ONE) {  // (positions are below 2^26; hist holds cursor - soff until it is cleared)
         const uint32_t n = hist[PAD(c)];
         if (n) {
-          const uint64_t lim = b.foff[c + 1], at = atomicAdd(&b.fcur[c], (unsigned long long)n);
+          const uint64_t lim = (fine ? b.foff : b.cstart)[c + 1], at = atomicAdd(&b.fcur[c], (unsigned long long)n);
           fits = fits && at + n <= lim;
           hist[PAD(c)] = (uint32_t)at - soff[PAD(c)];
         }
@@ -1050,7 +1076,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
       for (uint32_t i = t; i < n_sub; i += NT) {
         const K key = stage[i];
         const uint32_t c = coarse_field_rev(top32_of(key, s.k), canonical, ONE ? s.bb : s.b1);  // as above, from the key
-        if constexpr (ONE) store_key(b.sbuf, (uint32_t)(hist[PAD(map[c])] + i), key);
+        if constexpr (ONE) store_key(fine ? b.sbuf : b.kbuf, (uint32_t)(hist[PAD(map[c])] + i), key);
         else store_key(b.kbuf, cursor[c] + i, key);
       }
     } else if (t == 0) {
@@ -1161,6 +1187,7 @@ __device__ __forceinline__ void fine_hist_body(const Shape& s, const Buffers& b,
   typedef typename KeyT<KW>::T K;
   extern __shared__ __align__(16) uint8_t sm[];
   if (redo && !b.meta->fine_spill) return;  // the exact fine split runs again only after a spill
+  if (s.one_level && b.meta->one) return;
   // a sampled layout counts one chunk in 2^kFineSampleLog2 (the exact split: every chunk)
   const uint64_t cstep = (s.fine_sampled && !redo) ? ((uint64_t)kFineChunk << kFineSampleLog2) : (uint64_t)kFineChunk;
   const int P1 = 1 << s.b1;
@@ -1262,6 +1289,7 @@ __device__ __forceinline__ uint64_t coarse_room(uint64_t n_c, uint64_t s_c, uint
 __device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b, uint32_t c, bool redo = false) {
   __shared__ uint64_t wt[32];
   if (redo && !b.meta->fine_spill) return;
+  if (sh.one_level && b.meta->one) return;
   const bool sampled = sh.fine_sampled && !redo;
   const int P1 = 1 << sh.b1, t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
   const uint64_t NF = min(b.meta->n_fine, sh.nf_max);
@@ -1384,6 +1412,7 @@ __device__ __forceinline__ void fine_scatter_body(const Shape& s, const Buffers&
   // not written at all.  In a sampled layout a run that would pass its region's end is not
   // written: the spill is recorded and the exact split follows.
   if (redo ? !b.meta->fine_spill : (s.fine_sampled && b.meta->fine_spill)) return;
+  if (s.one_level && b.meta->one) return;
   const bool sampled = s.fine_sampled && !redo;
   constexpr uint64_t kSpilledRun = 1ull << 63;  // never a run's offset
   const int P1 = 1 << s.b1;
@@ -2485,7 +2514,10 @@ __global__ void __launch_bounds__(256) k_compact_batch(BatchTab t) {
 constexpr size_t kScatterStaticSmem = 6144;  // pass B's static shared memory (batched form included), rounded up
 static size_t scatter_smem(const Shape& s, int nt) {
   const size_t sub = (size_t)nt * (s.kw == 1 ? 32 : 16) * s.kw * 8;
-  if (s.one_level) return sub + 2 * padded_len(s.nf_max + 32) * 4 + ((size_t)2 << s.bb);
+  if (s.one_level) {
+    const size_t most = s.one_level == kEitherLevel ? kEitherFine : s.nf_max;
+    return sub + 2 * padded_len(most + 32) * 4 + ((size_t)2 << s.bb);
+  }
   const size_t P1 = (size_t)1 << s.b1;
   return sub + P1 * 8 + 2 * padded_len(P1 + 32) * 4;
 }
@@ -2630,7 +2662,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
     ++launches;
     KC_STEP("k_scatter");
   }
-  if (!s.one_level) {
+  if (s.one_level != kOneLevel) {
     pdl_launch(k_fine_plan, P1, 256, padded_len(P1) * 4, st, s, b);
     ++launches;
     KC_STEP("k_fine_plan");
@@ -2667,7 +2699,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
   }
   ++launches;
   KC_STEP("k_count_emit");
-  if (s.one_level) {
+  if (s.one_level == kOneLevel) {
     if (s.kw == 1) pdl_launch(k_finish_one<1>, compact_blocks(s, n_sms), 256, 0, st, s, b);
     else pdl_launch(k_finish_one<2>, compact_blocks(s, n_sms), 256, 0, st, s, b);
     ++launches;
@@ -2694,16 +2726,16 @@ uint32_t batch_blocks(BatchKernel k, const Shape& s, int n_sms, uint64_t bases_t
     case BK_SCATTER: return s.one_level ? 0u : (uint32_t)s.n_tiles;
     case BK_SCATTER_ONE: return s.one_level ? (uint32_t)s.n_tiles : 0u;
     case BK_FINE_PLAN:
-    case BK_FINE_SCAN: return s.one_level ? 0u : 1u << s.b1;
+    case BK_FINE_SCAN: return s.one_level == kOneLevel ? 0u : 1u << s.b1;
     case BK_FINE_HIST:
-    case BK_FINE_SCATTER: return s.one_level ? 0u : clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
+    case BK_FINE_SCATTER: return s.one_level == kOneLevel ? 0u : clampu((s.L + 4ull * kFineChunk - 1) / (4ull * kFineChunk), 1, 2 * nsm);
     case BK_COUNT: {
       const double share = bases_total ? (double)s.L / (double)bases_total : 1.0;
       return clampu((uint64_t)(2.0 * (double)nsm * share + 0.999), 1, nsm * kCountBlocksPerSM);
     }
-    case BK_SCAN_DISTINCT: return s.one_level ? 0u : scan_blocks(s);
-    case BK_COMPACT: return s.one_level ? 0u : compact_blocks(s, n_sms);
-    case BK_FINISH_ONE: return s.one_level ? compact_blocks(s, n_sms) : 0u;
+    case BK_SCAN_DISTINCT: return s.one_level == kOneLevel ? 0u : scan_blocks(s);
+    case BK_COMPACT: return s.one_level == kOneLevel ? 0u : compact_blocks(s, n_sms);
+    case BK_FINISH_ONE: return s.one_level == kOneLevel ? compact_blocks(s, n_sms) : 0u;
     default: return 1u;
   }
 }

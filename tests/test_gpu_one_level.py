@@ -90,3 +90,35 @@ def test_two_level_plan_and_scans(torch_cuda, hint, slots, genome):
         res.free()
         c.close()
         assert np.array_equal(keys, want_k) and np.array_equal(counts, want_c), kw
+
+
+# From 12 Mi bases on the number of fine partitions decides: a 30x genome leaves few (one level),
+# unrelated reads leave more than 2048 (two levels).  Compared with a plan that always takes two.
+@pytest.mark.parametrize("genome,few", [(450_000, True), (0, False)])
+@pytest.mark.parametrize("k,canonical", [(31, True), (12, True), (32, False)])
+@pytest.mark.parametrize("defer", [False, True])
+def test_either_level(torch_cuda, genome, few, k, canonical, defer):
+    from paper_2505_04431_gb300 import KmerCounter
+    torch = torch_cuda
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(genome + k)
+    n, length = 90_001, 147
+    letters = torch.tensor(list(b"ACGT"), dtype=torch.uint8, device="cuda")
+    if genome:
+        g = torch.randint(0, 4, (genome,), generator=gen, device="cuda")
+        at = torch.randint(0, genome - length, (n, 1), generator=gen, device="cuda")
+        codes = g[at + torch.arange(length, device="cuda")]
+    else:
+        codes = torch.randint(0, 4, (n, length), generator=gen, device="cuda")
+    reads = letters[codes].reshape(-1)
+    offsets = torch.arange(n + 1, device="cuda") * length
+    got = []
+    for kw in ({}, {"n_partitions_hint": 2}):
+        c = KmerCounter(defer_all=defer, **kw)
+        res = c.count(reads, offsets, k, canonical)
+        got.append((res.keys_tensor().clone(), res.counts_tensor().clone(), res.n_valid_windows, c.stats()["n_fine"]))
+        res.free()
+        c.close()
+    assert got[0][2] == got[1][2] and torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    if k >= 31:
+        assert (got[0][3] <= 2048) == few
