@@ -87,7 +87,6 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
     if (bt < bT_max) bT_max = bt;
   }
   s.bT_max = bT_max;
-  s.tail = bT_max >= 10 ? 1024 : (1 << bT_max);
   const double ft = (double)(1u << bT_max) * o.load;  // distinct keys per fine partition aimed at
   s.fine_target = ft < 16 ? 16u : (uint32_t)ft;
   s.cap = L > 0 ? L : 1;
@@ -921,7 +920,7 @@ kc_status kc_count(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, u
     }
     first = p->rb->ends[0];
     L = p->rb->ends[1];
-  } else {  // their order is checked on the device (k_check_offsets), as for device offsets
+  } else {  // their order is checked on the device (check_offsets), as for device offsets
     first = offsets[0];
     L = offsets[n_reads];
   }

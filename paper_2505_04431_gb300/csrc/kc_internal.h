@@ -5,8 +5,9 @@
 //                the two most significant bits (Algorithm 1's kmer << 2 order).
 //   inv32[w]     bit i set iff byte 32w+i is not one of ACGTacgt, or lies past
 //                the end of the input.
-//   hist[t][c]   phase-1 histogram: valid windows of tile t in coarse partition c.
+//   hist[t][c]   phase-1 histogram: valid windows of tile t in coarse partition c
 //                (in sbuf's memory: read by pass B, before sbuf is written).
+//   bins, bmap   one-level counts: valid windows per bin, and each bin's fine partition.
 //   kbuf         keys grouped by coarse partition (the owner partition of
 //                Algorithm 3's AsyncAdd, here a key range so that outputs concatenate
 //                in sorted order).
@@ -20,7 +21,7 @@ namespace kc {
 constexpr int kWordBases = 32;                 // bases per packed code word
 constexpr int kTileWordsMax = 8192;            // a phase-1 tile has 256 .. 8192 code words (Shape::tile_words)
 constexpr int kTileWordsStep = 256;
-constexpr uint64_t kTilesWanted = 4864;        // 16 waves of pass B's 2 blocks on each of 152 SMs
+constexpr uint64_t kTilesWanted = 4864;        // over 10 waves of pass B's 3 blocks on each of 152 SMs
 constexpr int kPackThreads = 256;              // pass A: one code word per thread per sub-step
 constexpr int kMaxCoarseLog2 = 12;             // at most 4096 coarse partitions
 constexpr int kMaxFine = 4096;                 // at most this many fine partitions per coarse one
@@ -99,7 +100,6 @@ struct Shape {
   int kw;               // key words: 1 or 2
   int b1;               // log2 coarse partitions
   int bT_max;           // log2 of the largest table
-  int tail;             // table slots past the home range (linear probing never wraps)
   uint32_t fine_target; // keys per fine partition aimed for
   uint64_t cap;         // capacity of kbuf / sbuf / outputs in keys
   uint64_t nf_max;      // capacity of the fine-partition arrays
@@ -200,7 +200,7 @@ uint32_t batch_blocks(BatchKernel k, const Shape& s, int n_sms, uint64_t bases_t
 int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mark);
 int configure_kernels(int device);  // sets shared-memory attributes; returns 0 or a cudaError_t
 
-size_t count_kernel_smem(int kw, int bT_max, int tail);
+size_t count_kernel_smem(int kw, int bT_max);
 void set_error_message(const char* msg);  // the text kc_last_error returns on this thread
 int table_log2_max(int kw, size_t smem_optin, size_t smem_per_sm);
 

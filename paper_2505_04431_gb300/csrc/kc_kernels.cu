@@ -1,12 +1,15 @@
 // kc_kernels.cu - the k-mer counting hot path on sm_103a.
 //
+// k_prepare                 clears the sketch, the histogram's totals and the status record,
+//                           and finds the first read of every phase-1 tile.
 // Phase 1 (Section III-C, Algorithm 3 first loop; Section V "Phase 1"):
 //   pass A  k_pack_count    ASCII -> 2-bit codes + invalid mask (the paper's Encode),
 //                           rolling forward / reverse-complement keys (Algorithm 1's
 //                           kmer = (kmer << 2) OR Encode), owner partition of every
-//                           valid window, per-tile partition histogram.
-//   scan    k_bucket_scan   partition starts; a tile then reserves its run in each partition
-//                           with one atomic add on that partition's cursor.
+//                           valid window, per-tile partition histogram.  Its last block
+//                           scans the totals to partition starts; a tile of pass B then
+//                           reserves its run in each partition with one atomic add on that
+//                           partition's cursor.
 //   pass B  k_scatter       recomputes the keys from the packed codes and writes each
 //                           key to its owner partition.  A tile's keys are first
 //                           grouped per partition in shared memory (a counting sort)
@@ -26,7 +29,12 @@
 //                           decoupled look-back over the fine partitions, or in its own
 //                           input region when that offset is not known in time.
 //   k_scan_distinct, k_compact   output offsets of all runs; the runs written in place
-//                           move to their offsets.
+//                           move to their offsets; the last kernel also checks that the read
+//                           offsets ascend (the earlier ones stay in bounds if they do not).
+// One level (small inputs, and larger ones whose repeats leave few fine partitions): pass A
+// counts the windows of 2^10 .. 2^13 bins instead of the coarse partitions' and fills the
+// sketch; its last block groups the bins into fine partitions, pass B writes these, and the
+// fine split is left out.  k_finish_one then does k_scan_distinct's and k_compact's work.
 // Variants: every kernel body also runs as a batched kernel (one launch for a group of
 // counts, each thread block working for one count found through a block table); pass B
 // without the shared-memory staging (DIRECT) and the count kernel with a warp-level merge
@@ -1596,7 +1604,7 @@ struct Table {
 // up to 3/4 of the slots, grouped by bucket, the slot numbers and (64-bit keys) the keys.
 constexpr int kTableLog2Cap = kCountThreads == 1024 ? 13 : 12;  // 8 slots per thread
 
-size_t count_kernel_smem(int kw, int bT_max, int /*unused*/) {
+size_t count_kernel_smem(int kw, int bT_max) {
   const size_t slots = (size_t)1 << bT_max;
   return slots * (size_t)(kw * 8 + 4) + slots * 2 + 16 + ((3 * slots) >> 2) * (kw == 1 ? 10 : 2) + 256;
 }
@@ -1611,7 +1619,7 @@ int table_log2_max(int kw, size_t smem_optin, size_t smem_per_sm) {
   }
   int best = 6;
   for (int bt = 6; bt <= kTableLog2Cap; ++bt)
-    if (count_kernel_smem(kw, bt, 0) + 12288 <= budget) best = bt;
+    if (count_kernel_smem(kw, bt) + 12288 <= budget) best = bt;
   return best;
 }
 
@@ -2688,7 +2696,7 @@ int launch_phase2(const Shape& s, const Buffers& b, int n_sms, uint32_t nf_max, 
       KC_STEP(redo ? "k_fine_scatter_redo" : "k_fine_scatter");
     }
   }
-  const size_t smC = count_kernel_smem(s.kw, s.bT_max, s.tail);
+  const size_t smC = count_kernel_smem(s.kw, s.bT_max);
   if (s.aggr & kAggrWarpMerge) {
     if (s.kw == 1) pdl_launch(k_count_emit<1, true>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
     else pdl_launch(k_count_emit<2, true>, (unsigned)(n_sms * kCountBlocksPerSM), kCountThreads, smC, st, s, b);
@@ -2810,7 +2818,7 @@ int launch_batch(const BatchPlan& bp, int n_sms, void* stream, const Marker& mar
                  redo ? "k_fine_scatter_redo" : "k_fine_scatter");
     }
   }
-  const size_t smC = count_kernel_smem(bp.kw, s0.bT_max, s0.tail);
+  const size_t smC = count_kernel_smem(bp.kw, s0.bT_max);
   if (bp.kw == 1) {
     KC_BLAUNCH(BK_COUNT, (k_count_emit_batch<1><<<bp.grid[BK_COUNT], kCountThreads, smC, st>>>(tab(BK_COUNT))),
                "k_count_emit");
