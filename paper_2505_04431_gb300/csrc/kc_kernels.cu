@@ -640,6 +640,40 @@ __device__ __forceinline__ void sketch_add(uint32_t* hll, K key) {
   const uint32_t v = (uint32_t)min(__clzll(h << kHllLog2) + 1, 64 - kHllLog2 + 1);
   if (v > hll[reg]) atomicMax(&hll[reg], v);
 }
+// The canonical (or forward) key of the window whose last base is s bases before the end of
+// the 96 bases (w2 : w1 : w0); 0 <= s < 32.  For the few windows picked out by a run-time index.
+__device__ __forceinline__ void window_key(uint64_t, uint64_t w1, uint64_t w0, uint32_t s, int k, int canonical,
+                                           uint64_t& key) {
+  const int x = 64 - 2 * k;
+  const uint64_t f = (s ? (w0 >> (2 * s)) | (w1 << (64 - 2 * s)) : w0) << x >> x;
+  const uint64_t r = revcomp(f, k);
+  key = canonical && r < f ? r : f;
+}
+__device__ __forceinline__ void window_key(uint64_t w2, uint64_t w1, uint64_t w0, uint32_t s, int k, int canonical,
+                                           u128& key) {
+  const int x = 128 - 2 * k;
+  u128 f = ((u128)w1 << 64 | w0) >> (2 * s);
+  if (s) f |= (u128)(w2 << (64 - 2 * s)) << 64;
+  f = f << x >> x;
+  const u128 r = revcomp(f, k);
+  key = canonical && r < f ? r : f;
+}
+// A thread's sampled windows (bit i of m: the window whose last base is last - i bases before
+// the end of the words) go to the sketch after its loop over the windows.  Inside that loop
+// two warps in five left it at every window for the one lane that had a sampled key. (Pass B of
+// 2.4 G windows 11.93 -> 10.77 ms, of 59 M 128-bit windows 596 -> 565 us; pass A of 10 M bases,
+// one level, 45 -> 40.)
+template <class K>
+__device__ __forceinline__ void sketch_windows(uint32_t* hll, uint32_t m, uint32_t last, uint64_t w2, uint64_t w1,
+                                               uint64_t w0, int k, int canonical) {
+  while (m) {
+    const uint32_t i = __ffs(m) - 1;
+    m &= m - 1;
+    K key;
+    window_key(w2, w1, w0, last - i, k, canonical, key);
+    sketch_add(hll, key);
+  }
+}
 
 // The keys a fine partition aims at, from the sketch of a count of K windows: fine_target
 // distinct keys, i.e. fine_target * K / D keys; where that gives an SM few partitions, as much
@@ -826,22 +860,17 @@ __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint
       Win W;
       const uint32_t vm = valid_mask(inv_s[t], inv_s[t + 1], inv, st_s[t], st_s[t + 1], st_s[t + 2], s.k);
       win_setup<KW, 32>(code_s[t], code_s[t + 1], code, vm, 0, s.k, W);
+      uint32_t picked = 0;  // windows for the sketch
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
         uint32_t f, r;
         const uint32_t c = coarse_field_rev(win_top32<KW, 32, VAR>(W, i, canonical, f, r), canonical, bits);
         const uint32_t v = W.valid & (1u << i);
         red_shared_if(hist_a + 4 * c, v);  // predicated: no branch, no bin for the invalid windows
-        if constexpr (ONE) {
-          if (v && sketch_sampled(f, r)) {
-            uint64_t c0, c1;
-            K key;
-            win_top<KW, 32>(W, i, canonical, c0, c1);
-            top_to_key(c0, c1, s.k, key);
-            sketch_add(b.hll, key);
-          }
-        }
+        if (ONE && sketch_sampled(f, r)) picked |= 1u << i;
       }
+      if constexpr (ONE)
+        sketch_windows<K>(b.hll, picked & W.valid, 31, code_s[t], code_s[t + 1], code_s[t + 2], s.k, canonical);
     }
   }
   __syncthreads();
@@ -935,7 +964,7 @@ __global__ void __launch_bounds__(256) k_fine_plan_batch(BatchTab t) {
 // its canonical value alone, and its rank inside the partition from a shared-memory atomic (a
 // counting sort's first step); after the block scan of the partition histogram the whole keys
 // are computed, go to their partition's run in the staging buffer, and the runs leave in
-// order.  Bound by instruction issue and latency, not by HBM (19.2 GB written in 11.9 ms at 2.4 G
+// order.  Bound by instruction issue and latency, not by HBM (19.2 GB written in 10.8 ms at 2.4 G
 // windows): no key is kept in registers across the scan (each is computed once, after it) and
 // a staged key's partition is found from the key again, so that three blocks fit an SM (80
 // registers, 73 KB).  With the keys held and the partitions kept in shared memory there were
@@ -1011,10 +1040,11 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
     win_setup<KW, WPT>(code_s[sw - 2], code_s[sw - 1], code_s[sw], vm, h, s.k, W);
     const uint32_t valid = W.valid & (WPT == 32 ? 0xffffffffu : 0xffffu);
     uint32_t cr[WPT];  // each window's partition and its rank there
+    uint32_t picked = 0;  // windows for the sketch
     // every window is ranked without a branch (so that the windows' dependency chains
     // interleave): an invalid window is ranked in bin P1 + lane, which no scan reads (one such
-    // bin per lane, so that a warp's invalid windows do not share an address), and only the
-    // rare sketch update depends on the window being valid
+    // bin per lane, so that a warp's invalid windows do not share an address), and the sketch's
+    // windows are only noted
 #pragma unroll
     for (int i = 0; i < WPT; ++i) {
       uint32_t f, r;
@@ -1036,16 +1066,10 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
         const uint32_t cc = v ? c : (uint32_t)P1 + (t & 31);
         cr[i] = (cc << 16) | atomicAdd(&hist[PAD(cc)], 1u);  // bin below 2^13, rank below 2^13
       }
-      if constexpr (!ONE) {
-        if (v && sketch_sampled(f, r)) {
-          uint64_t c0, c1;
-          K key;
-          win_top<KW, WPT>(W, i, canonical, c0, c1);
-          top_to_key(c0, c1, s.k, key);
-          sketch_add(b.hll, key);
-        }
-      }
+      if (!ONE && sketch_sampled(f, r)) picked |= 1u << i;
     }
+    if constexpr (!ONE)
+      sketch_windows<K>(b.hll, picked & valid, 31 - 16 * h, code_s[sw - 2], code_s[sw - 1], code_s[sw], s.k, canonical);
     if constexpr (DIRECT) continue;
     __syncthreads();
     for (int c = t; c < P1; c += NT) soff[PAD(c)] = hist[PAD(c)];

@@ -122,3 +122,29 @@ def test_either_level(torch_cuda, genome, few, k, canonical, defer):
     assert got[0][2] == got[1][2] and torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
     if k >= 31:
         assert (got[0][3] <= 2048) == few
+
+
+@pytest.mark.parametrize("k", [12, 16, 21, 31, 32, 33, 48, 63, 64])
+def test_sketch_of_sampled_windows(torch_cuda, k):
+    """The sketch takes its keys from a thread's noted windows by their index.  Sixteen copies
+    of a sequence and eight of each strand have the same canonical keys, so the same estimate
+    and the same number of fine partitions; that number gives the distinct keys within 20%:
+    5 x (1.04 / sqrt(1024) for the sketch and 1 / sqrt(5900) for the sample it sees), and less
+    than 1% for the partitions rounded up in each of four coarse ones."""
+    from paper_2505_04431_gb300 import KmerCounter
+    rng = np.random.default_rng(k)
+    seq = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, 380_000)]
+    other = np.frombuffer(b"TGCA", np.uint8)[np.searchsorted(np.frombuffer(b"ACGT", np.uint8), seq)][::-1]
+    offsets = torch_cuda.from_numpy(np.arange(17, dtype=np.int64) * len(seq)).cuda()
+    for options in ({"n_partitions_hint": 4, "table_slots_max": 256, "table_load": 0.5}, {}):
+        c = KmerCounter(**options)
+        n_fine = []
+        for copies in ([seq] * 16, [seq, other] * 8):
+            res = c.count(torch_cuda.from_numpy(np.concatenate(copies)).cuda(), offsets, k)
+            distinct = res.n
+            res.free()
+            n_fine.append(c.stats()["n_fine"])
+        c.close()
+        assert n_fine[0] == n_fine[1]
+        if options:
+            assert abs(n_fine[0] * 128 * 0.9 / distinct - 1) < 0.2
