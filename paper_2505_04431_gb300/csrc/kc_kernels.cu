@@ -2558,7 +2558,6 @@ static uint32_t prepare_blocks(const Shape& s, uint64_t most) {
   const uint64_t want = std::max<uint64_t>((s.nf_max + 255) / 256, (s.n_tiles + 7) / 8) + 4;
   return (uint32_t)(want < most ? want : most);
 }
-// pass A: one block per tile (one-level: at most one wave, 4 blocks on 152 SMs)
 // Pass A: a block per tile, or (one level) at most four per SM, each adding up the bins of
 // several tiles (pass A of 10 M / 45 M bases: 608 blocks 40 / 93 us, 912 44 / 107, 1216 51 /
 // 100; as few blocks as give each the same number of tiles, 407 / 550: 42 / 102).
