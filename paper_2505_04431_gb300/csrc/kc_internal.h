@@ -85,6 +85,7 @@ struct Meta {
   uint64_t d_estimate;  // distinct keys estimated by the sketch
   uint32_t done;        // blocks of pass A that have finished
   uint32_t one;         // either-level counts: 1 = pass B writes the fine partitions
+  uint32_t fine_unfit;  // the sampled fine layout does not fit its room (set by the fine scan, with fine_spill)
   uint64_t sub_cycles[8];    // profiled plans only: ordering sub-steps (range, rank, scan, place, small sorts, big sorts, #big)
   uint64_t phase_cycles[8];  // profiled plans only: SM cycles per phase of k_count_emit, summed over CTAs
 };

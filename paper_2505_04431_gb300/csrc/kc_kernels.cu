@@ -1370,7 +1370,7 @@ __device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b
   }
   if (t == 0) {
     if ((int)c == P1 - 1) b.foff[NF] = base + room;
-    if (sampled && (total > room || base + room > sh.cap_kb)) b.meta->fine_spill = 1;
+    if (sampled && (total > room || base + room > sh.cap_kb)) b.meta->fine_unfit = b.meta->fine_spill = 1;
   }
 }
 __global__ void __launch_bounds__(256) k_fine_scan(Shape sh, Buffers b, int redo) {
@@ -1442,8 +1442,10 @@ __device__ __forceinline__ void fine_scatter_body(const Shape& s, const Buffers&
   extern __shared__ __align__(16) uint8_t sm[];
   // the exact split runs again only after a spill; a sampled layout given up by the scan is
   // not written at all.  In a sampled layout a run that would pass its region's end is not
-  // written: the spill is recorded and the exact split follows.
-  if (redo ? !b.meta->fine_spill : (s.fine_sampled && b.meta->fine_spill)) return;
+  // written: the spill is recorded and the exact split follows.  (The first split is left by
+  // fine_unfit, which only the scan sets: other blocks of this launch may be setting fine_spill
+  // meanwhile, and warps of one block that read it on either side of that would part here.)
+  if (redo ? !b.meta->fine_spill : (s.fine_sampled && b.meta->fine_unfit)) return;
   if (s.one_level && b.meta->one) return;
   const bool sampled = s.fine_sampled && !redo;
   constexpr uint64_t kSpilledRun = 1ull << 63;  // never a run's offset

@@ -156,3 +156,33 @@ def test_batch_with_sampled_fine_layouts(torch_cuda, tight):
                 res.free()
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("k", [31, 63])
+def test_batch_spills_with_blocks_still_to_start(counter, torch_cuda, k):
+    """Sampled regions without slack overflow in a launch of more blocks (about 160 a sample)
+    than run at once, so that blocks start while others record the spill: whether a block
+    works is not read from what they write.  Every sample equals its count alone."""
+    from paper_2505_04431_gb300 import KmerCounter
+    torch = torch_cuda
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(k)
+    samples = []
+    for i in range(8):
+        n = 17_000 + 500 * i
+        genome = torch.randint(0, 4, (200_000 + 30_000 * i,), generator=gen, device="cuda")
+        at = torch.randint(0, len(genome) - 150, (n, 1), generator=gen, device="cuda")
+        reads = torch.tensor(list(b"ACGT"), dtype=torch.uint8, device="cuda")[genome[at + torch.arange(150, device="cuda")]]
+        samples.append((reads.reshape(-1), torch.arange(n + 1, device="cuda") * 150, n * 150))
+    c = KmerCounter(test_fine_sampled=True, test_tight_slack=True)
+    try:
+        for _ in range(3):
+            for i, ((r, o, _n), res) in enumerate(zip(samples, c.count_batch(samples, k, True))):
+                ref = counter.count(r, o, k, True)
+                assert res.n_valid_windows == ref.n_valid_windows
+                assert torch.equal(res.keys_tensor(), ref.keys_tensor()), (k, i)
+                assert torch.equal(res.counts_tensor(), ref.counts_tensor()), (k, i)
+                ref.free()
+                res.free()
+    finally:
+        c.close()
