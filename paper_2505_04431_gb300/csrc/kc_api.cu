@@ -459,14 +459,14 @@ bool enqueue_job(const Job& j, uint8_t* ws, cudaStream_t st, kc::Meta* meta_dst,
 
 kc_status job_status(const Job& j, const kc::Meta& m, const char* who, std::string* msg) {
   const std::string w(who);
+  if (m.status & kc::ST_BAD_OFFSETS) {
+    *msg = w + ": offsets must start at 0, be non-decreasing and end at the base count";
+    return KC_EINVAL;
+  }
   // the status record must describe a result that fits the buffers of this count
   if (m.n_windows > j.L || m.n_distinct > m.n_windows || m.n_fine > j.nf_max || m.n_deferred > m.n_fine) {
     *msg = w + ": inconsistent status record";
     return KC_ECUDA;
-  }
-  if (m.status & kc::ST_BAD_OFFSETS) {
-    *msg = w + ": offsets must start at 0, be non-decreasing and end at the base count";
-    return KC_EINVAL;
   }
   if (m.status & kc::ST_PARTITION_OVERFLOW) {
     *msg = w + ": one key range holds 2^32 windows or more; use more partitions";

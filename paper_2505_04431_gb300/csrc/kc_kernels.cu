@@ -29,8 +29,9 @@
 //                           decoupled look-back over the fine partitions, or in its own
 //                           input region when that offset is not known in time.
 //   k_scan_distinct, k_compact   output offsets of all runs; the runs written in place
-//                           move to their offsets; the last kernel also checks that the read
-//                           offsets ascend (the earlier ones stay in bounds if they do not).
+//                           move to their offsets.
+// Pass A also checks the read offsets; where they do not ascend from 0 to the base count, it
+// records that, plans no partition, and the later kernels of the count find nothing to do.
 // One level (small inputs, and larger ones whose repeats leave few fine partitions): pass A
 // counts the windows of 2^10 .. 2^13 bins instead of the coarse partitions' and fills the
 // sketch; its last block groups the bins into fine partitions, pass B writes these, and the
@@ -324,15 +325,20 @@ __global__ void __launch_bounds__(256) k_prepare_batch(BatchTab t) {
   prepare_body(d.s, d.b, bid, nblk);
 }
 
-// Offsets start at 0, do not decrease and end at L: a share for each block of the last kernel
-// (no kernel indexes memory by an unchecked offset: bad ones only make the counts meaningless).
+// Offsets start at 0, do not decrease and end at L: a share for each block of pass A, which by
+// itself stays in bounds whatever they hold.  Passes A and B mark the read starts of sub-steps
+// of different lengths with a cursor that only ascending offsets move alike, so with others
+// pass B would find windows that pass A has not counted and that no partition has room for:
+// pass A's last block then plans nothing, and no later kernel works on such a count.
 __device__ __forceinline__ void check_offsets(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
+  const uint64_t share = (s.n_reads + nblk - 1) / nblk, lo = min(s.n_reads, bid * share), hi = min(s.n_reads, lo + share);
   bool bad = false;
-  for (uint64_t i = bid * (uint64_t)blockDim.x + threadIdx.x; i < s.n_reads; i += (uint64_t)nblk * blockDim.x)
-    bad |= b.offsets[i + 1] < b.offsets[i];
+  for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) bad |= b.offsets[i + 1] < b.offsets[i];
   if (bid == 0 && threadIdx.x == 0) bad |= b.offsets[0] != 0 || b.offsets[s.n_reads] != s.L;
   if (bad) atomicOr(&b.meta->status, ST_BAD_OFFSETS);
 }
+// Set by pass A only, so the same for every thread of a later kernel.
+__device__ __forceinline__ bool bad_offsets(const Buffers& b) { return (__ldcg(&b.meta->status) & ST_BAD_OFFSETS) != 0; }
 
 // ------------------------------------------------------------------ phase 1 helpers
 // ASCII -> codes for 32 bytes given as 8 little-endian words.  The 2-bit codes of a word's four
@@ -819,7 +825,7 @@ __device__ __forceinline__ void pack_tile(const Shape& s, const Buffers& b, uint
   if (t == 0) {
     rcur_s = b.tile_first[tile];
     // bases read: never past the end the offsets give (a base count that disagrees with
-    // them is reported by the last kernel; the reads buffer is not overrun meanwhile)
+    // them is reported by check_offsets; the reads buffer is not overrun meanwhile)
     const uint64_t e = b.offsets[s.n_reads];
     len_s = e < s.L ? e : s.L;
   }
@@ -879,7 +885,8 @@ template <int KW, bool ONE, int VAR>
 __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
   extern __shared__ __align__(16) uint32_t hist_s[];  // [P1], partitions from the last to the first
   const int t = threadIdx.x, P1 = 1 << (ONE ? s.bb : s.b1);
-  if (bid < s.n_tiles) {  // (an empty input has one block and no tile)
+  check_offsets(s, b, bid, nblk);
+  if (bid < s.n_tiles) {  // (an empty input has a block and no tile; many short reads, blocks for their offsets only)
     for (int c = t; c < P1; c += kPackThreads) hist_s[c] = 0;
     if constexpr (ONE) {  // several tiles, so that the bins are added up less often
       for (uint64_t tile = bid; tile < s.n_tiles; tile += nblk) pack_tile<KW, true, VAR>(s, b, tile, hist_s);
@@ -898,6 +905,7 @@ __device__ __forceinline__ void pack_count_body(const Shape& s, const Buffers& b
     }
   }
   if (!last_block(&b.meta->done, nblk)) return;
+  if (bad_offsets(b)) return;  // no windows, no fine partitions (both 0 since k_prepare)
   if constexpr (ONE) one_level_plan(s, b, hist_s);
   else bucket_scan(s, b, reinterpret_cast<uint64_t*>(hist_s));
 }
@@ -921,6 +929,7 @@ __device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b,
   extern __shared__ uint32_t fsc[];  // [padded P1]
   __shared__ uint32_t wt[32];
   const int P1 = 1 << s.b1;
+  if (bad_offsets(b)) return;
   if (s.one_level && b.meta->one) {  // planned before pass B; what is left is the partitions' first values
     for (int i = c * blockDim.x + threadIdx.x; i < (1 << s.bb); i += P1 * blockDim.x)
       for (int q = i ? b.bmap[i - 1] + 1 : 0; q <= b.bmap[i]; ++q) b.flo[q] = (uint32_t)i << (32 - s.bb);
@@ -983,6 +992,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   constexpr int SUB = NT * WPT;             // windows per sub-step
   extern __shared__ __align__(16) uint8_t sm[];
   constexpr bool DIRECT = MODE == SC_DIRECT, ONE = MODE == SC_ONE;
+  const bool refused = bad_offsets(b);
   const int canonical = VAR == V_SHORT ? s.canonical : VAR == V_CANON;
   const bool fine = ONE && b.meta->one;  // (ONE without: an either-level count that takes two)
   const int PM = ONE ? (s.one_level == kEitherLevel ? (int)kEitherFine : (int)s.nf_max) : 1 << s.b1;
@@ -1013,6 +1023,7 @@ __device__ __forceinline__ void scatter_body(const Shape& s, const Buffers& b, u
   if constexpr (ONE)
     for (int i = t; i < (1 << s.bb); i += NT) map[i] = (fine ? b.bmap : b.bmap2)[(1 << s.bb) - 1 - i];
   if (t == 0) rcur_s = (ONE && !fine ? b.tile_first2 : b.tile_first)[tile];
+  if (refused) return;  // (here, so that the load's latency is shared with those above, all in bounds)
   for (int sub = 0; sub < (int)s.tile_words / NW; ++sub) {
     const uint64_t j0 = tile * s.tile_words + (uint64_t)sub * NW;
     if (j0 >= s.n_words) break;
@@ -1321,7 +1332,7 @@ __device__ __forceinline__ uint64_t coarse_room(uint64_t n_c, uint64_t s_c, uint
 __device__ __forceinline__ void fine_scan_body(const Shape& sh, const Buffers& b, uint32_t c, bool redo = false) {
   __shared__ uint64_t wt[32];
   if (redo && !b.meta->fine_spill) return;
-  if (sh.one_level && b.meta->one) return;
+  if (bad_offsets(b) || (sh.one_level && b.meta->one)) return;
   const bool sampled = sh.fine_sampled && !redo;
   const int P1 = 1 << sh.b1, t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
   const uint64_t NF = min(b.meta->n_fine, sh.nf_max);
@@ -1877,7 +1888,7 @@ __host__ __device__ constexpr uint32_t big_bucket(int kw) { return kw == 1 ? 512
 constexpr int kBigMax = 32;  // more than d / big_bucket <= 6144 / 257
 
 // Exclusive scan of `words` words of two 16-bit counts each (worker warps; warp 0 is busy with
-// the look-back meanwhile).  The total fits in 16 bits.
+// the look-back meanwhile).  The total fits in 16 bits and goes behind the last word.
 __device__ void workers_exclusive_scan16(uint32_t* data, int words, uint32_t* warp_tmp) {
   constexpr int nt = kWorkers, nw = kWorkers / 32;
   const int t = threadIdx.x - 32, lane = t & 31, wid = t >> 5;
@@ -1901,6 +1912,7 @@ __device__ void workers_exclusive_scan16(uint32_t* data, int words, uint32_t* wa
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
   uint32_t run = before + x - s;
+  if (t == nt - 1) reinterpret_cast<uint16_t*>(data)[2 * words] = (uint16_t)(before + x);
   for (int i = lo; i < hi; ++i) {
     const uint32_t v = data[i], a = v & 0xffffu;
     data[i] = run | ((run + a) << 16);
@@ -1942,10 +1954,11 @@ __device__ __forceinline__ uint32_t bucket_of(u128 off, const OrderMap<u128>& o)
 // Group the table's d occupied slots by bucket (worker warps only): an ordered counting sort
 // of the slot numbers into idx[0, d) and, for 64-bit keys, of the keys into gkey[0, d), buckets
 // ascending, slots unordered inside a bucket.  hist (cleared before) is left holding bucket
-// b's first position in its b-th 16 bits, d after the last; big_s[0, *big_n) lists the
-// buckets above kBigBucket entries.
+// b's first position in its b-th 16 bits, their number after the last; big_s[0, *big_n) lists
+// the buckets above big_bucket entries.  Returns the number of entries placed: d, or the status
+// says that the table does not hold what was counted (no more than these entries may be read).
 template <int KW>
-__device__ __forceinline__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, uint32_t NB,
+__device__ __forceinline__ uint32_t bucket_slots(Table<KW> tb, uint32_t nslots, uint32_t d, uint32_t NB,
                                              const OrderMap<typename KeyT<KW>::T>& o, uint32_t* hist, uint16_t* idx,
                                              uint64_t* gkey, uint32_t* wtmp, uint32_t* big_s, uint32_t* big_n,
                                              uint32_t* status, unsigned long long* prof = nullptr) {
@@ -1987,10 +2000,11 @@ __device__ __forceinline__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint
   }
   bar_workers();
   mark(5);
-  if (t == 0) reinterpret_cast<uint16_t*>(hist)[NB] = (uint16_t)d;  // past the scanned words (NB > 1), or scanned as 0
   workers_exclusive_scan16(hist, (int)(NB / 2), wtmp);
   mark(6);
   const uint16_t* start = reinterpret_cast<const uint16_t*>(hist);
+  const uint32_t placed = start[NB];
+  if (t == 0 && placed != d) atomicOr(status, ST_INTERNAL);
 #pragma unroll
   for (int m = 0; m < kSlotsPerWorker; ++m)
     if (br[m] != 0xffffffffu) {
@@ -2000,6 +2014,7 @@ __device__ __forceinline__ void bucket_slots(Table<KW> tb, uint32_t nslots, uint
     }
   bar_workers();
   mark(7);
+  return placed;
 }
 
 // Worker warps: the rank of the entry at each bucket-grouped position j (its bucket's first
@@ -2180,7 +2195,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       // waiting on unpublished predecessors only as long as the workers are busy.  Without a
       // prefix by then, the partition's run is written to its own input region instead
       // (deferred) and k_compact moves it once all counts are known.
-      uint32_t rank[kRankRegs];
+      uint32_t rank[kRankRegs], placed = 0;
       if (wid == 0) {
         const long long lb0 = clock64();
         // (with a withheld prefix, a test that needs the wait to run out, it does not give up
@@ -2203,9 +2218,9 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
         uint32_t NB = 2;
         while (NB < dn) NB <<= 1;
         const OrderMap<K> om = order_map<K>(range_s[0], range_s[1], NB);
-        bucket_slots<KW>(tb, 1u << bT, dn, NB, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status, prof);
+        placed = bucket_slots<KW>(tb, 1u << bT, dn, NB, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status, prof);
         if (prof && threadIdx.x == 32) atomicAdd(&prof[1], (unsigned long long)(clock64() - tm));
-        rank_slots<KW>(tb, idx, gkey, dn, hist, om, big_s, big_n, rank, prof);
+        rank_slots<KW>(tb, idx, gkey, placed, hist, om, big_s, big_n, rank, prof);
         bar_workers();
         if (threadIdx.x == 32) ordered_s = 1;
       }
@@ -2221,7 +2236,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
       uint64_t* okeys = direct ? b.out_keys : b.sbuf;
       uint32_t* ocnts = direct ? b.out_counts : reinterpret_cast<uint32_t*>(b.kbuf);
       const uint64_t obase = direct ? ex : f0, olim = direct ? s.cap : f0 + n;
-      if (wid > 0) emit_slots<KW>(tb, idx, dn, rank, obase, okeys, ocnts, olim, &b.meta->status);
+      if (wid > 0) emit_slots<KW>(tb, idx, placed, rank, obase, okeys, ocnts, olim, &b.meta->status);
       if (threadIdx.x == 0) {
         if (special_s) {
           if (obase + dn < olim) {
@@ -2294,7 +2309,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
           continue;
         }
         {
-          uint32_t rank2[kRankRegs];
+          uint32_t rank2[kRankRegs], placed = 0;
           if (wid == 0) {  // the prefix is waited for while the first part is ordered
             if (!have_prefix) {
               const uint64_t ex = g == 0 ? 0 : lookback(b.look, g, &b.meta->status, s.spin_limit);
@@ -2304,13 +2319,13 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
             uint32_t NB2 = 2;
             while (NB2 < dn2) NB2 <<= 1;
             const OrderMap<K> om = order_map<K>(lo, hi, NB2);
-            bucket_slots<KW>(tb, cap_slots, dn2, NB2, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status);
-            rank_slots<KW>(tb, idx, gkey, dn2, hist, om, big_s, big_n, rank2, nullptr);
+            placed = bucket_slots<KW>(tb, cap_slots, dn2, NB2, om, hist, idx, gkey, wtmp, big_s, &big_n, &b.meta->status);
+            rank_slots<KW>(tb, idx, gkey, placed, hist, om, big_s, big_n, rank2, nullptr);
           }
           have_prefix = true;
           block_sync();
           const uint64_t base = excl_s + written;
-          if (wid > 0) emit_slots<KW>(tb, idx, dn2, rank2, base, b.out_keys, b.out_counts, s.cap, &b.meta->status);
+          if (wid > 0) emit_slots<KW>(tb, idx, placed, rank2, base, b.out_keys, b.out_counts, s.cap, &b.meta->status);
         }
         written += dn2;
         block_sync();
@@ -2478,7 +2493,6 @@ __device__ __forceinline__ void move_run(const Shape& s, const Buffers& b, uint6
 }
 template <int KW>
 __device__ __forceinline__ void compact_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
-  check_offsets(s, b, bid, nblk);
   const uint64_t n_def = min(b.meta->n_deferred, s.nf_max);
   for (uint64_t q = bid; q < n_def; q += nblk) {
     const uint64_t g = b.flo[q];
@@ -2496,7 +2510,6 @@ template <int KW>
 __device__ __forceinline__ void finish_one_body(const Shape& s, const Buffers& b, uint32_t bid, uint32_t nblk) {
   __shared__ uint32_t pre[kOneLevelFine + kOneLevelFine / 32 + 1];
   __shared__ uint32_t wt[32];
-  check_offsets(s, b, bid, nblk);
   const int NF = (int)min(b.meta->n_fine, min(s.nf_max, kOneLevelFine));
   for (int g = threadIdx.x; g < NF; g += blockDim.x) pre[PAD(g)] = b.fhist[g] & 0x7fffffffu;
   __syncthreads();
@@ -2563,17 +2576,19 @@ static uint32_t prepare_blocks(const Shape& s, uint64_t most) {
 // Pass A: a block per tile, or (one level) at most four per SM, each adding up the bins of
 // several tiles (pass A of 10 M / 45 M bases: 608 blocks 40 / 93 us, 912 44 / 107, 1216 51 /
 // 100; as few blocks as give each the same number of tiles, 407 / 550: 42 / 102).
+// Many short or empty reads: more blocks than tiles, a share of the offsets each.
 static uint32_t pack_blocks(const Shape& s) {
-  return (uint32_t)std::max<uint64_t>(1, s.one_level ? std::min<uint64_t>(s.n_tiles, 608) : s.n_tiles);
+  const uint64_t tiles = s.one_level ? std::min<uint64_t>(s.n_tiles, 608) : s.n_tiles;
+  return (uint32_t)std::max<uint64_t>(tiles, std::min<uint64_t>(s.n_reads / 8192 + 1, 608));
 }
 // the scan of the distinct counts: a share of about 4096 fine partitions each
 static uint32_t scan_blocks(const Shape& s) {
   const uint64_t want = s.nf_max / 4096 + 1;
   return (uint32_t)(want < 128 ? want : 128);
 }
-// the last kernel: deferred runs to move (at most one per fine partition), offsets to check
+// the last kernel: deferred runs to move (at most one per fine partition)
 static uint32_t compact_blocks(const Shape& s, int n_sms) {
-  const uint64_t want = std::max<uint64_t>(s.nf_max / 8, s.n_reads / 2048) + 1, most = (uint64_t)n_sms * 8;
+  const uint64_t want = s.nf_max / 8 + 1, most = (uint64_t)n_sms * 8;
   return (uint32_t)(want < most ? want : most);
 }
 // pass A: the histogram, and the last block's scan of the partitions' totals

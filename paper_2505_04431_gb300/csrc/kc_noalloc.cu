@@ -151,11 +151,11 @@ extern "C" kc_status kc_count_noalloc(const uint8_t* reads, const uint64_t* offs
     return nfail(KC_ECUDA, std::string("kc_count_noalloc: launch: ") + cudaGetErrorString((cudaError_t)(-launches)));
   if (ce != cudaSuccess || se != cudaSuccess)
     return nfail(KC_ECUDA, std::string("kc_count_noalloc: ") + cudaGetErrorString(ce != cudaSuccess ? ce : se));
+  if (m.status & kc::ST_BAD_OFFSETS) return nfail(KC_EINVAL, "kc_count_noalloc: offsets must be non-decreasing");
   // the status record must describe a result that fits the caller's buffers
   if (m.n_windows > L || m.n_distinct > m.n_windows || m.n_fine > s.nf_max || m.n_deferred > m.n_fine ||
       m.n_distinct > out_capacity)
     return nfail(KC_ECUDA, "kc_count_noalloc: inconsistent status record");
-  if (m.status & kc::ST_BAD_OFFSETS) return nfail(KC_EINVAL, "kc_count_noalloc: offsets must be non-decreasing");
   if (m.status & kc::ST_PARTITION_OVERFLOW) return nfail(KC_EOVERFLOW, "kc_count_noalloc: a key range holds 2^32 windows");
   if (m.status & kc::ST_COUNT_OVERFLOW) return nfail(KC_EOVERFLOW, "kc_count_noalloc: a count exceeds 2^32 - 1");
   if (m.status & kc::ST_TIMEOUT) return nfail(KC_ETIMEOUT, "kc_count_noalloc: a device-side wait timed out");
