@@ -118,3 +118,34 @@ def test_count_above_the_limit_gives_eoverflow(lib):
     finally:
         c.close()
     assert counts_like_the_oracle(r, o, 31)
+
+
+# Reads whose k-mers share a prefix of 16 bases (one fine partition, however many there are)
+# and come in order, each up to `jitter` places away from its own: a table that overflows holds
+# the first of them, so that a split at their median may leave nearly all on one side.
+@pytest.mark.parametrize("n,slots,jitter", [(3000, 64, 1), (50_000, 64, 2000), (300_000, 1024, 1), (1_500_000, 0, 1),
+                                            (1_500_000, 0, 4000)])
+@pytest.mark.parametrize("k", [31, 33])
+@pytest.mark.parametrize("falling", [True, False])
+def test_overflowing_partition_in_order(lib, n, slots, jitter, k, falling):
+    from paper_2505_04431_gb300 import KmerCounter
+    rng = np.random.default_rng(n + k)
+    codes = np.sort(rng.choice(1 << 30, n, replace=False))  # the bases 16 .. 30
+    codes = codes[np.argsort(np.arange(n) + rng.random(n) * jitter)]
+    if falling:
+        codes = codes[::-1]
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    reads = np.full((n, k), ord("C"), np.uint8)
+    for i in range(15):
+        reads[:, 16 + i] = acgt[(codes >> (2 * (14 - i))) & 3]
+    offsets = np.arange(n + 1, dtype=np.uint64) * k
+    c = KmerCounter(table_slots_max=slots)
+    try:
+        res = c.count(reads.reshape(-1), offsets, k, False)
+        keys, counts = res.to_numpy()
+        res.free()
+        assert c.stats()["n_overflow_fine"] == 1
+    finally:
+        c.close()
+    want_k, want_c, _ = oracle.count(reads.reshape(-1), offsets, k, False)
+    assert np.array_equal(keys, want_k) and np.array_equal(counts, want_c)
