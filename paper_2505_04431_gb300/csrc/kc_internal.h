@@ -82,7 +82,6 @@ struct Meta {
   uint32_t status;
   uint32_t fine_spill;  // the sampled fine layout overflowed a region: the exact fine split ran
   uint64_t ticket;      // phase-2 work counter
-  uint64_t d_estimate;  // distinct keys estimated by the sketch
   uint32_t done;        // blocks of pass A that have finished
   uint32_t one;         // either-level counts: 1 = pass B writes the fine partitions
   uint32_t fine_unfit;  // the sampled fine layout does not fit its room (set by the fine scan, with fine_spill)

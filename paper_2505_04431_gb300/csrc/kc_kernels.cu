@@ -681,53 +681,88 @@ __device__ __forceinline__ void sketch_windows(uint32_t* hll, uint32_t m, uint32
   }
 }
 
+// Estimated distinct keys D from the sketch's m = 1024 registers, each r (HyperLogLog, over one
+// key in 64): 64 c / Z for Z = the sum of 2^-r, and 64 m log(m / zeros) (linear counting) while
+// many registers are 0.  What a count needs is 9/10 of its windows per distinct key; the sketch
+// gives it as an integer, 0.9 * 2^68 / D, to be multiplied by the windows.  Z is added up exactly
+// (in units of 2^-53) and the quotients are constants, so that the way from the last key's
+// register to the plan, on which every later kernel waits, has no division, logarithm or double
+// precision on it.  (In double precision pass A of 0.2 M and of 10 M bases took 21.5 and 43 us
+// instead of 17.5 and 38, and the calls 13 and 16 us more: its constants come from memory that is
+// not in the caches between counts.  That holds for any constant that is not in the code: the two
+// below as loads cost 5 to 11 us a call.)
+constexpr double kTwo53 = 9007199254740992.0, kHllM = kHllRegs;
+constexpr double kHllC = 0.7213 / (1.0 + 1.079 / kHllM) * kHllM * kHllM;
+constexpr uint64_t kHllMul = (uint64_t)(0.9 / (kHllSample * kHllC) * 67108864.0 * kTwo53);  // times Z * 2^53: the top word
+constexpr uint64_t kHllFew = (uint64_t)(kHllC / (2.5 * kHllM) * kTwo53);  // Z * 2^53 above which D is below 64 * 2.5 m
+struct FewKeys {
+  uint64_t at[kHllRegs + 1];  // [zeros]: linear counting (0 if every register is 0: no key seen)
+};
+constexpr double ln_series(double f) {  // log(f), f in [1, 2], by the series of atanh((f - 1) / (f + 1))
+  const double t = (f - 1.0) / (f + 1.0);
+  double p = t, sum = 0.0;
+  for (int i = 1; i < 40; i += 2) {
+    sum += p / i;
+    p *= t * t;
+  }
+  return 2.0 * sum;
+}
+constexpr FewKeys few_keys() {
+  FewKeys k{};
+  const double ln2 = ln_series(2.0);
+  for (int z = 1; z < kHllRegs; ++z) {
+    double f = kHllM / z, l = 0.0;
+    for (; f >= 2.0; f *= 0.5) l += ln2;
+    l += ln_series(f);
+    k.at[z] = (uint64_t)(0.9 / (kHllSample * kHllM * l) * 32768.0 * kTwo53);
+  }
+  return k;
+}
+static __device__ const FewKeys kFewKeys = few_keys();
+
 // The keys a fine partition aims at, from the sketch of a count of K windows: fine_target
-// distinct keys, i.e. fine_target * K / D keys; where that gives an SM few partitions, as much
-// less as makes them a whole number (one partition too many for a last wave costs a small
-// count a wave: 10 M bases had 497 for 152 SMs, and 0.2 M bases 11).  `extra`: partitions that
-// come on top of K / target.  All threads of the block call it.
-__device__ double sketch_target(const uint32_t* hll, uint64_t K, const Shape& s, uint32_t extra, Meta* meta) {
-  __shared__ float zsum_s[32], zeros_s[32];
-  __shared__ double target_s;
+// distinct keys, i.e. fine_target * K / D keys (a tenth less, for the estimate's error, and at
+// most 32 times as many); where that gives an SM few partitions, as much less as makes them a
+// whole number (one partition too many for a last wave costs a small count a wave: 10 M bases
+// had 497 for 152 SMs, and 0.2 M bases 11).  `extra`: partitions that come on top of K / target.
+// All threads of the block call it.
+__device__ uint32_t sketch_target(const uint32_t* hll, uint64_t K, const Shape& s, uint32_t extra) {
+  __shared__ uint64_t zsum_s[32];
+  __shared__ uint32_t zeros_s[32], target_s;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // HyperLogLog estimate over the 1/64 sample of the keys (read from L2: written by every SM)
-  float z = 0.f, zeros = 0.f;
-  for (int i = threadIdx.x; i < kHllRegs; i += blockDim.x) {
+  uint64_t z = 0;  // in units of 2^-53 (at most 1024 registers of 1: below 2^64)
+  uint32_t zeros = 0;
+  for (int i = threadIdx.x; i < kHllRegs; i += blockDim.x) {  // (read from L2: written by every SM)
     const uint32_t r = __ldcg(&hll[i]);
-    z += exp2f(-(float)r);
-    zeros += r == 0 ? 1.f : 0.f;
+    z += (1ull << 53) >> r;
+    zeros += r == 0;
   }
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    z += __shfl_xor_sync(0xffffffffu, z, d);
-    zeros += __shfl_xor_sync(0xffffffffu, zeros, d);
-  }
+  for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
+  zeros = __reduce_add_sync(0xffffffffu, zeros);
   if (lane == 0) {
     zsum_s[wid] = z;
     zeros_s[wid] = zeros;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    float zs = 0, zr = 0;
+    z = zeros = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      zs += zsum_s[w];
-      zr += zeros_s[w];
+      z += zsum_s[w];
+      zeros += zeros_s[w];
     }
-    // (single precision: the estimate is good to 3%, and double precision is slow here)
-    const float m = kHllRegs;
-    float e = 0.7213f / (1.0f + 1.079f / m) * m * m / zs;
-    if (e < 2.5f * m && zr > 0) e = m * logf(m / zr);
-    const float d_est = e * (float)kHllSample;
-    float dup = d_est > 1.0f ? (float)K / d_est : 1.0f;
-    dup = fminf(fmaxf(dup, 1.0f), 32.0f);
-    float target = (float)s.fine_target * fmaxf(0.9f * dup, 1.0f);
-    const float per_sm = ceilf(((float)K / target + (float)extra) / (float)s.n_sms);
-    if (per_sm <= 16.0f) {
+    const uint64_t per_window = zeros && z > kHllFew ? kFewKeys.at[zeros] : __umul64hi(z, kHllMul);
+    // 0.9 K / D in units of 2^-32, between 1 and 0.9 * 32
+    const uint64_t hi = __umul64hi(K, per_window), lo = K * per_window, most = (uint64_t)(28.8 * 4294967296.0);
+    const uint64_t dup = max((uint64_t)1 << 32, hi >= 512 ? most : min(most, (hi << 28) | (lo >> 36)));
+    const uint64_t keys = s.fine_target * dup;
+    uint32_t target = (uint32_t)((keys + 0xffffffffull) >> 32);
+    const float per_sm = ceilf(((float)K / ((float)keys * 2.3283064e-10f) + (float)extra) / (float)s.n_sms);
+    if (per_sm <= 16.0f) {  // (an empty count may have no partition left for keys: 0 / 0, which fmaxf drops)
       const float parts = per_sm * (float)s.n_sms - (float)extra;
-      target = fminf(target, fmaxf((float)K / parts + 1.0f, (float)kMinFineKeys));
+      target = (uint32_t)fminf((float)target, ceilf(fmaxf((float)K / parts + 1.0f, (float)kMinFineKeys)));
     }
     target_s = target;
-    meta->d_estimate = (uint64_t)d_est;
   }
   __syncthreads();
   return target_s;
@@ -765,12 +800,13 @@ __device__ __forceinline__ void bucket_scan(const Shape& s, const Buffers& b, ui
 __device__ __forceinline__ void one_level_plan(const Shape& s, const Buffers& b, uint32_t* sc) {
   __shared__ uint32_t wt[32];
   const int NB = 1 << s.bb;
+  if (threadIdx.x <= kHllRegs / 16)  // linear counting's table, a line each, while the bins are added up
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(&kFewKeys.at[threadIdx.x * 16]));
 #pragma unroll 8
   for (int i = threadIdx.x; i < NB; i += blockDim.x) sc[PAD(i)] = __ldcg(&b.bins[i]);
   __syncthreads();
   const uint32_t K = block_exclusive_scan_pad<uint32_t>(sc, NB, wt);  // below 2^26
-  const double target = sketch_target(b.hll, K, s, 0, b.meta);
-  const uint32_t T = max((uint32_t)ceil(target), (uint32_t)(K / s.nf_max) + 1u);
+  const uint32_t T = max(sketch_target(b.hll, K, s, 0), (uint32_t)(K / s.nf_max) + 1u);
   const uint32_t NF = sc[PAD(NB - 1)] / T + 1;  // the last bin's partition is the last: at most K / T + 1 <= nf_max
   const bool either = s.one_level == kEitherLevel;
   if (either && NF > kEitherFine) {  // two levels: the coarse partitions are the bins' top bits
@@ -936,7 +972,7 @@ __device__ __forceinline__ void fine_plan_body(const Shape& s, const Buffers& b,
     if (c == 0 && threadIdx.x == 0) b.flo[min(b.meta->n_fine, s.nf_max)] = 0;
     return;
   }
-  const uint32_t T = (uint32_t)ceil(sketch_target(b.hll, b.cstart[P1], s, P1, b.meta));
+  const uint32_t T = sketch_target(b.hll, b.cstart[P1], s, P1);
   auto parts = [&](uint64_t n) -> uint32_t {  // (n is below 2^32)
     const uint32_t m = n ? ((uint32_t)n - 1) / T + 1 : 1;
     return m < (uint32_t)kMaxFine ? m : (uint32_t)kMaxFine;

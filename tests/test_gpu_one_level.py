@@ -148,3 +148,62 @@ def test_sketch_of_sampled_windows(torch_cuda, k):
         assert n_fine[0] == n_fine[1]
         if options:
             assert abs(n_fine[0] * 128 * 0.9 / distinct - 1) < 0.2
+
+
+@pytest.mark.parametrize("genome", [100_000, 140_000, 700_000])  # two where registers stay empty, one where none does
+@pytest.mark.parametrize("k,canonical", [(31, True), (63, True), (21, False)])
+def test_fine_partitions_from_the_sketch(torch_cuda, genome, k, canonical):
+    """The fine partitions are those that the sketch's estimate gives in double precision (a
+    coarse partition of n windows is cut into ceil(n / T), T = 0.9 fine_target K / D rounded up);
+    K / T is beyond 16 per SM, where the target is the estimate's alone."""
+    from paper_2505_04431_gb300 import KmerCounter
+    rng = np.random.default_rng(genome + k)
+    length = 100 + k
+    n = 2_500_000 // (length - k + 1)
+    codes = rng.integers(0, 4, genome)
+    at = rng.integers(0, genome - length, n)
+    windows = codes[at[:, None] + np.arange(length)].astype(np.uint64)  # [read, base]
+    reads = np.frombuffer(b"ACGT", np.uint8)[windows.astype(np.int64)].reshape(-1)
+    offsets = np.arange(n + 1, dtype=np.uint64) * length
+    last = length - k + 1
+
+    def value(cols, a, b):  # 64-bit value of the bases a .. b - 1 of every window
+        v = np.zeros((n, last), np.uint64)
+        for i in range(a, b):
+            v = (v << np.uint64(2)) | cols(i)
+        return v
+
+    fwd = lambda i: windows[:, i:i + last]
+    rev = lambda i: np.uint64(3) - windows[:, k - 1 - i:k - 1 - i + last]
+    hi_n = max(0, k - 32)
+    f = (value(fwd, 0, hi_n), value(fwd, hi_n, k))
+    r = (value(rev, 0, hi_n), value(rev, hi_n, k))
+    take = ((r[0] < f[0]) | ((r[0] == f[0]) & (r[1] < f[1]))) & canonical
+    hi, lo = np.where(take, r[0], f[0]), np.where(take, r[1], f[1])
+    top_f, top_r = value(fwd, 0, 16), value(rev, 0, 16)
+    x = np.where(take, top_r, top_f)
+    y = np.uint64(0xffffffff) - x
+    u = np.uint64(0xffffffff) - ((y * y) >> np.uint64(32)) if canonical else x
+    n_c = np.bincount((u >> np.uint64(30)).astype(np.int64).reshape(-1), minlength=4)
+    sampled = (((top_f + top_r) * np.uint64(0x9E3779B1)) & np.uint64(0xffffffff)) >> np.uint64(26) == 0
+    h = ((lo ^ (hi * np.uint64(0xC2B2AE3D27D4EB4F))) * np.uint64(0x9E3779B97F4A7C15))[sampled]
+    regs = np.zeros(1024, np.int64)
+    low = [int(v) & ((1 << 54) - 1) for v in np.unique(h)]
+    np.maximum.at(regs, (np.unique(h) >> np.uint64(54)).astype(np.int64), [min(55 - v.bit_length(), 55) for v in low])
+    e = 0.7213 / (1 + 1.079 / 1024) * 1024.0 ** 2 / np.sum(2.0 ** -regs)
+    zeros = int(np.sum(regs == 0))
+    if e < 2560 and zeros:
+        e = 1024 * np.log(1024 / zeros)
+    assert (e < 2560) == (genome < 700_000)
+    total = n * last
+    dup = min(max(total / (64 * e), 1.0), 32.0)
+    T = int(np.ceil(35 * max(0.9 * dup, 1.0)))
+    assert total / T > 17 * 152
+    c = KmerCounter(n_partitions_hint=4, table_slots_max=64)
+    res = c.count(torch_cuda.from_numpy(reads.copy()).cuda(), torch_cuda.from_numpy(offsets.view(np.int64)).cuda(), k,
+                  canonical)
+    assert res.n_valid_windows == total
+    res.free()
+    got = c.stats()["n_fine"]
+    c.close()
+    assert got == sum(min(max(1, -(-int(v) // T)), 4096) for v in n_c)
