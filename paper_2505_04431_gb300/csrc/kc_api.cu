@@ -398,8 +398,9 @@ void plan_job(const kc_plan_s* p, const uint8_t* reads, const uint64_t* offsets,
 }
 
 // One allocation for a count's keys and, behind them, its counts; false if there is none.
+size_t out_bytes(const Job& j) { return counts_at(j.out_key_bytes) + j.out_cnt_bytes; }
 bool alloc_outputs(kc_plan_s* p, Job& j) {
-  j.okeys = dev_alloc(p, counts_at(j.out_key_bytes) + j.out_cnt_bytes);
+  j.okeys = dev_alloc(p, out_bytes(j));
   j.ocnts = j.okeys ? (uint8_t*)j.okeys + counts_at(j.out_key_bytes) : nullptr;
   return j.okeys != nullptr;
 }
@@ -571,7 +572,6 @@ bool plan_groups(const kc_plan_s* p, const std::vector<Job>& jobs, GroupPlan& gp
                                             : kBatchArenaBytes;
   for (uint32_t i = 0; i < (uint32_t)jobs.size(); ++i) {
     const Job& j = jobs[i];
-    gp.out_total += j.out_key_bytes + j.out_cnt_bytes;
     const size_t w = align_up(j.ws_bytes, 256);
     if (w > arena_cap) {
       gp.alone.push_back(i);
@@ -600,7 +600,9 @@ bool plan_groups(const kc_plan_s* p, const std::vector<Job>& jobs, GroupPlan& gp
       ++gi;
     }
   }
+  for (uint32_t i : gp.alone) gp.out_total += out_bytes(jobs[i]);
   for (Group& g : gp.groups) {
+    gp.out_total += g.keys + g.cnts;
     gp.arena = std::max(gp.arena, g.ws);
     const uint32_t n = (uint32_t)g.idx.size();
     size_t words = 0;
@@ -845,7 +847,7 @@ kc_status kc_footprint(kc_plan_t p, uint64_t n_reads, uint64_t n_bases, int k, i
   o.allow_sampled = 1;  // as kc_count and kc_submit size a count
   kc::make_shape(o, n_bases, n_reads, k, 1, n_bases > 0 && !reads_on_device, !offsets_on_device, s, lay);
   *scratch_bytes = lay.total;
-  *result_bytes = s.cap * s.kw * 8 + s.cap * 4;
+  *result_bytes = counts_at(s.cap * s.kw * 8) + s.cap * 4;
   return KC_OK;
 }
 
@@ -929,7 +931,7 @@ kc_status kc_count(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, u
 
   Job j;
   plan_job(p, reads, offsets, n_reads, L, off_dev, k, canonical, j, false, true);
-  if (p->max_bytes && (uint64_t)(j.ws_bytes + j.out_key_bytes + j.out_cnt_bytes) > p->max_bytes)
+  if (p->max_bytes && (uint64_t)(j.ws_bytes + out_bytes(j)) > p->max_bytes)
     return fail(KC_ENOMEM, "kc_count: input needs more device memory than max_device_bytes");
   if (p->ws_bytes < j.ws_bytes) {
     dev_free(p, p->ws);
@@ -1119,7 +1121,7 @@ kc_status kc_submit(kc_plan_t p, const uint8_t* reads, const uint64_t* offsets, 
   const size_t stage_r = a->j.stage_r ? (n_bases + 16 + 255) / 256 * 256 : 0;
   const size_t stage_o = a->j.stage_o ? (n_reads + 1) * 8 : 0;
   if (p->max_bytes &&
-      (uint64_t)(a->j.ws_bytes + stage_r + stage_o + a->j.out_key_bytes + a->j.out_cnt_bytes) > p->max_bytes) {
+      (uint64_t)(a->j.ws_bytes + stage_r + stage_o + out_bytes(a->j)) > p->max_bytes) {
     delete a;
     return fail(KC_ENOMEM, "kc_submit: input needs more device memory than max_device_bytes");
   }

@@ -149,3 +149,57 @@ def test_overflowing_partition_in_order(lib, n, slots, jitter, k, falling):
         c.close()
     want_k, want_c, _ = oracle.count(reads.reshape(-1), offsets, k, False)
     assert np.array_equal(keys, want_k) and np.array_equal(counts, want_c)
+
+
+# 3 bases, and lengths whose keys do not end on a 256-byte boundary; the last one as a batch
+@pytest.mark.parametrize("lengths", [[3], [1001], [300_007], [501, 20_003, 77]])
+@pytest.mark.parametrize("k", [31, 63])
+def test_footprint_and_limit_are_what_is_allocated(lib, lengths, k):
+    import torch
+
+    from paper_2505_04431_gb300 import (_ALLOC_FN, _FREE_FN, KC_ENOMEM, KC_OK, KcError, KmerCounter, PlanOpts,
+                                        Result)
+    rng = np.random.default_rng(k)
+    samples = [np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, n)] for n in lengths]
+    dev = [(torch.from_numpy(r).cuda(), torch.tensor([0, len(r)], device="cuda"), len(r)) for r in samples]
+    sizes = []
+
+    def allocate(n, s, c):
+        sizes.append(n)
+        return int(torch.cuda.caching_allocator_alloc(int(n), 0, s or 0))
+
+    alloc = _ALLOC_FN(allocate)
+    free = _FREE_FN(lambda p, s, c: torch.cuda.caching_allocator_delete(int(p)) if p else None)
+    opts = PlanOpts()
+    opts.device, opts.alloc, opts.free_ = 0, alloc, free
+    plan = ctypes.c_void_p()
+    assert lib.kc_plan(ctypes.byref(opts), ctypes.byref(plan)) == KC_OK
+    n = len(dev)
+    res = (Result * n)()
+    if n == 1:
+        scratch, result = ctypes.c_uint64(), ctypes.c_uint64()
+        assert lib.kc_footprint(plan, 1, dev[0][2], k, 1, 1, ctypes.byref(scratch), ctypes.byref(result)) == KC_OK
+        st = lib.kc_count(plan, dev[0][0].data_ptr(), dev[0][1].data_ptr(), 1, k, 1, res)
+        assert st == KC_OK and sum(sizes) == scratch.value + result.value
+    else:
+        arrays = [(ctypes.c_void_p * n)(*[d[i].data_ptr() for d in dev]) for i in range(2)]
+        one = (ctypes.c_uint64 * n)(*[1] * n)
+        st = lib.kc_count_batch(plan, n, *arrays, one, (ctypes.c_uint64 * n)(*lengths), k, 1, res)
+        assert st == KC_OK
+    for r in res:
+        lib.kc_free(plan, ctypes.byref(r))
+    lib.kc_plan_destroy(plan)
+    for limit, fits in ((sum(sizes), True), (sum(sizes) - 1, False)):
+        c = KmerCounter(max_device_bytes=limit)
+        calls = [lambda: c.count_batch(dev, k)] if n > 1 else [
+            lambda: [c.count(dev[0][0], dev[0][1], k)],
+            lambda: [c.wait(c.submit(dev[0][0], dev[0][1], k, n_bases=dev[0][2]))]]
+        for call in calls:
+            if fits:
+                for r in call():
+                    r.free()
+            else:
+                with pytest.raises(KcError) as e:
+                    call()
+                assert e.value.status == KC_ENOMEM
+        c.close()
