@@ -207,3 +207,59 @@ def test_fine_partitions_from_the_sketch(torch_cuda, genome, k, canonical):
     got = c.stats()["n_fine"]
     c.close()
     assert got == sum(min(max(1, -(-int(v) // T)), 4096) for v in n_c)
+
+
+def random_reads_dev(torch, n_bases, seed, genome=0):
+    """n_bases bases in reads of 150 (the last one shorter), of a genome or of i.i.d. bases."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    n = -(-n_bases // 150)
+    if genome:
+        g = torch.randint(0, 4, (genome,), generator=gen, device="cuda")
+        at = torch.randint(0, genome - 150, (n, 1), generator=gen, device="cuda")
+        codes = g[at + torch.arange(150, device="cuda")].reshape(-1)[:n_bases]
+    else:
+        codes = torch.randint(0, 4, (n_bases,), generator=gen, device="cuda")
+    reads = torch.tensor(list(b"ACGT"), dtype=torch.uint8, device="cuda")[codes]
+    return reads, torch.clamp(torch.arange(n + 1, device="cuda") * 150, max=n_bases)
+
+
+def same(torch, a, b):
+    return (a.n_valid_windows == b.n_valid_windows and torch.equal(a.keys_tensor(), b.keys_tensor())
+            and torch.equal(a.counts_tensor(), b.counts_tensor()))
+
+
+# the lengths at which one level, the choice by pass A and two levels meet; just below 6 Mi bases
+# of 128-bit keys a block of pass A takes several tiles
+@pytest.mark.parametrize("k,line", [(31, 12 << 20), (31, 48 << 20), (63, 6 << 20)])
+@pytest.mark.parametrize("more", [-1, 0, 1])
+@pytest.mark.parametrize("genome", [0, 400_000])
+def test_lengths_around_the_paths_lines(torch_cuda, k, line, more, genome):
+    from paper_2505_04431_gb300 import KmerCounter
+    r, o = random_reads_dev(torch_cuda, line + more, k + genome, genome)
+    a, b = KmerCounter(), KmerCounter(n_partitions_hint=8)
+    x, y = a.count(r, o, k), b.count(r, o, k)
+    assert same(torch_cuda, x, y)
+    for res in (x, y):
+        res.free()
+    a.close()
+    b.close()
+
+
+# one group of batched launches with counts of every path: one level, either level (both
+# outcomes), two levels (128-bit keys: beyond 6 Mi bases) and an empty one
+@pytest.mark.parametrize("k,canonical,defer", [(31, True, False), (31, True, True), (63, True, False), (21, False, False)])
+def test_paths_side_by_side_in_a_batch(torch_cuda, k, canonical, defer):
+    from paper_2505_04431_gb300 import KmerCounter
+    torch = torch_cuda
+    sets = [random_reads_dev(torch, n, i + k, g) for i, (n, g) in enumerate(
+        [(300_000, 0), (13_631_489, 0), (13_700_001, 450_000), (1, 0), (5_900_003, 0), (20_000_000, 700_000)])]
+    sets.insert(2, (torch.zeros(0, dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int64, device="cuda")))
+    a, b = KmerCounter(defer_all=defer), KmerCounter(n_partitions_hint=2)
+    for i, ((r, o), x) in enumerate(zip(sets, a.count_batch([(r, o, r.numel()) for r, o in sets], k, canonical))):
+        y = b.count(r, o, k, canonical)
+        assert same(torch, x, y), i
+        x.free()
+        y.free()
+    a.close()
+    b.close()
