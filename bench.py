@@ -859,7 +859,7 @@ def run_ablation(args):
             ms = ev0.elapsed_time(ev1) / args.steps
             kms = {kn: sum(v) / len(v) for kn, v in ktimes.items()}
             res_wl[name] = {"value": dig[1] / (ms / 1e3) / 1e9, "ms_per_step": ms,
-                            "pass_b_ms": kms.get("k_scatter", 0.0) + kms.get("k_direct_cursors", 0.0),
+                            "pass_b_ms": kms.get("k_scatter", 0.0),
                             "count_ms": kms.get("k_count_emit", 0.0)}
             c.close()
         base = res_wl["L0-L1"]["ms_per_step"]

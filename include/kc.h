@@ -166,11 +166,11 @@ typedef struct {
                                   (their output offset was not known in time) */
   uint64_t workspace_bytes;    /* scratch currently held by the plan */
   uint64_t phase_cycles[8];    /* KC_PLAN_PROFILE only: SM cycles of the count kernel's phases
-                                  (clear, insert, sort, count, look-back, emit, overflow path,
+                                  (-, clear and count, -, order, look-back, emit, overflow path,
                                   setup), summed over its thread blocks */
-  uint64_t sub_cycles[8];      /* KC_PLAN_PROFILE only: cycles of the ordering sub-steps (key
-                                  range, rank, scan, place, small sorts, large sorts) and the
-                                  number of large buckets */
+  uint64_t sub_cycles[8];      /* KC_PLAN_PROFILE only: cycles of the ordering's steps (-, grouping
+                                  in all, -, sort of large buckets, rank; of the grouping:
+                                  histogram, scan, place) */
   uint32_t fine_sampled;       /* 1 if the fine partitions' regions were sized from a sample
                                   of the keys (large single counts) */
   uint32_t fine_resplit;       /* 1 if a sampled region overflowed and the exact fine split

@@ -55,9 +55,12 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
   s.L = L;
   s.n_reads = n_reads;
   s.n_words = (L + 31) / 32;
-  // phase-1 tiles (one thread block each): 16 waves of pass B's resident blocks where the input
-  // is long enough for that, never less than one sub-step of 256 words (a tile's fixed work,
-  // its partition cursors and its share of the sketch, is then still small beside it).  With
+  // phase-1 tiles (one thread block each): as many sub-steps of 256 words as give at most
+  // kTilesWanted tiles.  That is one sub-step up to 39.8 M bases (10 M bases: 1221 tiles), from
+  // there to 1.2 G bases 2432 to 4864 tiles, 5 to 11 waves of pass B's 456 resident blocks (the
+  // fewest just above 39.8 M, where a tile goes from one sub-step to two), and tiles of 8192
+  // words, more waves, beyond.  A tile's fixed work, its partition cursors and its share of the
+  // sketch, is small beside one sub-step.  With
   // 8192 words for every size, 0.2 M bases ran on one SM (pass A 56 + pass B 223 us; now 8 +
   // 16), 10 M bases on 39 (76 + 287; 25 + 68) and 100 M bases of k = 63 in two waves of which
   // the second was a quarter full (215 + 916; 165 + 678).
@@ -108,9 +111,14 @@ uint32_t make_shape(const ShapeOpts& o, uint64_t L, uint64_t n_reads, int k, int
                 s.nf_max <= kOneLevelFine;
   // Up to 48 Mi bases of 64-bit keys, repeats may leave as few fine partitions: pass A counts
   // bins and fills the sketch for these too, and its last block takes one level if at most
-  // kEitherFine partitions come out (45 M bases of a 30x genome: 1824; kernels 867 -> 747 us, 21 M
+  // kEitherFine partitions come out (45 M bases of a 30x genome: 1672; kernels 869 -> 719 us, 21 M
   // bases 447 -> 379), two if not (20 M bases of noisy long reads: 830 -> 895 us, the price of
-  // having looked).
+  // having looked).  Both lines lie on the side of the two-level path, where a wrong guess costs
+  // least.  Beyond 48 Mi bases (two levels -> with the line at 128 Mi, us of kernels) genomes read
+  // 60x would still gain, 52 M bases 901 -> 804 and 60 M 1035 -> 896, but from 75 M on they have
+  // more than kEitherFine partitions and pay for the look, 1178 -> 1277, at 90 M 1387 -> 1509, as
+  // genomes read 30x do from 50 M on.  Beyond 2048 partitions one level would still win at 2280
+  // (45 M bases read 12x): 817, against 998 now and 936 without the look.
   // (128-bit keys: 20 M bases 567 -> 534 us, but 25 M of noisy long reads, which take two levels
   // after all, 1476 -> 1565: they stay with two.)
   if (!s.one_level && b1 > 0 && s.kw == 1 && L < kEitherBases && !o.p_hint && !o.force_sampled &&

@@ -21,7 +21,7 @@ namespace kc {
 constexpr int kWordBases = 32;                 // bases per packed code word
 constexpr int kTileWordsMax = 8192;            // a phase-1 tile has 256 .. 8192 code words (Shape::tile_words)
 constexpr int kTileWordsStep = 256;
-constexpr uint64_t kTilesWanted = 4864;        // over 10 waves of pass B's 3 blocks on each of 152 SMs
+constexpr uint64_t kTilesWanted = 4864;        // 32 per SM: 10.7 waves of pass B's 3 blocks on each of 152 SMs
 constexpr int kPackThreads = 256;              // pass A: one code word per thread per sub-step
 constexpr int kMaxCoarseLog2 = 12;             // at most 4096 coarse partitions
 constexpr int kMaxFine = 4096;                 // at most this many fine partitions per coarse one
@@ -30,7 +30,8 @@ constexpr int kMaxFine = 4096;                 // at most this many fine partiti
 // which pass B writes directly.
 constexpr uint64_t kOneLevelFine = 3072;
 // Larger inputs below these bases take either path: one level if their repeats leave at most
-// this many fine partitions (four bins each), decided by pass A's last block.
+// this many fine partitions (four bins each), decided by pass A's last block (make_shape has
+// what both lines were measured at).
 constexpr uint64_t kEitherBases = 48ull << 20;
 constexpr uint32_t kEitherFine = 2048;
 enum { kTwoLevel, kOneLevel, kEitherLevel };   // Shape::one_level
@@ -46,13 +47,10 @@ constexpr uint64_t coarse_bases(int kw) { return kw == 1 ? (12ull << 20) : (6ull
 constexpr int kCountThreads = KC_COUNT_THREADS;
 constexpr int kCountBlocksPerSM = 1024 / kCountThreads;
 static_assert(kCountThreads == 1024 || kCountThreads == 512, "count blocks of 1024 or 512 threads");
-constexpr int kFineChunk1 = 8192;              // fine-scatter chunk, 64-bit keys
-constexpr int kFineChunk2 = 4096;              // fine-scatter chunk, 128-bit keys
 constexpr int kFineLocalCap = 2048;            // fine partitions one chunk may span (shared histogram)
 constexpr int kHllLog2 = 10;                   // distinct-key sketch: 1024 registers
 constexpr int kHllRegs = 1 << kHllLog2;
-constexpr int kHllSampleLog2 = 6;              // ... over a 1/64 hash sample of the keys (a rarer sample
-                                               // leaves pass B's warps out of the sketch update more often)
+constexpr int kHllSampleLog2 = 6;              // ... over a 1/64 hash sample of the keys
 constexpr double kHllSample = 64.0;
 constexpr uint32_t kLookbackSpinLimit = 1u << 22;  // x ~100 ns sleep: ~0.4 s, then give up
 constexpr uint32_t kTestSpinLimit = 64;            // the same wait when a test withholds a prefix
@@ -67,7 +65,7 @@ constexpr uint64_t kFineSampledMinBases = 1ull << 26;
 enum : uint32_t {
   ST_COUNT_OVERFLOW = 1u,   // a count exceeded 2^32 - 1
   ST_TIMEOUT = 2u,          // a bounded wait gave up
-  ST_BAD_OFFSETS = 4u,      // offsets not non-decreasing
+  ST_BAD_OFFSETS = 4u,      // offsets not ascending from 0 to L (set by pass A; nothing else is done then)
   ST_INTERNAL = 8u,         // an internal consistency check failed
   ST_PARTITION_OVERFLOW = 16u,  // a coarse partition holds 2^32 keys or more
 };
@@ -85,7 +83,7 @@ struct Meta {
   uint32_t done;        // blocks of pass A that have finished
   uint32_t one;         // either-level counts: 1 = pass B writes the fine partitions
   uint32_t fine_unfit;  // the sampled fine layout does not fit its room (set by the fine scan, with fine_spill)
-  uint64_t sub_cycles[8];    // profiled plans only: ordering sub-steps (range, rank, scan, place, small sorts, big sorts, #big)
+  uint64_t sub_cycles[8];    // profiled plans only: the ordering's steps (-, grouping, -, large sorts, rank, histogram, scan, place)
   uint64_t phase_cycles[8];  // profiled plans only: SM cycles per phase of k_count_emit, summed over CTAs
 };
 
@@ -130,7 +128,7 @@ struct Buffers {
   uint64_t* cstart;       // [P1 + 1] coarse partition starts
   uint32_t* fine_base;    // [P1 + 1] first fine index of each coarse partition
   uint32_t* fine_m;       // [P1] fine partitions of each coarse partition
-  uint32_t* hll;          // [kHllRegs] distinct-key sketch (max-merged by pass B)
+  uint32_t* hll;          // [kHllRegs] distinct-key sketch (max-merged by pass B, with one level by pass A)
   uint32_t* fhist;        // [nf_max] keys per fine partition (fine split); then distinct keys | deferred bit 31
   uint64_t* foff;         // [nf_max + 1] fine partition starts
   uint32_t* flo;          // [nf_max + 1] first range-map value u of each fine partition (0 after the last)

@@ -61,10 +61,10 @@ typedef unsigned __int128 u128;
 
 // The kernels of a single count are launched so that each may be set up while the one before it
 // still runs (programmatic dependent launch); a kernel first waits for that one's end and its
-// writes.  12 launches 2 us apart were 4% of a count of 21 M bases (565 -> 546 us), 2% at 45 M
-// (1079 -> 1059).  Letting the next kernel's blocks onto the SMs early, before the last one's
-// have ended, cost more than it gave (50.9 -> 52.4 ms at 3 G bases), and so did this form for
-// the batched launches (32 small samples 932 -> 951 us), which stay as they are.
+// writes.  When it came in, a count of 21 M bases, then 10 launches 2 us apart, went from 547 to
+// 533 us, one of 90 M from 1942 to 1913.  Letting the next kernel's blocks onto the SMs early,
+// before the last one's have ended, cost more than it gave (50.9 -> 52.4 ms at 3 G bases), and
+// so did this form for the batched launches (32 small samples 932 -> 951 us), which stay as they are.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
 static void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
@@ -134,9 +134,7 @@ __device__ __forceinline__ u128 shfl_key(u128 v, int src) {
   return ((u128)hi << 64) | lo;
 }
 
-// Look-back status words carry their own payload (flag and value in one 64-bit word) and
-// guard no other data, so relaxed GPU-scope accesses are enough.
-// Asynchronous 4- and 8-byte copies from global to shared memory (cp.async); the issuing
+// Asynchronous 4-, 8- and 16-byte copies from global to shared memory (cp.async); the issuing
 // thread waits for all of its copies with cp_async_wait_all.
 __device__ __forceinline__ void cp_async4(void* dst_smem, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
@@ -152,6 +150,8 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Look-back status words carry their own payload (flag and value in one 64-bit word) and
+// guard no other data, so relaxed GPU-scope accesses are enough.
 __device__ __forceinline__ void st_status(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -2167,7 +2167,7 @@ __device__ __forceinline__ void count_emit_body(const Shape& s, const Buffers& b
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long* prof = s.profile ? reinterpret_cast<unsigned long long*>(b.meta->sub_cycles) : nullptr;
   unsigned long long* ticket = reinterpret_cast<unsigned long long*>(&b.meta->ticket);
-  // profiled plans: thread 0 adds the cycles spent in each phase (0 clear, 1 count, 2 -,
+  // profiled plans: thread 0 adds the cycles spent in each phase (0 -, 1 clear and count, 2 -,
   // 3 order, 4 look-back (warp 0, overlapped), 5 emit, 6 overflow path, 7 ticket + setup)
   long long t_mark = clock64();
   auto phase = [&](int i) {
@@ -2619,9 +2619,10 @@ static uint32_t prepare_blocks(const Shape& s, uint64_t most) {
   const uint64_t want = std::max<uint64_t>((s.nf_max + 255) / 256, (s.n_tiles + 7) / 8) + 4;
   return (uint32_t)(want < most ? want : most);
 }
-// Pass A: a block per tile, or (one level) at most four per SM, each adding up the bins of
-// several tiles (pass A of 10 M / 45 M bases: 608 blocks 40 / 93 us, 912 44 / 107, 1216 51 /
-// 100; as few blocks as give each the same number of tiles, 407 / 550: 42 / 102).
+// Pass A: a block per tile, or (one level) at most four per SM of 152, in a batch for each of its
+// counts, each adding up the bins of several tiles (pass A of 10 M / 45 M bases: 608 blocks 40 /
+// 93 us, 912 44 / 107, 1216 51 / 100; as few blocks as give each the same number of tiles, 407 /
+// 550: 42 / 102).
 // Many short or empty reads: more blocks than tiles, a share of the offsets each.
 static uint32_t pack_blocks(const Shape& s) {
   const uint64_t tiles = s.one_level ? std::min<uint64_t>(s.n_tiles, 608) : s.n_tiles;
