@@ -781,7 +781,7 @@ __device__ __forceinline__ void bucket_scan(const Shape& s, const Buffers& b, ui
   for (int c = threadIdx.x; c < P1; c += blockDim.x) {
     const uint64_t n = __ldcg(&b.cstart[c]);
     sc[c] = n;
-    if (n > 0xffffffffull) atomicOr(&b.meta->status, ST_PARTITION_OVERFLOW);  // pass B keeps 32-bit cursors
+    if (n > 0xffffffffull) atomicOr(&b.meta->status, ST_PARTITION_OVERFLOW);  // (the fine split counts in 32 bits)
   }
   __syncthreads();
   const uint64_t K = block_exclusive_scan<uint64_t>(sc, P1, wt);
